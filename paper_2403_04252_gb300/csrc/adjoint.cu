@@ -821,7 +821,11 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     WPCCC_CUDA(cudaMemsetAsync(flags, 0, sizeof(int), st));
     WPCCC_CUDA(cudaMemcpyAsync(d_v, sv.data(), gs * sizeof(double), cudaMemcpyHostToDevice, st));
     // element-adjoint sub-batches: positions per launch and the scratch they need
-    const ElemScratch EL = elem_scratch_layout(B);
+    const ElemScratch EL = elem_scratch_layout(B, ELEM_F64);
+    // S and H of a segment: positions per launch that the element-adjoint workspace holds in the elements' layout
+    int elem_prec = ELEM_F64;
+    if ((s = fp64_route(B, &elem_prec)) != WPCCC_OK) return s;
+    const size_t elem_bytes = elem_scratch_layout(B, elem_prec).bytes_per_eval;
     const TanLayout TL = tan_layout(B);
     const int NB = std::max(1, std::min(max_pos, 256));
     const int n_tiles = (B->G + ADJ_NODES - 1) / ADJ_NODES;
@@ -838,7 +842,9 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     if ((s = D.get(&tnode, (size_t)NB * TL.doubles, "adjoint node derivatives")) != WPCCC_OK) return s;
     if ((s = D.get(&d_terms, (size_t)max_pos * 2 * n_obs, "adjoint terms")) != WPCCC_OK) return s;
     if ((s = D.get(&d_jobs, (size_t)max_terms * ADJ_KINDS, "adjoint jobs")) != WPCCC_OK) return s;
-    if ((s = ensure_workspace(B, (size_t)NB * EL.bytes_per_eval)) != WPCCC_OK) return s;
+    const size_t ws_need = std::max((size_t)NB * EL.bytes_per_eval, elem_bytes);
+    const int NE = (int)std::max<size_t>(1, std::min<size_t>(NB, ws_need / elem_bytes));
+    if ((s = ensure_workspace(B, ws_need)) != WPCCC_OK) return s;
     double* node = static_cast<double*>(B->ws_ptr);
     const int adj_smem = (int)adj_rk_smem_bytes(N, n_obs);
     WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, adj_smem));
@@ -903,11 +909,12 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
         WPCCC_CUDA(cudaMemcpyAsync(d_z, zseg.data(), zseg.size() * sizeof(double), cudaMemcpyHostToDevice, st));
         WPCCC_CUDA(cudaMemcpyAsync(d_terms, terms.data(), terms.size() * sizeof(AdjTerm), cudaMemcpyHostToDevice, st));
         // S, H and the LU factors of every position of the segment
+        for (int p0 = 0; p0 < npos; p0 += NE)
+            if ((s = launch_elements(B, d_ev + p0, std::min(NE, npos - p0), segS + (size_t)p0 * mat,
+                                     segH + (size_t)p0 * mat, B->ws_ptr, st, elem_prec)) != WPCCC_OK)
+                return s;
         for (int p0 = 0; p0 < npos; p0 += NB) {
             const int nb = std::min(NB, npos - p0);
-            if ((s = launch_elements(B, d_ev + p0, nb, segS + (size_t)p0 * mat, segH + (size_t)p0 * mat, B->ws_ptr, st,
-                                     0)) != WPCCC_OK)
-                return s;
             if ((s = launch_solve(N, nb, segS + (size_t)p0 * mat, nullptr, piv + (size_t)p0 * N, info + p0, st)) !=
                 WPCCC_OK)
                 return s;
@@ -1141,6 +1148,7 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     WPCCC_CUDA(cudaMemcpyAsync(gph.data(), gphase, gph.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaMemcpyAsync(&hflags, flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaStreamSynchronize(st));
+    if ((s = check_tc_err(B, "wpccc_propagate_adjoint")) != WPCCC_OK) return s;
     if (hflags & 1) return fail(WPCCC_ESINGULAR, "wpccc_propagate_adjoint: an overlap matrix had a zero pivot");
     if (hflags & 2) return fail(WPCCC_ENONFINITE, "wpccc_propagate_adjoint: the adjoint became non-finite");
     for (size_t k = 0; k < gph.size(); ++k) grad[(size_t)g0 * n_obs * npar + k] = gph[k] + gel[k];

@@ -107,6 +107,10 @@ struct NodeArgs {
     const int* tc_row;          // [2 N_T]: row of each target state in the slice planes, then its tile's size
     int tc_rows;
     size_t t6_ap_off, t6_w_off, t6_sc_off;
+    // FP64 tensor-core form (T = double, f64 != 0): instead of W, the rows W_K / r_T (re, im per d) at f64_w2 and
+    // r_T, r_T V_T at f64_r (byte offsets, rows of Gp nodes, zero past the last node)
+    int f64, Gp;
+    size_t f64_w2, f64_r;
     // sqrt((2l+1)/2 (l-q)!/(l+q)!) at l(l+1)/2 + q, and 1/k for k = 0..WPCCC_LMAX (entry 0 unused): the
     // Legendre recurrence's constants, formed once on the host instead of per node
     double th_nrm[(WPCCC_LMAX + 1) * (WPCCC_LMAX + 2) / 2];
@@ -152,7 +156,14 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
     using T2 = typename Vec2<T>::type;
     const int e = blockIdx.y;
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= A.G) return;
+    if (g >= A.G) {
+        if (sizeof(T) == 8 && A.f64 && g < A.Gp) {
+            char* nb = reinterpret_cast<char*>(A.node + (size_t)e * A.node_doubles);
+            for (int d = 0; d < 2 * (A.dmax + 1); ++d) reinterpret_cast<double*>(nb + A.f64_w2)[(size_t)d * A.Gp + g] = 0.0;
+            for (int d = 0; d < 2; ++d) reinterpret_cast<double*>(nb + A.f64_r)[(size_t)d * A.Gp + g] = 0.0;
+        }
+        return;
+    }
     const int k = g / A.Gtau, t = g - k * A.Gtau;
     const double b = ev[e].b, v = ev[e].v, z = ev[e].z;
     const double R = dist_R(b, z);
@@ -340,6 +351,11 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
     const double irT = 1.0 / rT;
     const double uQ = A.mp_c == 0.0 ? -A.Z_T * irT
                                     : (-A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT)) * irT;
+    if (sizeof(T) == 8 && A.f64) {
+        double* rr = reinterpret_cast<double*>(reinterpret_cast<char*>(base) + A.f64_r);
+        rr[g] = rT;
+        rr[(size_t)A.Gp + g] = A.mp_c == 0.0 ? -A.Z_T : -A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT);
+    }
     const size_t stride = (size_t)(A.dmax + 1) * A.G;
     double Jd[BESSEL_MAX + 1];
     bessel_j_orders(A.dmax, x, Jd);
@@ -361,6 +377,10 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
             float2* w6 = reinterpret_cast<float2*>(reinterpret_cast<float*>(base) + A.t6_w_off);
             w6[((size_t)d * 2) * A.G + g] = df_split(w0.x * irT);
             w6[((size_t)d * 2 + 1) * A.G + g] = df_split(w0.y * irT);
+        } else if (sizeof(T) == 8 && A.f64) {
+            double* w2 = reinterpret_cast<double*>(reinterpret_cast<char*>(base) + A.f64_w2);
+            w2[(size_t)(2 * d) * A.Gp + g] = w0.x * irT;
+            w2[(size_t)(2 * d + 1) * A.Gp + g] = w0.y * irT;
         } else {
             T2 a, bq;
             a.x = (T)w0.x;
@@ -1203,7 +1223,7 @@ __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __r
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-ElemScratch elem_scratch_layout(const wpccc_basis_s* B) {
+ElemScratch elem_scratch_layout(const wpccc_basis_s* B, int precision) {
     ElemScratch L{};
     const int lrot = std::max(B->T.lmax, B->n_centres == 2 ? B->P.lmax : 0);
     for (int l = 0; l <= lrot; ++l) L.dtot += (2 * l + 1) * (2 * l + 1);
@@ -1229,7 +1249,8 @@ ElemScratch elem_scratch_layout(const wpccc_basis_s* B) {
         L.w_off_f = nf;
         nf += (size_t)NX * (B->dmax + 1) * B->G * 2;
         L.node_doubles = std::max(nd, (nf + 1) / 2);
-        if (B->tc_layout) {
+        if (precision == ELEM_F64_TC) f64_layout(B, nd, L);
+        if (precision == ELEM_TC4 || precision == ELEM_TC7) {
             L.tc_rows = 2 * B->N_T;
             // tensor-core layout (precision modes 3-5): up to seven bf16 slice planes [7][tc_rows][G], the
             // scales per 128-node window, A_P [n_half][G] and W_K / r_T [d][re, im][G] as double-floats
@@ -1273,7 +1294,7 @@ static DirArgs dir_args(const wpccc_basis_s* B, const CentreDev& c, int off, dou
     a.S = S;
     a.H = H;
     a.mat = (size_t)B->N * B->N;
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, ELEM_F64);   // the small tables' layout is the same in every form
     a.cp_off = L.cp_off[off == 0 ? 0 : 1];
     a.dtot = L.dtot;
     a.npb = L.npb;
@@ -1287,7 +1308,8 @@ static DirArgs dir_args(const wpccc_basis_s* B, const CentreDev& c, int off, dou
 static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int nev, void* scratch,
                                   cudaStream_t st, int precision) {
     const bool two = B->n_centres == 2;
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, precision);
+    const bool fp64 = precision == ELEM_F64 || precision == ELEM_F64_TC;   // FP64 node tables
     double* node = static_cast<double*>(scratch);
     double2* mol = reinterpret_cast<double2*>(node + L.node_doubles * nev);
     double* et = reinterpret_cast<double*>(mol + L.mol_elems * nev);
@@ -1345,7 +1367,7 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
     na.inv_den = B->inv_den;
     na.node = node;
     na.node_doubles = L.node_doubles;
-    na.w_off = precision == 0 ? L.w_off : L.w_off_f;
+    na.w_off = fp64 ? L.w_off : L.w_off_f;
     na.N_T = B->N_T;
     na.n_half = B->n_half;
     na.stT_index = B->T.st_index;
@@ -1359,6 +1381,10 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
     na.t6_ap_off = L.t6_ap_off;
     na.t6_w_off = L.t6_w_off;
     na.t6_sc_off = L.t6_sc_off;
+    na.f64 = precision == ELEM_F64_TC;
+    na.Gp = L.Gp;
+    na.f64_w2 = L.f64_w2;
+    na.f64_r = L.f64_r;
     for (int l = 0; l <= WPCCC_LMAX; ++l) {
         na.inv_int[l] = l > 0 ? 1.0 / l : 0.0;
         for (int q = 0; q <= l; ++q) {
@@ -1368,12 +1394,13 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
             na.th_nrm[l * (l + 1) / 2 + q] = std::sqrt((2.0 * l + 1.0) * 0.5 * num / den);
         }
     }
-    if (na.tc && !B->tc_layout) return fail(WPCCC_EINVAL, "tensor-core layout not prepared");
+    if (na.tc && (!B->tc_layout || !B->fT2)) return fail(WPCCC_EINVAL, "tensor-core layout not prepared");
     if (na.tc && B->G % 128 != 0) return fail(WPCCC_EUNSUPPORTED, "the tensor-core layout needs a multiple of 128 nodes");
     const size_t nsm = node_tables_smem(B, na.tc);
     cudaEvent_t e0 = B->prof.begin(PROF_NODES, st);
-    if (precision == 0) {
-        k_node_tables<double><<<dim3((B->G + 127) / 128, nev), 128, 0, st>>>(na, evals);
+    if (fp64) {
+        const int gn = na.f64 ? L.Gp : B->G;   // the padded nodes of the FP64 tensor-core form are written as zeros
+        k_node_tables<double><<<dim3((gn + 127) / 128, nev), 128, 0, st>>>(na, evals);
     } else {
         if (nsm > 48 * 1024)
             WPCCC_CUDA(cudaFuncSetAttribute(k_node_tables<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nsm));
@@ -1393,9 +1420,10 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
                              double2* H, void* scratch, cudaStream_t st, int precision) {
     if (nev <= 0) return WPCCC_OK;
     const bool two = B->n_centres == 2;
-    if (two && B->mp_c != 0.0 && precision != 0)
+    const bool fp64 = precision == ELEM_F64 || precision == ELEM_F64_TC;
+    if (two && B->mp_c != 0.0 && !fp64)
         return fail(WPCCC_EUNSUPPORTED, "model-potential targets need FP64 elements (precision mode 0 or 2)");
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, precision);
     double* node = static_cast<double*>(scratch);
     double2* mol = reinterpret_cast<double2*>(node + L.node_doubles * nev);
     double* et = reinterpret_cast<double*>(mol + L.mol_elems * nev);
@@ -1421,16 +1449,19 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
         ga.half_state = B->half_state;
         ga.node = node;
         ga.node_doubles = L.node_doubles;
-        ga.w_off = precision == 0 ? L.w_off : L.w_off_f;
+        ga.w_off = fp64 ? L.w_off : L.w_off_f;
         ga.mol = mol;
         const int n_row_tiles = (B->N_T + GT_I - 1) / GT_I;
         cudaEvent_t e0 = B->prof.begin(PROF_MOL, st);
-        if (precision == 0) {
+        if (precision == ELEM_F64) {
             const size_t gsm = (size_t)GT_K * (GT_I + 1 + GT_J + 1) * sizeof(double) +
                                (size_t)NX * (B->dmax + 1) * GT_K * sizeof(double2);
             WPCCC_CUDA(cudaFuncSetAttribute(k_mol_gemm<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)gsm));
             k_mol_gemm<double><<<dim3(n_row_tiles * ga.n_col_tiles, nev), 256, gsm, st>>>(ga);
+        } else if (precision == ELEM_F64_TC) {
+            wpccc_status ms = launch_mol_f64tc(B, nev, node, mol, B->tc_err, st);
+            if (ms != WPCCC_OK) return ms;
         } else if (precision == 3 || precision == 4) {
             wpccc_status ms = launch_mol_tc64(B, nev, node, mol, B->tc_err, st,
                                                precision == 3 ? OZ_FAST_SLICES : OZ_SLICES);
@@ -1562,6 +1593,17 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
     return WPCCC_OK;
 }
 
+// Reads and clears the device word in which the tensor-core kernels' bounded waits record a give-up.
+wpccc_status check_tc_err(wpccc_basis_s* B, const char* where) {
+    if (!B->tc_err) return WPCCC_OK;
+    int e = 0;
+    WPCCC_CUDA(cudaMemcpy(&e, B->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
+    if (e == 0) return WPCCC_OK;
+    WPCCC_CUDA(cudaMemset(B->tc_err, 0, sizeof(int)));
+    return fail(WPCCC_ETIMEOUT, std::string(where) + ": a wait of a tensor-core kernel timed out (stage " +
+                                    std::to_string(e) + ")");
+}
+
 // Grows the basis-owned scratch buffer to at least `bytes`.
 wpccc_status ensure_workspace(wpccc_basis_s* B, size_t bytes) {
     if (B->ws_bytes >= bytes) return WPCCC_OK;
@@ -1616,12 +1658,16 @@ static wpccc_status matrix_elements_prec(wpccc_basis B, double b, double v, int 
     if (!(b > 0.0) || !(v > 0.0)) return fail(WPCCC_EINVAL, "wpccc_matrix_elements: b and v must be > 0");
     if (precision == 3 || precision == 4) {
         WPCCC_CUDA(cudaSetDevice(B->device));
-        wpccc_status ts = tc_prepare(B);
+        wpccc_status ts = tc_prepare(B, true);
         if (ts != WPCCC_OK) return ts;
     }
     WPCCC_CUDA(cudaSetDevice(B->device));
+    if (precision == ELEM_F64) {
+        wpccc_status rs = fp64_route(B, &precision);
+        if (rs != WPCCC_OK) return rs;
+    }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, precision);
     // evaluations per launch bounded by the workspace limit
     size_t per = L.bytes_per_eval + sizeof(EvalDesc);
     int chunk = (int)std::min<size_t>({(size_t)nz, (size_t)MAX_EVALS_PER_LAUNCH,
@@ -1644,14 +1690,7 @@ static wpccc_status matrix_elements_prec(wpccc_basis B, double b, double v, int 
         // the host list is reused: wait for the copy before refilling it
         WPCCC_CUDA(cudaStreamSynchronize(st));
     }
-    if (precision == 3 || precision == 4) {
-        int e = 0;
-        WPCCC_CUDA(cudaMemcpy(&e, B->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-        if (e) {
-            WPCCC_CUDA(cudaMemset(B->tc_err, 0, sizeof(int)));
-            return fail(WPCCC_ETIMEOUT, "a wait of the tensor-core contraction timed out (stage " + std::to_string(e) + ")");
-        }
-    }
+    if (precision >= ELEM_TC4) return check_tc_err(B, "wpccc_matrix_elements");
     return WPCCC_OK;
 }
 }  // namespace wpccc

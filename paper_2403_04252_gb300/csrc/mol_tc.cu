@@ -36,12 +36,15 @@ constexpr int TC_TILE_STATES = 56;
 // Row tiles: each q' group cut into tiles of at most 56 states (near-equal sizes).  A tile of n states owns
 // 2 n consecutive rows of the slice planes: its A_T r_T rows, then its A_T r_T V_T rows.  Enables the
 // layout on the basis.
-wpccc_status tc_prepare(wpccc_basis_s* B) {
-    if (B->tc_layout) return WPCCC_OK;
+wpccc_status tc_prepare(wpccc_basis_s* B, bool tables) {
+    wpccc_status s;
+    if (B->tc_layout) {
+        if (tables && !B->fT2 && (s = split_table(B->T.f, (long long)B->T.n_rad * B->Nr, &B->fT2)) != WPCCC_OK) return s;
+        if (tables && !B->fP2 && (s = split_table(B->P.f, (long long)B->P.n_rad * B->Nr, &B->fP2)) != WPCCC_OK) return s;
+        return WPCCC_OK;
+    }
     if (B->n_centres != 2) return fail(WPCCC_EUNSUPPORTED, "the tensor-core contraction needs a two-centre basis");
     if (!encode_fn()) return fail(WPCCC_EUNSUPPORTED, "tensor-core contraction: cuTensorMapEncodeTiled unavailable");
-    if (B->G % 128 != 0)
-        return fail(WPCCC_EUNSUPPORTED, "tensor-core contraction: the node count must be a multiple of 128");
     const int L = B->T.lmax;
     std::vector<std::vector<int>> groups(2 * L + 1);
     for (int i = 0; i < B->N_T; ++i) groups[B->T.h_st_m[i] + L].push_back(i);
@@ -84,18 +87,15 @@ wpccc_status tc_prepare(wpccc_basis_s* B) {
         WPCCC_CUDA(cudaMemcpy(hs.data(), B->half_state, B->n_half * sizeof(int), cudaMemcpyDeviceToHost));
         for (int h = 0; h < B->n_half; ++h) halfq[h] = B->P.h_st_m[hs[h]];
     }
-    wpccc_status s;
     if ((s = up(&B->tc_row, trow)) != WPCCC_OK) return s;
     if ((s = up(&B->qg_off, qg)) != WPCCC_OK) return s;
     if ((s = up(&B->qg_rows, rows)) != WPCCC_OK) return s;
     if ((s = up(&B->tc_halfq, halfq)) != WPCCC_OK) return s;
     if ((s = ensure_tc_err(B)) != WPCCC_OK) return s;
-    if ((s = split_table(B->T.f, (long long)B->T.n_rad * B->Nr, &B->fT2)) != WPCCC_OK) return s;
-    if ((s = split_table(B->P.f, (long long)B->P.n_rad * B->Nr, &B->fP2)) != WPCCC_OK) return s;
     B->n_qgroups = ntl;
     B->qg_max = qmax;
     B->tc_layout = true;
-    return WPCCC_OK;
+    return tables ? tc_prepare(B, true) : WPCCC_OK;
 }
 
 wpccc_status ensure_tc_err(wpccc_basis_s* B) {

@@ -632,9 +632,9 @@ wpccc_status launch_mol_tc64(wpccc_basis_s* B, int nev, const void* node, double
                              int slices) {
     if (slices != OZ_FAST_SLICES && slices != OZ_SLICES)
         return fail(WPCCC_EINVAL, "tensor-core contraction: 4 or 7 slices");
-    if (!B->tc_layout) return fail(WPCCC_EINVAL, "tensor-core layout not prepared");
+    if (!B->tc_layout || !B->fT2) return fail(WPCCC_EINVAL, "tensor-core layout not prepared");
     if (B->G % (T6_K * T6_WIN) != 0) return fail(WPCCC_EUNSUPPORTED, "the node count must be a multiple of 128");
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, slices == OZ_SLICES ? ELEM_TC7 : ELEM_TC4);
     const size_t node_bytes = L.node_doubles * sizeof(double);
     // seven slice planes as one 3-D bf16 tensor: x = node (G), y = slice plane row (7 x tc_rows), z = evaluation
     Tc64Maps maps;

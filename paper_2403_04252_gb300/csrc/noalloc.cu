@@ -50,7 +50,7 @@ extern "C" wpccc_status wpccc_matrix_elements_noalloc(wpccc_basis B, double b, d
     if (!B || !z || !S || !H) return fail(WPCCC_EINVAL, "wpccc_matrix_elements_noalloc: null argument");
     if (nz < 1) return fail(WPCCC_EINVAL, "wpccc_matrix_elements_noalloc: nz < 1");
     if (!(b > 0.0) || !(v > 0.0)) return fail(WPCCC_EINVAL, "wpccc_matrix_elements_noalloc: b and v must be > 0");
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, ELEM_F64);
     // one position needs its element scratch plus its entry of the position list (the list is rounded up
     // to 256 bytes, so 256 bytes cover that rounding and any list of up to 256 / sizeof(EvalDesc) entries)
     if (L.bytes_per_eval + 256 > NOALLOC_SCRATCH_BYTES)
@@ -77,7 +77,7 @@ extern "C" wpccc_status wpccc_matrix_elements_noalloc(wpccc_basis B, double b, d
         for (int k = 0; k < n; ++k) ev[k] = EvalDesc{b, v, z[k0 + k], 0, 0};
         WPCCC_CUDA(cudaMemcpyAsync(dev_ev, ev.data(), n * sizeof(EvalDesc), cudaMemcpyHostToDevice, st));
         s = launch_elements(B, dev_ev, n, static_cast<double2*>(S) + k0 * mat, static_cast<double2*>(H) + k0 * mat,
-                            scratch, st);
+                            scratch, st, ELEM_F64);
         if (s != WPCCC_OK) return s;
         // the host list and the scratch are reused by the next chunk
         WPCCC_CUDA(cudaStreamSynchronize(st));

@@ -145,13 +145,15 @@ extern "C" wpccc_status wpccc_overlap_norms(wpccc_basis B, int n_paths, const do
     WPCCC_CUDA(cudaSetDevice(B->device));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t N = (size_t)B->N;
-    const ElemScratch L = elem_scratch_layout(B);
+    int prec = ELEM_F64;
+    wpccc_status s = fp64_route(B, &prec);
+    if (s != WPCCC_OK) return s;
+    const ElemScratch L = elem_scratch_layout(B, prec);
     // positions in groups that the workspace limit holds (scratch of the element kernels), S and H per group
     const int per = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_paths,
                                                                (B->ws_limit - 256) / (L.bytes_per_eval + sizeof(EvalDesc))));
     const size_t need = (size_t)per * L.bytes_per_eval + 256 + (size_t)per * sizeof(EvalDesc);
-    wpccc_status s = ensure_workspace(B, need);
-    if (s != WPCCC_OK) return s;
+    if ((s = ensure_workspace(B, need)) != WPCCC_OK) return s;
     double2* SH = nullptr;
     if (cudaMalloc(&SH, 2 * (size_t)per * N * N * sizeof(double2)) != cudaSuccess) {
         cudaGetLastError();
@@ -169,7 +171,7 @@ extern "C" wpccc_status wpccc_overlap_norms(wpccc_basis B, int n_paths, const do
             s = cuda_fail(e, "cudaMemcpyAsync(positions)");
             break;
         }
-        s = launch_elements(B, dev_ev, n, SH, SH + (size_t)per * N * N, scratch, st, 0);
+        s = launch_elements(B, dev_ev, n, SH, SH + (size_t)per * N * N, scratch, st, prec);
         if (s != WPCCC_OK) break;
         k_overlap_norms<<<n, 256, 0, st>>>((int)N, static_cast<const double2*>(c) + (size_t)p0 * N, SH, out + 2 * p0);
         e = cudaGetLastError();
@@ -177,7 +179,7 @@ extern "C" wpccc_status wpccc_overlap_norms(wpccc_basis B, int n_paths, const do
         if (e != cudaSuccess) s = cuda_fail(e, "k_overlap_norms");
     }
     cudaFree(SH);
-    return s;
+    return s != WPCCC_OK ? s : check_tc_err(B, "wpccc_overlap_norms");
 }
 
 extern "C" wpccc_status wpccc_basis_states(wpccc_basis B, int* qn, double* eps) {

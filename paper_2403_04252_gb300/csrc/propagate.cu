@@ -349,7 +349,7 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     if (precision_mode >= 3 && B->n_centres == 2) {
         if (B->G % 128 != 0)
             return fail(WPCCC_EUNSUPPORTED, "precision modes 3-5 need a node count that is a multiple of 128");
-        wpccc_status ts = tc_prepare(B);
+        wpccc_status ts = tc_prepare(B, true);
         if (ts != WPCCC_OK) return ts;
     }
     const int np = paths->n_paths;
@@ -379,12 +379,16 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     P.df_rhs = P.mixed && precision_mode != 5;
     P.elem_precision = !P.two ? 0
                        : (precision_mode == 1 || precision_mode == 3) ? precision_mode
-                       : (precision_mode == 4 || precision_mode == 5) ? 4 : 0;
+                       : (precision_mode == 4 || precision_mode == 5) ? ELEM_TC7 : ELEM_F64;
+    if (P.two && P.elem_precision == ELEM_F64) {
+        wpccc_status rs = fp64_route(B, &P.elem_precision);
+        if (rs != WPCCC_OK) return rs;
+    }
     P.stage = P.two && !P.mixed && B->solve_mode != WPCCC_SOLVE_MATRIX;
     P.schur = P.two && B->solve_mode == WPCCC_SOLVE_SCHUR;
     const bool want_tc = B->schur_update == WPCCC_SCHUR_UPDATE_TENSOR ||
                          (B->schur_update == WPCCC_SCHUR_UPDATE_AUTO && B->N_P >= 256);
-    P.schur_tc = P.mixed && P.schur && want_tc && schur_tc_applicable(B, elem_scratch_layout(B).bytes_per_eval);
+    P.schur_tc = P.mixed && P.schur && want_tc && schur_tc_applicable(B, elem_scratch_layout(B, P.elem_precision).bytes_per_eval);
     if (P.schur_tc) {
         wpccc_status ts = schur_tc_prepare(B);
         if (ts != WPCCC_OK) return ts;
@@ -398,7 +402,7 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     if (!P.wide && !fits)
         return fail(WPCCC_EINVAL, "wpccc_propagate: N too large for the RK4 kernel's shared memory in this mode");
     const size_t mat = (size_t)N * N;
-    const ElemScratch L = elem_scratch_layout(B);
+    const ElemScratch L = elem_scratch_layout(B, P.elem_precision);
     // device bytes per evaluation: S (two-centre only), H, FP32 factors, pivots and info, element scratch
     P.per_eval = (P.two ? 2 : 1) * mat * sizeof(double2) + (P.mixed ? mat * sizeof(float2) : 0) + L.bytes_per_eval +
                  (P.two ? (size_t)N * sizeof(int) + sizeof(int) : 0) + sizeof(EvalDesc);
@@ -607,7 +611,8 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S) 
         if (P.two) {
             cudaEvent_t e0 = B->prof.begin(PROF_SOLVE, st);
             if (P.mixed && P.schur && P.schur_tc)
-                s = launch_schur_factor_f32_tc(B, nev, bS, bL, bI, P.d_scr, elem_scratch_layout(B).bytes_per_eval, st);
+                s = launch_schur_factor_f32_tc(B, nev, bS, bL, bI, P.d_scr,
+                                               elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
             else if (P.mixed && P.schur) s = launch_schur_factor_f32(N, B->N_T, nev, bS, bL, bI, st);
             else if (P.mixed) s = launch_factor_f32(N, nev, bS, bL, bP, bI, st);
             else if (P.schur) s = launch_schur_factor(N, B->N_T, nev, bS, bI, st);
@@ -697,15 +702,7 @@ wpccc_status propagate_internal(wpccc_basis_s* B, const wpccc_paths* paths, int 
     int flags = 0;
     WPCCC_CUDA(cudaMemcpyAsync(&flags, P.d_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaStreamSynchronize(st));
-    if (B->tc_err) {
-        int e = 0;
-        WPCCC_CUDA(cudaMemcpy(&e, B->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-        if (e) {
-            WPCCC_CUDA(cudaMemset(B->tc_err, 0, sizeof(int)));
-            return fail(WPCCC_ETIMEOUT, "wpccc_propagate: a wait of a tensor-core kernel timed out (stage " +
-                                         std::to_string(e) + ")");
-        }
-    }
+    if ((s = check_tc_err(B, "wpccc_propagate")) != WPCCC_OK) return s;
     s = flags_status(flags);
     if (s != WPCCC_OK) set_error(std::string("wpccc_propagate: ") + wpccc_last_error());
     return s;
@@ -971,17 +968,11 @@ extern "C" wpccc_status wpccc_batch_status(wpccc_batch X, void* stream) {
         if (X->plans[k].d_flags)
             WPCCC_CUDA(cudaMemcpyAsync(&flags[k], X->plans[k].d_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaStreamSynchronize(st));
-    for (int k = 0; k < X->n_sets; ++k) {
-        wpccc_basis_s* B = X->plans[k].B;
-        if (B && B->tc_err) {
-            int e = 0;
-            WPCCC_CUDA(cudaMemcpy(&e, B->tc_err, sizeof(int), cudaMemcpyDeviceToHost));
-            if (e) {
-                WPCCC_CUDA(cudaMemset(B->tc_err, 0, sizeof(int)));
-                return fail(WPCCC_ETIMEOUT, "wpccc_batch_status: a wait of the tensor-core contraction timed out");
-            }
+    for (int k = 0; k < X->n_sets; ++k)
+        if (wpccc_basis_s* B = X->plans[k].B) {
+            wpccc_status ts = check_tc_err(B, "wpccc_batch_status");
+            if (ts != WPCCC_OK) return ts;
         }
-    }
     int all = 0;
     for (int f : flags) all |= f;
     wpccc_status s = flags_status(all);

@@ -131,7 +131,7 @@ struct wpccc_basis_s {
     double refine_tol = 1e-3;   // largest last correction / solution of a refinement (<= 0: not checked)
     long wait_polls = 1L << 20; // polls of an mbarrier before a tensor-core kernel's wait gives up
     // tensor-core contraction (precision mode 3): node tables carry the split operand tables
-    bool tc_layout = false;
+    bool tc_layout = false;     // row tiles made
     int n_qgroups = 0;          // row tiles: target states of one q', at most 56 per tile
     int* tc_row = nullptr;      // [2 N_T]: row of each target state in a split table, then its group's size
     int* tc_err = nullptr;      // device flag: a wait of the tensor-core pipeline gave up
@@ -140,6 +140,9 @@ struct wpccc_basis_s {
     int su_np = 0, su_ntiles = 0;
     int schur_update = WPCCC_SCHUR_UPDATE_AUTO;   // where the mixed Schur forms form I - K^+ K
     int* tc_halfq = nullptr;    // [n_half]: q of each half column
+    int* f64_items = nullptr;   // work lists of the FP64 tensor-core form (mol_fp64.cu); halves follow the items
+    int* f64_halves = nullptr;
+    int n_f64_items = 0;
     float2* fT2 = nullptr;      // [n_rad_T][Nr]: the target's radial tables as double-floats (hi, lo)
     float2* fP2 = nullptr;      // the projectile's
     int* qg_off = nullptr;      // [n_qgroups + 1]: first split-table row of each tile (2 x cumulative size),
@@ -176,18 +179,29 @@ struct ElemScratch {
     size_t ph_off;         // offset of the per-state energy phases exp(i eps_i z / v) (complex, N of them)
     int dtot, npb;         // sizes of their Wigner-d and Legendre parts
     size_t cp_off[2];      // per centre: Eq. 6 coefficients of the position, [LM][LM][nlam] (see k_direct_coef)
-    int tc_rows;           // rows of the tensor-core slice planes (2 N_T), when the basis enables the layout
+    int tc_rows;           // rows of the tensor-core slice planes (2 N_T)
     // tensor-core layout (precision modes 3-5): up to seven bf16 slice planes [7][tc_rows][G], then
     // (offsets in floats) the window scales, A_P and W_K / r_T as double-floats
     size_t t6_sc_off, t6_ap_off, t6_w_off;
+    // FP64 tensor-core form (ELEM_F64_TC): behind the FP64 node tables the digit planes, the scale exponents of the
+    // table rows and of the generated rows, A_P, W_K / r_T and r_T, r_T V_T in FP64 (byte offsets within a position's tables);
+    // Gp: nodes padded to a multiple of 32, f64_nwin: scaling windows
+    int Gp, f64_nwin;
+    size_t f64_pl, f64_ea, f64_eb, f64_ap, f64_w2, f64_r;
 };
-ElemScratch elem_scratch_layout(const wpccc_basis_s* B);
+// Element arithmetic: FP64 on the CUDA cores, FP32, the tensor-core forms of precision modes 3 and 4 / 5, and
+// the FP64 form's contraction on the tensor cores.
+enum : int { ELEM_F64 = 0, ELEM_F32 = 1, ELEM_TC4 = 3, ELEM_TC7 = 4, ELEM_F64_TC = 6 };
+ElemScratch elem_scratch_layout(const wpccc_basis_s* B, int precision);
+void f64_layout(const wpccc_basis_s* B, size_t node_doubles, ElemScratch& L);
+// The element arithmetic of a plain FP64 call (ELEM_F64_TC where the tensor cores take it, else ELEM_F64), with
+// its lists prepared on the basis (before any capture).
+wpccc_status fp64_route(wpccc_basis_s* B, int* precision);
+wpccc_status launch_mol_f64tc(wpccc_basis_s* B, int nev, void* node, double2* mol, int* err, cudaStream_t st);
 
 // Queue the element kernels for `nev` evaluations (device list `evals`), writing
 // S and H (matrix k at S + k*N*N).  S may be null (one-centre propagation).
-// `scratch` must hold elem_scratch_layout(B).bytes_per_eval * nev bytes (unused in
-// one-centre mode).
-// precision 0: FP64 throughout; 1: the Eq. 9 contraction on the FP32 pipe (mixed-precision form).
+// `scratch` must hold elem_scratch_layout(B, precision).bytes_per_eval * nev bytes.
 wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev,
                              double2* S, double2* H, void* scratch, cudaStream_t st, int precision = 0);
 
@@ -206,7 +220,8 @@ enum ProfCat { PROF_NODES = 0, PROF_MOL = 1, PROF_ROT_DIRECT = 2, PROF_SOLVE = 3
 
 // Tensor-core form of the Eq. 9 contraction (precision mode 3): from the node tables of the tensor-core
 // layout into the molecular-frame blocks, for `nev` evaluations.
-wpccc_status tc_prepare(wpccc_basis_s* B);
+// Row tiles of the tensor-core contractions; `tables`: also the radial tables as double-floats (modes 3-5).
+wpccc_status tc_prepare(wpccc_basis_s* B, bool tables);
 wpccc_status rotation_plan(wpccc_basis_s* B);
 // The tensor-core contraction over the slice planes: slices = 7 to FP64 accuracy (precision modes 4, 5),
 // 3 at FP32 level (precision mode 3).
@@ -236,6 +251,7 @@ wpccc_status launch_schur_factor_f32_tc(wpccc_basis_s* B, int nev, const double2
                                         void* scratch, size_t scratch_per_eval, cudaStream_t st);
 // Allocates the device flag of the tensor-core kernels' bounded waits, if the basis has none yet.
 wpccc_status ensure_tc_err(wpccc_basis_s* B);
+wpccc_status check_tc_err(wpccc_basis_s* B, const char* where);
 
 // Queue the batched solve of S X = H (results in place).
 wpccc_status launch_solve(int N, int batch, double2* S, double2* H, int* ipiv, int* info,

@@ -1,5 +1,5 @@
 // Batched complex linear solve S X = H with partial pivoting (the paper's ZGESV
-// step of Eq. 4), one thread block per system, in FP64.
+// step of Eq. 4) in FP64, and the FP32 factorisation of the mixed-precision forms.
 //
 // Blocked right-looking elimination of the augmented matrix [S | H]:
 //   for each panel of NB columns
@@ -10,8 +10,15 @@
 //     4. trailing update A22 -= L21 U12 (complex GEMM on the FP64 pipe)
 //   then blocked back substitution X = U^{-1} Y on H.
 // S is left holding L and U of P S = L U (LAPACK layout), H holds X.
+//
+// A system belongs to a cluster of one to eight blocks: the first factorises the panels, and the 32-column blocks of
+// S and of H belong to the blocks in turn (interchanges, U12 and the trailing update of a column block need the panel
+// only), so each panel takes two cluster barriers and the back substitution none.  One block per system leaves most
+// of the chip idle for a small batch: at two FP64 multiply-adds per clock an SM needs 70 ms for one N = 380 system
+// with N right-hand sides.  Every element goes through the same operations in the same order for any cluster size.
 #include <algorithm>
 
+#include "cluster.cuh"
 #include "wpccc_internal.cuh"
 
 namespace wpccc {
@@ -21,485 +28,301 @@ static_assert(NB == 32, "NB must equal the warp size");
 constexpr int LU_THREADS = 256;
 constexpr int TM = 64, TN = 32;   // update tile, complex elements
 
-// C[m x n] -= A[m x k] * B[k x n], column-major, k <= NB, whole block cooperating.
-__device__ void cta_gemm_sub(double2* __restrict__ C, int ldc, const double2* __restrict__ A, int lda,
-                             const double2* __restrict__ B, int ldb, int m, int n, int k,
-                             double2* sA, double2* sB) {
+template <typename R> struct LuC;
+template <> struct LuC<double> { using type = double2; };
+template <> struct LuC<float> { using type = float2; };
+
+// C[m x n] -= A[m x k] * B[k x n], column-major, k <= NB, n <= TN, whole block cooperating.
+template <typename C2>
+__device__ void cta_gemm_sub(C2* __restrict__ C, int ldc, const C2* __restrict__ A, int lda, const C2* __restrict__ B,
+                             int ldb, int m, int n, int k, C2* sA, C2* sB) {
+    using R = decltype(C2().x);
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const C2 zero = C2{R(0), R(0)};
+    for (int idx = tid; idx < NB * TN; idx += LU_THREADS) {
+        const int kk = idx % NB, jj = idx / NB;
+        sB[kk * TN + jj] = (jj < n && kk < k) ? B[(size_t)kk + (size_t)jj * ldb] : zero;
+    }
     for (int i0 = 0; i0 < m; i0 += TM) {
-        // A tile: sA[kk][ii]
         for (int idx = tid; idx < TM * NB; idx += LU_THREADS) {
-            int ii = idx % TM, kk = idx / TM;
-            sA[kk * TM + ii] = (i0 + ii < m && kk < k) ? A[(size_t)(i0 + ii) + (size_t)kk * lda]
-                                                       : make_double2(0.0, 0.0);
+            const int ii = idx % TM, kk = idx / TM;
+            sA[kk * TM + ii] = (i0 + ii < m && kk < k) ? __ldcg(A + (size_t)(i0 + ii) + (size_t)kk * lda) : zero;
         }
-        for (int j0 = 0; j0 < n; j0 += TN) {
-            for (int idx = tid; idx < NB * TN; idx += LU_THREADS) {
-                int kk = idx % NB, jj = idx / NB;
-                sB[kk * TN + jj] = (j0 + jj < n && kk < k) ? B[(size_t)kk + (size_t)(j0 + jj) * ldb]
-                                                           : make_double2(0.0, 0.0);
-            }
-            __syncthreads();
-            double2 acc[4][2];
+        __syncthreads();
+        C2 acc[4][2];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) acc[a][c] = zero;
+        for (int kk = 0; kk < k; ++kk) {
+            C2 av[4], bv[2];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) av[a] = sA[kk * TM + ty + 16 * a];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) bv[c] = sB[kk * TN + tx + 16 * c];
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int c = 0; c < 2; ++c) acc[a][c] = make_double2(0.0, 0.0);
-            for (int kk = 0; kk < k; ++kk) {
-                double2 av[4], bv[2];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) av[a] = sA[kk * TM + ty + 16 * a];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) bv[c] = sB[kk * TN + tx + 16 * c];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        acc[a][c].x = fma(av[a].x, bv[c].x, acc[a][c].x);
-                        acc[a][c].x = fma(-av[a].y, bv[c].y, acc[a][c].x);
-                        acc[a][c].y = fma(av[a].x, bv[c].y, acc[a][c].y);
-                        acc[a][c].y = fma(av[a].y, bv[c].x, acc[a][c].y);
-                    }
-            }
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                int i = i0 + ty + 16 * a;
-                if (i >= m) continue;
-#pragma unroll
                 for (int c = 0; c < 2; ++c) {
-                    int j = j0 + tx + 16 * c;
-                    if (j >= n) continue;
-                    double2* p = C + (size_t)i + (size_t)j * ldc;
-                    double2 v = *p;
-                    v.x -= acc[a][c].x;
-                    v.y -= acc[a][c].y;
-                    *p = v;
+                    acc[a][c].x = fma(av[a].x, bv[c].x, acc[a][c].x);
+                    acc[a][c].x = fma(-av[a].y, bv[c].y, acc[a][c].x);
+                    acc[a][c].y = fma(av[a].x, bv[c].y, acc[a][c].y);
+                    acc[a][c].y = fma(av[a].y, bv[c].x, acc[a][c].y);
                 }
-            }
-            __syncthreads();
         }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int i = i0 + ty + 16 * a;
+            if (i >= m) continue;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int j = tx + 16 * c;
+                if (j >= n) continue;
+                C2* p = C + (size_t)i + (size_t)j * ldc;
+                C2 v = *p;
+                v.x -= acc[a][c].x;
+                v.y -= acc[a][c].y;
+                *p = v;
+            }
+        }
+        __syncthreads();
     }
 }
 
-__device__ inline double2 crecip(double2 a) {
-    double d = a.x * a.x + a.y * a.y;
-    return make_double2(a.x / d, -a.y / d);
+template <typename C2>
+__device__ inline C2 crecip(C2 a) {
+    const auto d = a.x * a.x + a.y * a.y;
+    return C2{a.x / d, -a.y / d};
+}
+template <typename C2>
+__device__ inline C2 cprod(C2 a, C2 b) {
+    return C2{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
+}
+// x - l u
+template <typename C2>
+__device__ __forceinline__ C2 csub_prod(C2 x, C2 l, C2 u) {
+    x.x = fma(-l.x, u.x, x.x);
+    x.x = fma(l.y, u.y, x.x);
+    x.y = fma(-l.x, u.y, x.y);
+    x.y = fma(-l.y, u.x, x.y);
+    return x;
 }
 
-__global__ void __launch_bounds__(LU_THREADS) k_lu_solve(int N, double2* __restrict__ Sall,
-                                                         double2* __restrict__ Hall, int* __restrict__ ipiv_all,
-                                                         int* __restrict__ info_all) {
-    extern __shared__ double2 lu_smem[];
-    double2* sA = lu_smem;                 // TM * NB
-    double2* sB = sA + TM * NB;            // NB * TN
-    double2* sT = sB + NB * TN;            // NB * NB triangular block
-    double2* sD = sT + NB * NB;            // NB reciprocals of U's diagonal
-    __shared__ double red_v[LU_THREADS / 32];
+// Unblocked LU with partial pivoting of the panel's nb columns from k0 (rows k0..N-1), by one block; pivots (1-based)
+// to ipiv, the first zero pivot to *info.
+template <typename C2>
+__device__ void panel_lu(C2* __restrict__ A, int N, int k0, int nb, int* __restrict__ ipiv, int* info) {
+    using R = decltype(C2().x);
+    __shared__ R red_v[LU_THREADS / 32];
     __shared__ int red_i[LU_THREADS / 32];
-    __shared__ int s_piv[NB];
-    __shared__ int s_info;
-
-    const int sys = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const size_t mat = (size_t)N * N;
-    double2* A = Sall + (size_t)sys * mat;
-    double2* Bm = Hall ? Hall + (size_t)sys * mat : nullptr;
-    int* ipiv = ipiv_all + (size_t)sys * N;
-    if (tid == 0) s_info = 0;
-    __syncthreads();
-
-    for (int k0 = 0; k0 < N; k0 += NB) {
-        const int nb = min(NB, N - k0);
-        // ---- 1. panel factorisation
-        for (int kk = 0; kk < nb; ++kk) {
-            const int k = k0 + kk;
-            double best = -1.0;
-            int bi = N;
-            for (int i = k + tid; i < N; i += LU_THREADS) {
-                double2 a = A[(size_t)i + (size_t)k * N];
-                double v = fabs(a.x) + fabs(a.y);
-                if (v > best) {
-                    best = v;
-                    bi = i;
-                }
+    __shared__ int s_piv;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int kk = 0; kk < nb; ++kk) {
+        const int k = k0 + kk;
+        R best = R(-1);
+        int bi = N;
+        for (int i = k + tid; i < N; i += LU_THREADS) {
+            const C2 a = A[(size_t)i + (size_t)k * N];
+            const R v = fabs(a.x) + fabs(a.y);
+            if (v > best) {
+                best = v;
+                bi = i;
             }
+        }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                double ov = __shfl_down_sync(0xffffffffu, best, off);
-                int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                if (ov > best || (ov == best && oi < bi)) {
-                    best = ov;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) {
-                red_v[warp] = best;
-                red_i[warp] = bi;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double bv = red_v[0];
-                int bix = red_i[0];
-                for (int w = 1; w < LU_THREADS / 32; ++w)
-                    if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
-                        bv = red_v[w];
-                        bix = red_i[w];
-                    }
-                if (bix >= N) bix = k;
-                s_piv[kk] = bix;
-                ipiv[k] = bix + 1;
-                if (bv == 0.0 && s_info == 0) s_info = k + 1;
-            }
-            __syncthreads();
-            const int p = s_piv[kk];
-            if (p != k && tid < nb) {
-                const int c = k0 + tid;
-                double2 t = A[(size_t)k + (size_t)c * N];
-                A[(size_t)k + (size_t)c * N] = A[(size_t)p + (size_t)c * N];
-                A[(size_t)p + (size_t)c * N] = t;
-            }
-            __syncthreads();
-            const double2 piv = A[(size_t)k + (size_t)k * N];
-            if (piv.x != 0.0 || piv.y != 0.0) {
-                const double2 inv = crecip(piv);
-                for (int i = k + 1 + tid; i < N; i += LU_THREADS) {
-                    double2* q = A + (size_t)i + (size_t)k * N;
-                    *q = cmul(*q, inv);
-                }
-            }
-            __syncthreads();
-            const int ncol = nb - kk - 1, nrow = N - k - 1;
-            for (int idx = tid; idx < ncol * nrow; idx += LU_THREADS) {
-                const int i = k + 1 + idx % nrow, j = k + 1 + idx / nrow;
-                const double2 l = A[(size_t)i + (size_t)k * N];
-                const double2 u = A[(size_t)k + (size_t)j * N];
-                double2* q = A + (size_t)i + (size_t)j * N;
-                double2 v = *q;
-                v.x = fma(-l.x, u.x, v.x);
-                v.x = fma(l.y, u.y, v.x);
-                v.y = fma(-l.x, u.y, v.y);
-                v.y = fma(-l.y, u.x, v.y);
-                *q = v;
-            }
-            __syncthreads();
-        }
-        // ---- 2. interchanges on every column outside the panel (S) and on H
-        const int nS = N - nb;
-        const int nH = Bm ? N : 0;
-        for (int c = tid; c < nS + nH; c += LU_THREADS) {
-            double2* col;
-            if (c < nS) {
-                const int cc = c < k0 ? c : c + nb;
-                col = A + (size_t)cc * N;
-            } else {
-                col = Bm + (size_t)(c - nS) * N;
-            }
-            for (int kk = 0; kk < nb; ++kk) {
-                const int p = s_piv[kk], k = k0 + kk;
-                if (p != k) {
-                    double2 t = col[k];
-                    col[k] = col[p];
-                    col[p] = t;
-                }
+        for (int off = 16; off > 0; off >>= 1) {
+            const R ov = __shfl_down_sync(0xffffffffu, best, off);
+            const int oi = __shfl_down_sync(0xffffffffu, bi, off);
+            if (ov > best || (ov == best && oi < bi)) {
+                best = ov;
+                bi = oi;
             }
         }
+        if (lane == 0) {
+            red_v[warp] = best;
+            red_i[warp] = bi;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            R bv = red_v[0];
+            int bix = red_i[0];
+            for (int w = 1; w < LU_THREADS / 32; ++w)
+                if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
+                    bv = red_v[w];
+                    bix = red_i[w];
+                }
+            if (bix >= N) bix = k;
+            s_piv = bix;
+            ipiv[k] = bix + 1;
+            if (bv == R(0) && *info == 0) *info = k + 1;
+        }
+        __syncthreads();
+        const int p = s_piv;
+        if (p != k && tid < nb) {
+            const int c = k0 + tid;
+            const C2 t = A[(size_t)k + (size_t)c * N];
+            A[(size_t)k + (size_t)c * N] = A[(size_t)p + (size_t)c * N];
+            A[(size_t)p + (size_t)c * N] = t;
+        }
+        __syncthreads();
+        const C2 piv = A[(size_t)k + (size_t)k * N];
+        if (piv.x != R(0) || piv.y != R(0)) {
+            const C2 inv = crecip(piv);
+            for (int i = k + 1 + tid; i < N; i += LU_THREADS) {
+                C2* q = A + (size_t)i + (size_t)k * N;
+                *q = cprod(*q, inv);
+            }
+        }
+        __syncthreads();
+        const int ncol = nb - kk - 1, nrow = N - k - 1;
+        for (int idx = tid; idx < ncol * nrow; idx += LU_THREADS) {
+            const int i = k + 1 + idx % nrow, j = k + 1 + idx / nrow;
+            C2* q = A + (size_t)i + (size_t)j * N;
+            *q = csub_prod(*q, A[(size_t)i + (size_t)k * N], A[(size_t)k + (size_t)j * N]);
+        }
+        __syncthreads();
+    }
+}
+
+// One system per cluster.  R = double: Sall is factorised in place and, with Hall, S X = H solved.  R = float (the mixed
+// forms' preconditioner): S is read in FP64, rounded to FP32 into Fall and factorised there; Hall is null.
+template <typename R>
+__global__ void __launch_bounds__(LU_THREADS) k_lu(int N, const double2* Sall, typename LuC<R>::type* Fall,
+                                                   typename LuC<R>::type* __restrict__ Hall, int* __restrict__ ipiv_all,
+                                                   int* __restrict__ info_all) {
+    using C2 = typename LuC<R>::type;
+    extern __shared__ __align__(16) unsigned char lu_smem[];
+    C2* sA = reinterpret_cast<C2*>(lu_smem);   // TM * NB
+    C2* sB = sA + TM * NB;                     // NB * TN
+    C2* sT = sB + NB * TN;                     // NB * NB triangular block
+    C2* sD = sT + NB * NB;                     // NB reciprocals of U's diagonal
+    __shared__ int s_piv[NB];
+    const int rank = cluster_rank(), size = cluster_size();
+    const int sys = blockIdx.x / size, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int WARPS = LU_THREADS / 32;
+    const size_t mat = (size_t)N * N;
+    const C2 zero = C2{R(0), R(0)};
+    C2* A = Fall + (size_t)sys * mat;
+    C2* Bm = Hall ? Hall + (size_t)sys * mat : nullptr;
+    int* ipiv = ipiv_all + (size_t)sys * N;
+    int* info = info_all + sys;
+    if (sizeof(R) == 4) {
+        const double2* S = Sall + (size_t)sys * mat;
+        for (size_t q = (size_t)rank * LU_THREADS + tid; q < mat; q += (size_t)size * LU_THREADS)
+            A[q] = C2{(R)S[q].x, (R)S[q].y};
+    }
+    if (rank == 0 && tid == 0) *info = 0;
+    cluster_sync_all();
+    const int nbA = (N + NB - 1) / NB, nbH = Bm ? nbA : 0;   // column blocks of S, then of H
+    for (int k0 = 0; k0 < N; k0 += NB) {
+        const int nb = min(NB, N - k0), kb = k0 / NB;
+        // ---- 1. panel factorisation
+        if (rank == 0) panel_lu(A, N, k0, nb, ipiv, info);
+        cluster_sync_all();
+        if (tid < nb) s_piv[tid] = __ldcg(ipiv + k0 + tid) - 1;
         // L11 (unit lower) into shared memory
         for (int idx = tid; idx < NB * NB; idx += LU_THREADS) {
             const int i = idx % NB, j = idx / NB;
-            sT[idx] = (i < nb && j < nb) ? A[(size_t)(k0 + i) + (size_t)(k0 + j) * N] : make_double2(0.0, 0.0);
+            sT[idx] = (i < nb && j < nb) ? __ldcg(A + (size_t)(k0 + i) + (size_t)(k0 + j) * N) : zero;
         }
         __syncthreads();
-        // ---- 3. U12 = L11^{-1} A12 for trailing S columns and all H columns:
-        //         one warp per column, lane i holds row k0 + i (NB == warp size)
-        const int nTr = N - k0 - nb;
-        for (int c = warp; c < nTr + nH; c += LU_THREADS / 32) {
-            double2* col = (c < nTr) ? A + (size_t)(k0 + nb + c) * N + k0 : Bm + (size_t)(c - nTr) * N + k0;
-            double2 x = lane < nb ? col[lane] : make_double2(0.0, 0.0);
-            for (int j = 0; j < nb - 1; ++j) {
-                const double xr = __shfl_sync(0xffffffffu, x.x, j);
-                const double xi = __shfl_sync(0xffffffffu, x.y, j);
-                if (lane > j) {
-                    const double2 l = sT[j * NB + lane];
-                    x.x = fma(-l.x, xr, x.x);
-                    x.x = fma(l.y, xi, x.x);
-                    x.y = fma(-l.x, xi, x.y);
-                    x.y = fma(-l.y, xr, x.y);
-                }
-            }
-            if (lane < nb) col[lane] = x;
-        }
-        __syncthreads();
-        // ---- 4. trailing update
-        const int m = N - k0 - nb;
-        if (m > 0) {
-            const double2* L21 = A + (size_t)(k0 + nb) + (size_t)k0 * N;
-            if (nTr > 0)
-                cta_gemm_sub(A + (size_t)(k0 + nb) + (size_t)(k0 + nb) * N, N, L21, N,
-                             A + (size_t)k0 + (size_t)(k0 + nb) * N, N, m, nTr, nb, sA, sB);
-            if (Bm) cta_gemm_sub(Bm + (size_t)(k0 + nb), N, L21, N, Bm + (size_t)k0, N, m, N, nb, sA, sB);
-        }
-        __syncthreads();
-    }
-
-    const int info = s_info;
-    if (tid == 0) info_all[sys] = info;
-    if (info != 0 || !Bm) return;   // factor only, or no solution for a singular system (as ZGESV)
-
-    // ---- back substitution X = U^{-1} Y
-    const int last = ((N - 1) / NB) * NB;
-    for (int kb = last; kb >= 0; kb -= NB) {
-        const int nb = min(NB, N - kb);
-        for (int idx = tid; idx < NB * NB; idx += LU_THREADS) {
-            const int i = idx % NB, j = idx / NB;
-            sT[idx] = (i < nb && j < nb) ? A[(size_t)(kb + i) + (size_t)(kb + j) * N] : make_double2(0.0, 0.0);
-        }
-        if (tid < NB) sD[tid] = tid < nb ? crecip(A[(size_t)(kb + tid) + (size_t)(kb + tid) * N]) : make_double2(0.0, 0.0);
-        __syncthreads();
-        for (int c = warp; c < N; c += LU_THREADS / 32) {
-            double2* col = Bm + (size_t)c * N + kb;
-            double2 x = lane < nb ? col[lane] : make_double2(0.0, 0.0);
-            for (int j = nb - 1; j >= 0; --j) {
-                if (lane == j) x = cmul(x, sD[j]);
-                const double xr = __shfl_sync(0xffffffffu, x.x, j);
-                const double xi = __shfl_sync(0xffffffffu, x.y, j);
-                if (lane < j) {
-                    const double2 u = sT[j * NB + lane];
-                    x.x = fma(-u.x, xr, x.x);
-                    x.x = fma(u.y, xi, x.x);
-                    x.y = fma(-u.x, xi, x.y);
-                    x.y = fma(-u.y, xr, x.y);
-                }
-            }
-            if (lane < nb) col[lane] = x;
-        }
-        __syncthreads();
-        if (kb > 0)
-            cta_gemm_sub(Bm, N, A + (size_t)kb * N, N, Bm + kb, N, kb, N, nb, sA, sB);
-        __syncthreads();
-    }
-}
-
-// ---------------------------------------------------------------------------
-// FP32 factorisation for the mixed-precision form: P S = L U with S read in FP64,
-// rounded to FP32 and factorised on the FP32 pipe.  The factors serve as the
-// preconditioner of FP64 iterative refinement (the residuals use the FP64 S).
-// ---------------------------------------------------------------------------
-__device__ inline float2 cmulf(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-__device__ void cta_gemm_sub_f(float2* __restrict__ C, int ldc, const float2* __restrict__ A, int lda,
-                               const float2* __restrict__ B, int ldb, int m, int n, int k, float2* sA,
-                               float2* sB) {
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    for (int i0 = 0; i0 < m; i0 += TM) {
-        for (int idx = tid; idx < TM * NB; idx += LU_THREADS) {
-            int ii = idx % TM, kk = idx / TM;
-            sA[kk * TM + ii] = (i0 + ii < m && kk < k) ? A[(size_t)(i0 + ii) + (size_t)kk * lda] : make_float2(0.f, 0.f);
-        }
-        for (int j0 = 0; j0 < n; j0 += TN) {
-            for (int idx = tid; idx < NB * TN; idx += LU_THREADS) {
-                int kk = idx % NB, jj = idx / NB;
-                sB[kk * TN + jj] = (j0 + jj < n && kk < k) ? B[(size_t)kk + (size_t)(j0 + jj) * ldb] : make_float2(0.f, 0.f);
-            }
-            __syncthreads();
-            float2 acc[4][2];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) acc[a][c] = make_float2(0.f, 0.f);
-            for (int kk = 0; kk < k; ++kk) {
-                float2 av[4], bv[2];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) av[a] = sA[kk * TM + ty + 16 * a];
-#pragma unroll
-                for (int c = 0; c < 2; ++c) bv[c] = sB[kk * TN + tx + 16 * c];
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        acc[a][c].x = fmaf(av[a].x, bv[c].x, acc[a][c].x);
-                        acc[a][c].x = fmaf(-av[a].y, bv[c].y, acc[a][c].x);
-                        acc[a][c].y = fmaf(av[a].x, bv[c].y, acc[a][c].y);
-                        acc[a][c].y = fmaf(av[a].y, bv[c].x, acc[a][c].y);
-                    }
-            }
-#pragma unroll
-            for (int a = 0; a < 4; ++a) {
-                int i = i0 + ty + 16 * a;
-                if (i >= m) continue;
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    int j = j0 + tx + 16 * c;
-                    if (j >= n) continue;
-                    float2* p = C + (size_t)i + (size_t)j * ldc;
-                    float2 v = *p;
-                    v.x -= acc[a][c].x;
-                    v.y -= acc[a][c].y;
-                    *p = v;
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-__global__ void __launch_bounds__(LU_THREADS) k_lu_factor_f32(int N, const double2* __restrict__ Sall,
-                                                              float2* __restrict__ LUall, int* __restrict__ ipiv_all,
-                                                              int* __restrict__ info_all) {
-    extern __shared__ float2 luf_smem[];
-    float2* sA = luf_smem;            // TM * NB
-    float2* sB = sA + TM * NB;        // NB * TN
-    float2* sT = sB + NB * TN;        // NB * NB
-    __shared__ float red_v[LU_THREADS / 32];
-    __shared__ int red_i[LU_THREADS / 32];
-    __shared__ int s_piv[NB];
-    __shared__ int s_info;
-    const int sys = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const size_t mat = (size_t)N * N;
-    const double2* S = Sall + (size_t)sys * mat;
-    float2* A = LUall + (size_t)sys * mat;
-    int* ipiv = ipiv_all + (size_t)sys * N;
-    for (size_t q = tid; q < mat; q += LU_THREADS) A[q] = make_float2((float)S[q].x, (float)S[q].y);
-    if (tid == 0) s_info = 0;
-    __syncthreads();
-    for (int k0 = 0; k0 < N; k0 += NB) {
-        const int nb = min(NB, N - k0);
-        for (int kk = 0; kk < nb; ++kk) {
-            const int k = k0 + kk;
-            float best = -1.f;
-            int bi = N;
-            for (int i = k + tid; i < N; i += LU_THREADS) {
-                float2 a = A[(size_t)i + (size_t)k * N];
-                float v = fabsf(a.x) + fabsf(a.y);
-                if (v > best) {
-                    best = v;
-                    bi = i;
-                }
-            }
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                float ov = __shfl_down_sync(0xffffffffu, best, off);
-                int oi = __shfl_down_sync(0xffffffffu, bi, off);
-                if (ov > best || (ov == best && oi < bi)) {
-                    best = ov;
-                    bi = oi;
-                }
-            }
-            if (lane == 0) {
-                red_v[warp] = best;
-                red_i[warp] = bi;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                float bv = red_v[0];
-                int bix = red_i[0];
-                for (int w = 1; w < LU_THREADS / 32; ++w)
-                    if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
-                        bv = red_v[w];
-                        bix = red_i[w];
-                    }
-                if (bix >= N) bix = k;
-                s_piv[kk] = bix;
-                ipiv[k] = bix + 1;
-                if (bv == 0.f && s_info == 0) s_info = k + 1;
-            }
-            __syncthreads();
-            const int p = s_piv[kk];
-            if (p != k && tid < nb) {
-                const int c = k0 + tid;
-                float2 t = A[(size_t)k + (size_t)c * N];
-                A[(size_t)k + (size_t)c * N] = A[(size_t)p + (size_t)c * N];
-                A[(size_t)p + (size_t)c * N] = t;
-            }
-            __syncthreads();
-            const float2 piv = A[(size_t)k + (size_t)k * N];
-            if (piv.x != 0.f || piv.y != 0.f) {
-                const float d = piv.x * piv.x + piv.y * piv.y;
-                const float2 inv = make_float2(piv.x / d, -piv.y / d);
-                for (int i = k + 1 + tid; i < N; i += LU_THREADS) {
-                    float2* q = A + (size_t)i + (size_t)k * N;
-                    *q = cmulf(*q, inv);
-                }
-            }
-            __syncthreads();
-            const int ncol = nb - kk - 1, nrow = N - k - 1;
-            for (int idx = tid; idx < ncol * nrow; idx += LU_THREADS) {
-                const int i = k + 1 + idx % nrow, j = k + 1 + idx / nrow;
-                const float2 l = A[(size_t)i + (size_t)k * N];
-                const float2 u = A[(size_t)k + (size_t)j * N];
-                float2* q = A + (size_t)i + (size_t)j * N;
-                float2 v = *q;
-                v.x = fmaf(-l.x, u.x, v.x);
-                v.x = fmaf(l.y, u.y, v.x);
-                v.y = fmaf(-l.x, u.y, v.y);
-                v.y = fmaf(-l.y, u.x, v.y);
-                *q = v;
-            }
-            __syncthreads();
-        }
-        const int nS = N - nb;
-        for (int c = tid; c < nS; c += LU_THREADS) {
-            const int cc = c < k0 ? c : c + nb;
-            float2* col = A + (size_t)cc * N;
+        // ---- 2. interchanges on this block's columns outside the panel (a warp per column block, a column per lane)
+        for (int t = warp; t * size + rank < nbA + nbH; t += WARPS) {
+            const int cb = t * size + rank;
+            const int c = (cb < nbA ? cb : cb - nbA) * NB + lane;
+            if (cb == kb || c >= N) continue;
+            C2* col = (cb < nbA ? A : Bm) + (size_t)c * N;
             for (int kk = 0; kk < nb; ++kk) {
                 const int p = s_piv[kk], k = k0 + kk;
                 if (p != k) {
-                    float2 t = col[k];
+                    const C2 q = col[k];
                     col[k] = col[p];
-                    col[p] = t;
+                    col[p] = q;
                 }
             }
         }
+        __syncthreads();
+        // ---- 3. U12 = L11^{-1} A12 for this block's trailing S columns and H columns: a warp per column, lane i holds
+        //         row k0 + i; 4. their trailing update
+        const int m = N - k0 - nb;
+        for (int cb = rank; cb < nbA + nbH; cb += size) {
+            if (cb <= kb) continue;
+            C2* base = (cb < nbA ? A : Bm) + (size_t)(cb < nbA ? cb : cb - nbA) * NB * N;
+            const int n = min(NB, N - (cb < nbA ? cb : cb - nbA) * NB);
+            for (int c = warp; c < n; c += WARPS) {
+                C2* col = base + (size_t)c * N + k0;
+                C2 x = lane < nb ? col[lane] : zero;
+                for (int j = 0; j < nb - 1; ++j) {
+                    const C2 u = C2{__shfl_sync(0xffffffffu, x.x, j), __shfl_sync(0xffffffffu, x.y, j)};
+                    if (lane > j) x = csub_prod(x, sT[j * NB + lane], u);
+                }
+                if (lane < nb) col[lane] = x;
+            }
+            __syncthreads();
+            if (m > 0)
+                cta_gemm_sub<C2>(base + k0 + nb, N, A + (size_t)(k0 + nb) + (size_t)k0 * N, N, base + k0, N, m, n, nb, sA, sB);
+        }
+        cluster_sync_all();
+    }
+    if (!Bm || __ldcg(info) != 0) return;   // factor only, or no solution for a singular system (as ZGESV)
+
+    // ---- back substitution X = U^{-1} Y, every block on its own columns of H
+    for (int kb = ((N - 1) / NB) * NB; kb >= 0; kb -= NB) {
+        const int nb = min(NB, N - kb);
         for (int idx = tid; idx < NB * NB; idx += LU_THREADS) {
             const int i = idx % NB, j = idx / NB;
-            sT[idx] = (i < nb && j < nb) ? A[(size_t)(k0 + i) + (size_t)(k0 + j) * N] : make_float2(0.f, 0.f);
+            sT[idx] = (i < nb && j < nb) ? __ldcg(A + (size_t)(kb + i) + (size_t)(kb + j) * N) : zero;
         }
+        if (tid < NB) sD[tid] = tid < nb ? crecip(__ldcg(A + (size_t)(kb + tid) + (size_t)(kb + tid) * N)) : zero;
         __syncthreads();
-        const int nTr = N - k0 - nb;
-        for (int c = warp; c < nTr; c += LU_THREADS / 32) {
-            float2* col = A + (size_t)(k0 + nb + c) * N + k0;
-            float2 x = lane < nb ? col[lane] : make_float2(0.f, 0.f);
-            for (int j = 0; j < nb - 1; ++j) {
-                const float xr = __shfl_sync(0xffffffffu, x.x, j);
-                const float xi = __shfl_sync(0xffffffffu, x.y, j);
-                if (lane > j) {
-                    const float2 l = sT[j * NB + lane];
-                    x.x = fmaf(-l.x, xr, x.x);
-                    x.x = fmaf(l.y, xi, x.x);
-                    x.y = fmaf(-l.x, xi, x.y);
-                    x.y = fmaf(-l.y, xr, x.y);
+        for (int cb = nbA + (rank + size - nbA % size) % size; cb < nbA + nbH; cb += size) {
+            C2* base = Bm + (size_t)(cb - nbA) * NB * N;
+            const int n = min(NB, N - (cb - nbA) * NB);
+            for (int c = warp; c < n; c += WARPS) {
+                C2* col = base + (size_t)c * N + kb;
+                C2 x = lane < nb ? col[lane] : zero;
+                for (int j = nb - 1; j >= 0; --j) {
+                    if (lane == j) x = cprod(x, sD[j]);
+                    const C2 u = C2{__shfl_sync(0xffffffffu, x.x, j), __shfl_sync(0xffffffffu, x.y, j)};
+                    if (lane < j) x = csub_prod(x, sT[j * NB + lane], u);
                 }
+                if (lane < nb) col[lane] = x;
             }
-            if (lane < nb) col[lane] = x;
+            __syncthreads();
+            if (kb > 0) cta_gemm_sub<C2>(base, N, A + (size_t)kb * N, N, base + kb, N, kb, n, nb, sA, sB);
         }
-        __syncthreads();
-        if (nTr > 0)
-            cta_gemm_sub_f(A + (size_t)(k0 + nb) + (size_t)(k0 + nb) * N, N, A + (size_t)(k0 + nb) + (size_t)k0 * N, N,
-                           A + (size_t)k0 + (size_t)(k0 + nb) * N, N, nTr, nTr, nb, sA, sB);
         __syncthreads();
     }
-    if (tid == 0) info_all[sys] = s_info;
+}
+
+// Blocks per system: the chip's SMs shared out over the batch, as long as each has two column blocks.
+static int lu_cluster(int N, int batch, bool rhs, int device_sms) {
+    const int blocks = (N + NB - 1) / NB * (rhs ? 2 : 1);
+    return std::max(1, std::min({8, device_sms / batch, blocks / 2}));
+}
+
+template <typename R>
+static wpccc_status lu_launch(int N, int batch, const double2* S, typename LuC<R>::type* F, typename LuC<R>::type* H,
+                              int* ipiv, int* info, cudaStream_t st) {
+    using C2 = typename LuC<R>::type;
+    if (batch == 0) return WPCCC_OK;
+    const int smem = (int)(sizeof(C2) * (TM * NB + NB * TN + NB * NB + NB));
+    WPCCC_CUDA(cudaFuncSetAttribute(k_lu<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    int dev = 0, sms = 0;
+    WPCCC_CUDA(cudaGetDevice(&dev));
+    WPCCC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    ClusterLaunch L(batch, lu_cluster(N, batch, H != nullptr, sms), LU_THREADS, smem, st);
+    WPCCC_CUDA(cudaLaunchKernelEx(&L.cfg, k_lu<R>, N, S, F, H, ipiv, info));
+    return WPCCC_OK;
 }
 
 wpccc_status launch_factor_f32(int N, int batch, const double2* S, float2* LU, int* ipiv, int* info, cudaStream_t st) {
-    if (batch == 0) return WPCCC_OK;
-    const int smem = (int)(sizeof(float2) * (TM * NB + NB * TN + NB * NB));
-    WPCCC_CUDA(cudaFuncSetAttribute(k_lu_factor_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_lu_factor_f32<<<batch, LU_THREADS, smem, st>>>(N, S, LU, ipiv, info);
-    WPCCC_CHECK_LAUNCH("k_lu_factor_f32");
-    return WPCCC_OK;
+    return lu_launch<float>(N, batch, S, LU, nullptr, ipiv, info, st);
 }
-
-size_t solve_smem_bytes() { return sizeof(double2) * (TM * NB + NB * TN + NB * NB + NB); }
 
 // H == nullptr: factorisation only (P S = L U), no right-hand sides.
 wpccc_status launch_solve(int N, int batch, double2* S, double2* H, int* ipiv, int* info, cudaStream_t st) {
-    if (batch == 0) return WPCCC_OK;
-    const int smem = (int)solve_smem_bytes();
-    WPCCC_CUDA(cudaFuncSetAttribute(k_lu_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    k_lu_solve<<<batch, LU_THREADS, smem, st>>>(N, S, H, ipiv, info);
-    WPCCC_CHECK_LAUNCH("k_lu_solve");
-    return WPCCC_OK;
+    return lu_launch<double>(N, batch, S, S, H, ipiv, info, st);
 }
 
 }  // namespace wpccc

@@ -900,7 +900,7 @@ constexpr int ROT_WARPS_MAX = 8;
 constexpr int ROT_LANE_CAP = 256;   // block entries one item may hold (more when a single pair has more)
 
 // Work items of k_rotate: the radial pairs (a, b) grouped by (l_a, l_b), and per group the number P of
-// pairs one warp takes so that its P NX (2 l_a + 1)(2 l_b + 1) block entries fill the lanes best (the
+// pairs one warp takes so that its P NX (2 l_a + 1)(l_b + 1) half-block entries fill the lanes best (the
 // passes run over all entries of the item, lane by lane).
 wpccc_status rotation_plan(wpccc_basis_s* B) {
     std::vector<int> items, pairs;
@@ -917,11 +917,11 @@ wpccc_status rotation_plan(wpccc_basis_s* B) {
                         }
             const int np = (int)cls.size() / 2;
             if (np == 0) continue;
-            const int E = NX * (2 * la + 1) * (2 * lb + 1);
+            const int E = NX * (2 * la + 1) * (2 * lb + 1), Eh = NX * (2 * la + 1) * (lb + 1);
             int best = 1;
-            double bu = (double)E / (32.0 * ((E + 31) / 32));
+            double bu = (double)Eh / (32.0 * ((Eh + 31) / 32));
             for (int P = 2; P <= np && P * E <= std::max(ROT_LANE_CAP, E); ++P) {
-                const double u = (double)(P * E) / (32.0 * ((P * E + 31) / 32));
+                const double u = (double)(P * Eh) / (32.0 * ((P * Eh + 31) / 32));
                 if (u > bu + 1e-12) {
                     bu = u;
                     best = P;
@@ -945,10 +945,12 @@ wpccc_status rotation_plan(wpccc_basis_s* B) {
 }
 
 // One warp per work item: P radial pairs (a, b) of one (l_a, l_b).  For each pair the (2l_a+1) x (2l_b+1)
-// molecular-frame block of each integral (q < 0 columns from the reflection) is rotated in two passes
-// through shared memory, T[q'][m_b] = sum_q d^{l_b}_{m_b q} X[q'][q], then K[m_a][m_b] =
-// sum_q' d^{l_a}_{m_a q'} T[q'][m_b] with the energy phases; every pass runs over the item's P NX blk
-// entries, lane by lane.
+// molecular-frame block of each integral is rotated in two passes through shared memory,
+// T[q'][m_b] = sum_q d^{l_b}_{m_b q} X[q'][q], then K[m_a][m_b] = sum_q' d^{l_a}_{m_a q'} T[q'][m_b], then given its energy
+// phases; every pass runs over the item's entries, lane by lane.  The FP64 pipe bounds it, so the reflection
+// X[-q'][-q] = (-1)^(q + q') X[q'][q] is used throughout: with d^l_{-m,-q} = (-1)^(m + q) d^l_{m q} it gives
+// K[-m_a][-m_b] = (-1)^(m_a + m_b) K[m_a][m_b] before the phases, so X is read for q >= 0 and T and K are formed for
+// m_b >= 0 only (20 instead of 36 FP64 operations per entry at l = 3; both integrals share an entry's phase).
 __global__ void __launch_bounds__(32 * ROT_WARPS_MAX) k_rotate(RotArgs A, const EvalDesc* __restrict__ ev) {
     extern __shared__ double sd[];     // Wigner d^l_{m q}(theta) for l <= lmax, then per-warp blocks
     const int e = blockIdx.y;
@@ -962,7 +964,8 @@ __global__ void __launch_bounds__(32 * ROT_WARPS_MAX) k_rotate(RotArgs A, const 
     const int p0 = A.items[4 * item], P = A.items[4 * item + 1], la = A.items[4 * item + 2],
               lb = A.items[4 * item + 3];
     const int* pr = A.pairs + 2 * p0;
-    const int na = 2 * la + 1, nbq = 2 * lb + 1, blk = na * nbq, E = NX * blk, PE = P * E;
+    const int na = 2 * la + 1, nbq = 2 * lb + 1, blk = na * nbq, E = NX * blk;
+    const int hb = lb + 1, hblk = na * hb, Eh = NX * hblk, PEh = P * Eh;   // the half blocks, m_b (or q) >= 0
     const int tot_pad = (total + 1) & ~1;
     double2* X = reinterpret_cast<double2*>(sd + tot_pad) + (size_t)warp * 2 * A.rot_block;
     double2* T = X + A.rot_block;
@@ -973,56 +976,63 @@ __global__ void __launch_bounds__(32 * ROT_WARPS_MAX) k_rotate(RotArgs A, const 
     const double* db = sd + offb;
     const size_t plane = (size_t)A.N_T * A.n_half;
     const double2* mol = A.mol + (size_t)e * NX * plane;
-    // molecular blocks, entry p E + x blk + (q' + la) nbq + (q + lb)
-    for (int t = lane; t < PE; t += 32) {
-        const int p = t / E, r0 = t - p * E, x = r0 / blk, r = r0 - x * blk, qp = r / nbq - la, q = r % nbq - lb;
-        const int ra = pr[2 * p], rb = pr[2 * p + 1];
-        int row, col;
-        bool neg = false;
-        if (q >= 0) {
-            row = A.stT_index[ra * (2 * WPCCC_LMAX + 1) + qp + WPCCC_LMAX];
-            col = A.half_of[rb * (WPCCC_LMAX + 1) + q];
-        } else {
-            row = A.stT_index[ra * (2 * WPCCC_LMAX + 1) - qp + WPCCC_LMAX];
-            col = A.half_of[rb * (WPCCC_LMAX + 1) - q];
-            neg = (qp + q) & 1;
-        }
-        double2 val = mol[(size_t)x * plane + (size_t)row * A.n_half + col];
-        if (neg) val = make_double2(-val.x, -val.y);
-        X[t] = val;
+    // molecular half blocks, entry p Eh + x hblk + (q' + la) hb + q
+    for (int t = lane; t < PEh; t += 32) {
+        const int p = t / Eh, r0 = t - p * Eh, x = r0 / hblk, r = r0 - x * hblk, qp = r / hb - la, q = r % hb;
+        const int row = A.stT_index[pr[2 * p] * (2 * WPCCC_LMAX + 1) + qp + WPCCC_LMAX];
+        const int col = A.half_of[pr[2 * p + 1] * (WPCCC_LMAX + 1) + q];
+        X[t] = mol[(size_t)x * plane + (size_t)row * A.n_half + col];
     }
     __syncwarp();
     // T[p][x][q'][m_b] = sum_q d^{lb}_{m_b q} X[p][x][q'][q]
-    for (int t = lane; t < PE; t += 32) {
-        const int r = t % blk, qi = r / nbq, mb = r % nbq;
-        const double2* xr = X + (t - r) + qi * nbq;
-        const double* dr = db + mb * nbq;
-        double re = 0.0, im = 0.0;
-        for (int q = 0; q < nbq; ++q) {
-            re = fma(dr[q], xr[q].x, re);
-            im = fma(dr[q], xr[q].y, im);
+    for (int t = lane; t < PEh; t += 32) {
+        const int r = t % hblk, qi = r / hb, mb = r % hb;
+        const double2* xp = X + (t - r) + qi * hb;              // X[q'][q >= 0]
+        const double2* xm = X + (t - r) + (na - 1 - qi) * hb;   // X[-q'][q >= 0]
+        const double* dr = db + (mb + lb) * nbq + lb;
+        double re = dr[0] * xp[0].x, im = dr[0] * xp[0].y;
+        double sg = ((qi - la) & 1) ? 1.0 : -1.0;   // (-1)^(q' + q) from q = 1 on
+        for (int q = 1; q <= lb; ++q, sg = -sg) {
+            const double dm = sg * dr[-q];
+            re = fma(dr[q], xp[q].x, re);
+            im = fma(dr[q], xp[q].y, im);
+            re = fma(dm, xm[q].x, re);
+            im = fma(dm, xm[q].y, im);
         }
         T[t] = make_double2(re, im);
     }
     __syncwarp();
-    // K, Q [p][x][m_a][m_b] = sum_q' d^{la}_{m_a q'} T[p][x][q'][m_b] with the energy phases, into X
-    const double2* phs = reinterpret_cast<const double2*>(etd + A.ph_off);
-    for (int t = lane; t < PE; t += 32) {
-        const int p = t / E, r = t % blk, mi = r / nbq, mb = r % nbq;
+    // K, Q [p][x][m_a][m_b] = sum_q' d^{la}_{m_a q'} T[p][x][q'][m_b], into X
+    for (int t = lane; t < PEh; t += 32) {
+        const int r = t % hblk, mi = r / hb, mb = r % hb;
         const double* dr = da + mi * na;
         const double2* tc = T + (t - r) + mb;
         double re = 0.0, im = 0.0;
         for (int qi = 0; qi < na; ++qi) {
             const double w = dr[qi];
-            const double2 tv = tc[qi * nbq];
+            const double2 tv = tc[qi * hb];
             re = fma(w, tv.x, re);
             im = fma(w, tv.y, im);
         }
+        X[t] = make_double2(re, im);
+    }
+    __syncwarp();
+    // the whole blocks with the energy phases, entry p E + x blk + (m_a + la) nbq + (m_b + lb), into T
+    const double2* phs = reinterpret_cast<const double2*>(etd + A.ph_off);
+    for (int t = lane; t < P * blk; t += 32) {
+        const int p = t / blk, r = t - p * blk, mi = r / nbq, mb = r % nbq - lb;
         const int ra = pr[2 * p], rb = pr[2 * p + 1];
         const int i = A.stT_index[ra * (2 * WPCCC_LMAX + 1) + (mi - la) + WPCCC_LMAX];
-        const int j = A.stP_index[rb * (2 * WPCCC_LMAX + 1) + (mb - lb) + WPCCC_LMAX];
+        const int j = A.stP_index[rb * (2 * WPCCC_LMAX + 1) + mb + WPCCC_LMAX];
         const double2 ph = cmul(phs[i], cconj(phs[A.N_T + j]));
-        X[t] = cmul(make_double2(re, im), ph);
+        const bool neg = mb < 0 && ((mi - la + mb) & 1);
+        const double2* src = X + p * Eh + (mb < 0 ? (na - 1 - mi) * hb - mb : mi * hb + mb);
+#pragma unroll
+        for (int x = 0; x < NX; ++x) {
+            double2 k = src[x * hblk];
+            if (neg) k = make_double2(-k.x, -k.y);
+            T[p * E + x * blk + r] = cmul(k, ph);
+        }
     }
     __syncwarp();
     // S and H entries: the upper blocks with the target index fastest (consecutive rows of a column), the
@@ -1035,8 +1045,8 @@ __global__ void __launch_bounds__(32 * ROT_WARPS_MAX) k_rotate(RotArgs A, const 
         const int i = A.stT_index[ra * (2 * WPCCC_LMAX + 1) + (mi - la) + WPCCC_LMAX];
         const int j = A.stP_index[rb * (2 * WPCCC_LMAX + 1) + (mb - lb) + WPCCC_LMAX];
         const size_t up = (size_t)i + (size_t)(A.N_T + j) * A.N;     // row i, column N_T + j
-        S[up] = X[p * E + mi * nbq + mb];
-        H[up] = X[p * E + blk + mi * nbq + mb];
+        S[up] = T[p * E + mi * nbq + mb];
+        H[up] = T[p * E + blk + mi * nbq + mb];
     }
     for (int t = lane; t < P * blk; t += 32) {
         const int p = t / blk, r = t - p * blk, mi = r / nbq, mb = r % nbq;
@@ -1044,8 +1054,8 @@ __global__ void __launch_bounds__(32 * ROT_WARPS_MAX) k_rotate(RotArgs A, const 
         const int i = A.stT_index[ra * (2 * WPCCC_LMAX + 1) + (mi - la) + WPCCC_LMAX];
         const int j = A.stP_index[rb * (2 * WPCCC_LMAX + 1) + (mb - lb) + WPCCC_LMAX];
         const size_t lo = (size_t)(A.N_T + j) + (size_t)i * A.N;     // row N_T + j, column i
-        S[lo] = cconj(X[p * E + r]);
-        H[lo] = cconj(X[p * E + blk + r]);     // Eq. 1: the lower-left block of H is Q^+
+        S[lo] = cconj(T[p * E + r]);
+        H[lo] = cconj(T[p * E + blk + r]);     // Eq. 1: the lower-left block of H is Q^+
     }
 }
 

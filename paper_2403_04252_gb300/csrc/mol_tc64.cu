@@ -271,11 +271,17 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
             const uint32_t idesc = bf16_idesc_mn(T6_M, T6_N);
             bool ok = true;
             int last_mma = -1;   // the last chunk whose MMAs were issued (their completion commits to tempty)
+            // the MMA queue is short: the next chunk's barriers are tested between this chunk's MMAs, so that a chunk whose
+            // operands are there follows without the scalar latency of the waits
+            bool ready = false;
+            auto wait = [&](uint32_t bar, uint32_t par, int code) {
+                return mbar_test(bar, par) || mbar_wait(bar, par, abort_flag, A.err, code, A.wait_limit);
+            };
             for (int k = 0; k < nk && ok; ++k) {
                 const int s = k % T6_TSTAGES, s2 = k % T6_GSTAGES, w = k / T6_WIN, b = w & 1;
-                ok = mbar_wait(tfull0 + 8 * s, (k / T6_TSTAGES) & 1, abort_flag, A.err, 11, A.wait_limit);
-                if (ok) ok = mbar_wait(gfull0 + 8 * s2, (k / T6_GSTAGES) & 1, abort_flag, A.err, 16, A.wait_limit);
-                if (ok && k % T6_WIN == 0 && w >= 2) ok = mbar_wait(acce0 + 8 * b, ((w - 2) >> 1) & 1, abort_flag, A.err, 12, A.wait_limit);
+                if (!ready)
+                    ok = wait(tfull0 + 8 * s, (k / T6_TSTAGES) & 1, 11) && wait(gfull0 + 8 * s2, (k / T6_GSTAGES) & 1, 16);
+                if (ok && k % T6_WIN == 0 && w >= 2) ok = wait(acce0 + 8 * b, ((w - 2) >> 1) & 1, 12);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a0 = smem_u32(sm + s * T6_TSTAGE_BYTES), b0 = smem_u32(gsm + s2 * T6_GSTAGE_BYTES);
@@ -297,6 +303,9 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
                             tc_mma(dbase + (uint32_t)(i * T6_N), da + (uint64_t)((i * T6_A_TILE + kk * 32) >> 4),
                                    db + (uint64_t)((kk * 32) >> 4), bf16_idesc_mn(T6_M, (SL - i) * T6_N),
                                    kk == 0 && i == 0 ? fresh : 1u);
+                            if (kk == 1 && i == 0)
+                                ready = k + 1 < nk && mbar_test(tfull0 + 8 * ((k + 1) % T6_TSTAGES), ((k + 1) / T6_TSTAGES) & 1) &&
+                                        mbar_test(gfull0 + 8 * ((k + 1) % T6_GSTAGES), ((k + 1) / T6_GSTAGES) & 1);
                         }
                     }
                 } else {

@@ -295,10 +295,34 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu(int N, const double2* Sall, t
     }
 }
 
-// Blocks per system: the chip's SMs shared out over the batch, as long as each has two column blocks.
-static int lu_cluster(int N, int batch, bool rhs, int device_sms) {
+// Blocks per system: the size that finishes the batch soonest when a cluster's blocks sit on SMs of their own (the FP64
+// pipe bounds the work, so blocks that share an SM gain nothing): ceil(batch / clusters the chip holds) / size, with at
+// least two column blocks per block.  A cluster stays within a group of SMs, so the chip holds fewer clusters than SMs /
+// size: 24 systems, N = 380, with N right-hand sides take 96, 50, 35, 27, 25, 34 and 34 ms with 1, 2, 3, 4, 5, 6 and 8
+// (the rule takes 5; SMs / systems would be 6), 60 systems 98, 51, 65, 50, 62, 61 and 58 (2).
+template <typename R>
+static int lu_cluster(int N, int batch, bool rhs, int (&held)[9], cudaStream_t st) {
+    if (held[1] == 0) {
+        for (int size = 1; size <= 8; ++size) {
+            ClusterLaunch L(1, size, LU_THREADS, 120 * 1024, st);   // more than half an SM's shared memory
+            if (cudaOccupancyMaxActiveClusters(&held[size], k_lu<R>, &L.cfg) != cudaSuccess) {
+                cudaGetLastError();
+                held[size] = 0;
+            }
+        }
+    }
     const int blocks = (N + NB - 1) / NB * (rhs ? 2 : 1);
-    return std::max(1, std::min({8, device_sms / batch, blocks / 2}));
+    int best = 1;
+    double t = 0.0;
+    for (int size = 1; size <= std::max(1, std::min(8, blocks / 2)); ++size) {
+        if (held[size] < 1) continue;
+        const double s = (double)((batch + held[size] - 1) / held[size]) / size;
+        if (size == 1 || s < 0.95 * t) {
+            t = s;
+            best = size;
+        }
+    }
+    return best;
 }
 
 template <typename R>
@@ -307,11 +331,9 @@ static wpccc_status lu_launch(int N, int batch, const double2* S, typename LuC<R
     using C2 = typename LuC<R>::type;
     if (batch == 0) return WPCCC_OK;
     const int smem = (int)(sizeof(C2) * (TM * NB + NB * TN + NB * NB + NB));
-    WPCCC_CUDA(cudaFuncSetAttribute(k_lu<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    int dev = 0, sms = 0;
-    WPCCC_CUDA(cudaGetDevice(&dev));
-    WPCCC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    ClusterLaunch L(batch, lu_cluster(N, batch, H != nullptr, sms), LU_THREADS, smem, st);
+    WPCCC_CUDA(cudaFuncSetAttribute(k_lu<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(smem, 120 * 1024)));
+    static thread_local int held[9] = {};   // clusters an empty chip holds, by size
+    ClusterLaunch L(batch, lu_cluster<R>(N, batch, H != nullptr, held, st), LU_THREADS, smem, st);
     WPCCC_CUDA(cudaLaunchKernelEx(&L.cfg, k_lu<R>, N, S, F, H, ipiv, info));
     return WPCCC_OK;
 }

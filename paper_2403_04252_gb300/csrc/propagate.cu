@@ -11,6 +11,8 @@
 #include <cmath>
 #include <vector>
 
+#include "rk4_fp64.cuh"
+#include "rk4_mixed.cuh"
 #include "rk_device.cuh"
 #include "wpccc_internal.cuh"
 
@@ -61,31 +63,20 @@ struct PosMats {
     const int* piv;
 };
 
-// One block per path: the chunk's RK4 steps (Algorithm 1) with M(z) y = -(i/v) S(z)^{-1} H(z) y:
-//   RK_MATRIX  X = S^{-1} H stored (the paper's form; one-centre: X = H)
-//   RK_STAGE   S^{-1} applied from FP64 LU factors at every stage
-//   RK_SCHUR   S^{-1} applied through the Schur complement's Cholesky factor at every stage
-//   RK_MIXED   S^{-1} applied by FP64 refinement on FP32 LU factors
-//   RK_MIXED_SCHUR  the same on the FP32 Schur factors
-template <int MODE>
-__global__ void __launch_bounds__(RK_THREADS, 1) k_rk4(RkArgs A) {
+// The refined LU forms' sweep (RK_MIXED), one block per path: the chunk's RK4 steps (Algorithm 1) with
+// M(z) y = -(i/v) S(z)^{-1} H(z) y, S^{-1} applied by FP64 refinement on FP32 LU factors.
+__global__ void __launch_bounds__(RK_THREADS, 1) k_rk4_mixed_lu(RkArgs A) {
     extern __shared__ double2 rk_smem[];
     const int N = A.N;
     double2* c = rk_smem;
     double2* y = c + N;
     double2* kv = y + N;
     double2* acc = kv + N;
-    double2* t = acc + N;                       // stage: scratch; mixed: b
-    double2* xs = t + N;                        // mixed: x
-    double2* rs = xs + N;                       // mixed: r
-    float2* ds = reinterpret_cast<float2*>(rs + N);   // mixed: d
-    // 32 x 32 diagonal block of the triangular solves (after the vectors of the mode)
-    double2* us = t + N;                        // Schur: scratch of the projectile part
-    float2* us32 = ds + N + (N & 1);            // mixed Schur: FP32 scratch of the projectile part
-    constexpr bool MIX = MODE == RK_MIXED || MODE == RK_MIXED_SCHUR;
-    void* blk = MODE == RK_MIXED ? (void*)(ds + N + (N & 1))
-                                 : MODE == RK_MIXED_SCHUR ? (void*)(us32 + N + (N & 1))
-                                                          : (MODE == RK_SCHUR ? (void*)(us + N) : (void*)(t + N));
+    double2* t = acc + N;                       // b
+    double2* xs = t + N;                        // x
+    double2* rs = xs + N;                       // r
+    float2* ds = reinterpret_cast<float2*>(rs + N);   // d
+    float2* blk = ds + N + (N & 1);             // 32 x 32 diagonal block of the triangular solves
     const PathChunk pc = A.pcs[blockIdx.x];
     const size_t mat = (size_t)N * N;
     double2* cg = A.c + (size_t)pc.path * N;
@@ -102,15 +93,15 @@ __global__ void __launch_bounds__(RK_THREADS, 1) k_rk4(RkArgs A) {
     auto at = [&](int e) {
         PosMats m;
         m.H = A.H + (size_t)e * mat;
-        m.S = MODE != RK_MATRIX ? A.LU + (size_t)e * mat : nullptr;
-        m.L32 = MIX ? A.LU32 + (size_t)e * mat : nullptr;
-        m.piv = MODE != RK_MATRIX ? A.piv + (size_t)e * N : nullptr;
+        m.S = A.LU + (size_t)e * mat;
+        m.L32 = A.LU32 + (size_t)e * mat;
+        m.piv = A.piv + (size_t)e * N;
         return m;
     };
     // the staging slots of H for the reduced-precision forms' right-hand side (after the mode's vectors)
     Staging sg{};
     const Staging* sgp = nullptr;
-    if (MIX && A.stage_cols > 0) {
+    if (A.stage_cols > 0) {
         sg.buf = reinterpret_cast<double2*>(reinterpret_cast<char*>(rk_smem) + A.stage_off);
         sg.bars = reinterpret_cast<uint64_t*>(sg.buf + (size_t)2 * A.stage_cols * N);
         sg.cols = A.stage_cols;
@@ -118,30 +109,17 @@ __global__ void __launch_bounds__(RK_THREADS, 1) k_rk4(RkArgs A) {
         sgp = &sg;
     }
     auto apply = [&](const PosMats& m, const double2* in, double2* out) {
-        if (MODE == RK_MATRIX) {
-            matvec(m.H, N, in, out);
-            for (int i = threadIdx.x; i < N; i += RK_THREADS) out[i] = make_double2(out[i].y / v, -out[i].x / v);
-            __syncthreads();
-        } else if (MODE == RK_SCHUR) {
-            apply_schur(m.S, m.H, N, A.N_T, v, in, out, t, us, static_cast<double2*>(blk));
-        } else if (MODE == RK_STAGE) {
-            apply_LU(m.S, m.piv, m.H, N, v, in, out, t, static_cast<double2*>(blk));
-        } else if (MODE == RK_MIXED_SCHUR) {
-            apply_schur_mixed(m.S, m.L32, m.H, N, A.N_T, v, A.iters, in, out, t, xs, rs, ds, us32,
-                              static_cast<float2*>(blk), A.tol, A.flags, A.df_rhs != 0, sgp);
-        } else {
-            apply_LU_mixed(m.S, m.L32, m.piv, m.H, N, A.N_T, v, A.iters, in, out, t, xs, rs, ds,
-                           static_cast<float2*>(blk), A.tol, A.flags, A.df_rhs != 0, sgp);
-        }
+        apply_LU_mixed(m.S, m.L32, m.piv, m.H, N, A.N_T, v, A.iters, in, out, t, xs, rs, ds, blk, A.tol, A.flags,
+                       A.df_rhs != 0, sgp);
     };
     PosMats Mz;
     if (pc.start_local >= 0) {
         Mz = at(pc.start_local);
     } else {
         Mz.H = A.carryH + (size_t)pc.path * mat;
-        Mz.S = MODE != RK_MATRIX ? A.carryLU + (size_t)pc.path * mat : nullptr;
-        Mz.L32 = MIX ? A.carryLU32 + (size_t)pc.path * mat : nullptr;
-        Mz.piv = MODE != RK_MATRIX ? A.carryPiv + (size_t)pc.path * N : nullptr;
+        Mz.S = A.carryLU + (size_t)pc.path * mat;
+        Mz.L32 = A.carryLU32 + (size_t)pc.path * mat;
+        Mz.piv = A.carryPiv + (size_t)pc.path * N;
     }
     for (int s = 0; s < pc.nsteps; ++s) {
         const PosMats Mmid = at(pc.first_local + 2 * s), Mnew = at(pc.first_local + 2 * s + 1);
@@ -187,15 +165,218 @@ __global__ void __launch_bounds__(RK_THREADS, 1) k_rk4(RkArgs A) {
     double2* cH = A.carryH + (size_t)pc.path * mat;
     if (Mz.H != cH) {
         for (size_t q = threadIdx.x; q < mat; q += RK_THREADS) cH[q] = Mz.H[q];
+        double2* cL = A.carryLU + (size_t)pc.path * mat;
+        int* cP = A.carryPiv + (size_t)pc.path * N;
+        for (size_t q = threadIdx.x; q < mat; q += RK_THREADS) cL[q] = Mz.S[q];
+        for (int q = threadIdx.x; q < N; q += RK_THREADS) cP[q] = Mz.piv[q];
+        float2* cL32 = A.carryLU32 + (size_t)pc.path * mat;
+        for (size_t q = threadIdx.x; q < mat; q += RK_THREADS) cL32[q] = Mz.L32[q];
+    }
+}
+
+// The refined Schur forms' sweep (rk4_mixed.cuh): one cluster per path.  Every block keeps all vectors and updates them
+// alike; the products and solves inside a stage are shared out.
+__global__ void __launch_bounds__(RC_THREADS, 1) k_rk4_mixed_schur(RkArgs A) {
+    extern __shared__ double2 rk_smem[];
+    const RcCluster cl{cluster_rank(), cluster_size()};
+    const int N = A.N, tid = threadIdx.x;
+    double2* c = rk_smem;
+    double2* y = c + N;
+    double2* acc = y + N;
+    double2* bv = acc + N;
+    double2* x = bv + N;
+    double2* r = x + N;
+    float2* blk = reinterpret_cast<float2*>(r + N);   // 32 x 32
+    float2* d = blk + 32 * 32;
+    float2* u = d + N;
+    float2* w = u + (N - A.N_T);
+    const PathChunk pc = A.pcs[blockIdx.x / cl.size];
+    const size_t mat = (size_t)N * N;
+    double2* cg = A.c + (size_t)pc.path * N;
+    const double iv = 1.0 / pc.v;   // an FP64 division takes some 30 instructions of 64 cycles per warp
+    for (int i = tid; i < N; i += RC_THREADS) c[i] = y[i] = cg[i];
+    if (A.info && cl.rank == 0 && tid == 0) {
+        int bad = 0;
+        if (pc.start_local >= 0 && A.info[pc.start_local] != 0) bad = 1;
+        for (int s = 0; s < 2 * pc.nsteps; ++s)
+            if (A.info[pc.first_local + s] != 0) bad = 1;
+        if (bad) atomicOr(A.flags, FLAG_SINGULAR);
+    }
+    cl.sync();   // every block has started and read its amplitudes
+    auto at = [&](int e) { return PosMats{A.H + (size_t)e * mat, A.LU + (size_t)e * mat, A.LU32 + (size_t)e * mat, nullptr}; };
+    PosMats Mz = pc.start_local >= 0
+                     ? at(pc.start_local)
+                     : PosMats{A.carryH + (size_t)pc.path * mat, A.carryLU + (size_t)pc.path * mat,
+                               A.carryLU32 + (size_t)pc.path * mat, nullptr};
+    for (int s = 0; s < pc.nsteps; ++s) {
+        const PosMats Mmid = at(pc.first_local + 2 * s), Mnew = at(pc.first_local + 2 * s + 1);
+        const double h = A.z[pc.z0 + s + 1] - A.z[pc.z0 + s];
+        const double h2 = 0.5 * h, h6 = h / 6.0;
+#pragma unroll 1
+        for (int st = 1; st <= 4; ++st) {
+            const PosMats& m = st == 1 ? Mz : (st == 4 ? Mnew : Mmid);
+            rc_schur_refined(cl, m.S, m.L32, m.H, N, A.N_T, A.iters, y, bv, x, r, d, u, w, blk, A.tol, A.flags,
+                             A.df_rhs != 0);
+            const double f = st == 3 ? h : h2;
+            for (int i = tid; i < N; i += RC_THREADS) {
+                const double2 k = make_double2(x[i].y * iv, -x[i].x * iv), ci = c[i];
+                if (st == 4) {
+                    const double2 a = make_double2(acc[i].x + k.x, acc[i].y + k.y);
+                    c[i] = y[i] = make_double2(fma(h6, a.x, ci.x), fma(h6, a.y, ci.y));
+                } else {
+                    acc[i] = st == 1 ? k : make_double2(fma(2.0, k.x, acc[i].x), fma(2.0, k.y, acc[i].y));
+                    y[i] = make_double2(fma(f, k.x, ci.x), fma(f, k.y, ci.y));
+                }
+            }
+            __syncthreads();
+        }
+        Mz = Mnew;
+    }
+    bool finite = true;
+    const int first = cl.rank * RC_THREADS + tid, stride = cl.size * RC_THREADS;
+    for (int i = first; i < N; i += stride) {
+        cg[i] = c[i];
+        if (!isfinite(c[i].x) || !isfinite(c[i].y)) finite = false;
+    }
+    if (!finite) atomicOr(A.flags, FLAG_NONFINITE);
+    // carry the matrices at the chunk's last node into the next chunk
+    double2* cH = A.carryH + (size_t)pc.path * mat;
+    if (Mz.H != cH) {
+        double2* cL = A.carryLU + (size_t)pc.path * mat;
+        float2* cL32 = A.carryLU32 + (size_t)pc.path * mat;
+        for (size_t q = first; q < mat; q += stride) {
+            cH[q] = Mz.H[q];
+            cL[q] = Mz.S[q];
+            cL32[q] = Mz.L32[q];
+        }
+    }
+    cl.sync();   // no block leaves while another may still store into its shared memory
+}
+
+// The FP64 forms' sweep (rk4_fp64.cuh): one cluster per path, rows of every product shared out over its blocks.
+template <int MODE>
+__global__ void __launch_bounds__(RC_THREADS, 1) k_rk4_fp64(RkArgs A) {
+    extern __shared__ double2 rk_smem[];
+    const RcCluster cl{cluster_rank(), cluster_size()};
+    const int N = A.N, tid = threadIdx.x;
+    double2* y[2] = {rk_smem, rk_smem + N};       // the stage's input and the next one's, replicated
+    double2* c = rk_smem + 2 * N;                 // this block's rows are current
+    double2* acc = c + N;
+    double2* t = acc + N;                         // two-centre: right-hand side and solution, replicated
+    double2* blk = MODE == RK_MATRIX ? t : t + N; // RC_BLK
+    uint16_t* perm = reinterpret_cast<uint16_t*>(blk + RC_BLK);   // RK_STAGE
+    const PathChunk pc = A.pcs[blockIdx.x / cl.size];
+    const size_t mat = (size_t)N * N;
+    double2* cg = A.c + (size_t)pc.path * N;
+    const double iv = 1.0 / pc.v;
+    for (int i = tid; i < N; i += RC_THREADS) c[i] = y[0][i] = cg[i];
+    if (A.info && cl.rank == 0 && tid == 0) {
+        int bad = 0;
+        if (pc.start_local >= 0 && A.info[pc.start_local] != 0) bad = 1;
+        for (int s = 0; s < 2 * pc.nsteps; ++s)
+            if (A.info[pc.first_local + s] != 0) bad = 1;
+        if (bad) atomicOr(A.flags, FLAG_SINGULAR);
+    }
+    cl.sync();   // every block has started and read its amplitudes
+    auto at = [&](int e) {
+        PosMats m;
+        m.H = A.H + (size_t)e * mat;
+        m.S = MODE != RK_MATRIX ? A.LU + (size_t)e * mat : nullptr;
+        m.L32 = nullptr;
+        m.piv = MODE == RK_STAGE ? A.piv + (size_t)e * N : nullptr;
+        return m;
+    };
+    PosMats Mz;
+    if (pc.start_local >= 0) {
+        Mz = at(pc.start_local);
+    } else {
+        Mz.H = A.carryH + (size_t)pc.path * mat;
+        Mz.S = MODE != RK_MATRIX ? A.carryLU + (size_t)pc.path * mat : nullptr;
+        Mz.L32 = nullptr;
+        Mz.piv = MODE == RK_STAGE ? A.carryPiv + (size_t)pc.path * N : nullptr;
+    }
+    int b = 0;
+    // one RK4 stage from y[b] into y[b ^ 1]: slope k = -(i/v) S^{-1} H y, then the owner of a row updates it
+    RcRows R;   // RK_MATRIX: the first entries of this thread's share of the stage's matrix
+    auto stage = [&](const PosMats& m, int st, double h, double h6, const double2* next) {
+        const double2* in = y[b];
+        double2* out = y[b ^ 1];
+        auto upd = [&](int i, double2 x) {   // x = (S^{-1} H y)_i
+            const double2 k = make_double2(x.y * iv, -x.x * iv), ci = c[i];
+            if (st == 1) acc[i] = k;
+            else if (st < 4) acc[i] = make_double2(fma(2.0, k.x, acc[i].x), fma(2.0, k.y, acc[i].y));
+            if (st < 4) {
+                const double f = st == 3 ? h : 0.5 * h;
+                cl.bcast(out + i, make_double2(fma(f, k.x, ci.x), fma(f, k.y, ci.y)));
+            } else {
+                const double2 a = make_double2(acc[i].x + k.x, acc[i].y + k.y);
+                c[i] = make_double2(fma(h6, a.x, ci.x), fma(h6, a.y, ci.y));
+                cl.bcast(out + i, c[i]);
+            }
+        };
+        int lo, hi;
+        cl.rows(N, lo, hi);
+        if (MODE == RK_MATRIX) {
+            R.apply(m.H + lo, N, hi - lo, N, in, blk, [&](int r, double2 x) { upd(lo + r, x); });
+            if (next) R.load(next + lo, N, hi - lo, N);   // ahead of the barrier
+        } else {
+            rc_matvec(m.H + lo, N, hi - lo, N, in, blk, [&](int r, double2 x) { cl.bcast(t + lo + r, x); });
+            cl.sync();
+            if (MODE == RK_SCHUR) {
+                const int N_T = A.N_T;
+                rc_schur_solve(cl, m.S, N, N_T, t, out, blk);
+                cl.rows(N_T, lo, hi);
+                rc_matvec(m.S + lo + (size_t)N_T * N, N, hi - lo, N - N_T, t + N_T, blk, [&](int r, double2 x) {
+                    upd(lo + r, make_double2(t[lo + r].x - x.x, t[lo + r].y - x.y));
+                });
+                for (int r = tid; r < N - N_T; r += RC_THREADS)
+                    if ((r >> 5) % cl.size == cl.rank) upd(N_T + r, t[N_T + r]);
+            } else {
+                rc_lu_solve(cl, m.S, perm, N, t, out, blk);
+                for (int r = tid; r < N; r += RC_THREADS)
+                    if ((r >> 5) % cl.size == cl.rank) upd(r, t[r]);
+            }
+        }
+        cl.sync();
+        b ^= 1;
+    };
+    if (MODE == RK_STAGE) rc_permutation(Mz.piv, N, perm, blk);
+    if (MODE == RK_MATRIX) {
+        int lo, hi;
+        cl.rows(N, lo, hi);
+        R.load(Mz.H + lo, N, hi - lo, N);
+    }
+    for (int s = 0; s < pc.nsteps; ++s) {
+        const PosMats Mmid = at(pc.first_local + 2 * s), Mnew = at(pc.first_local + 2 * s + 1);
+        const double h = A.z[pc.z0 + s + 1] - A.z[pc.z0 + s], h6 = h / 6.0;
+#pragma unroll 1
+        for (int st = 1; st <= 4; ++st) {
+            const PosMats& m = st == 1 ? Mz : (st == 4 ? Mnew : Mmid);
+            if (MODE == RK_STAGE && (st == 2 || st == 4)) rc_permutation(m.piv, N, perm, blk);
+            // the next stage's matrix, where it is another one
+            stage(m, st, h, h6, st == 1 ? Mmid.H : (st == 3 ? Mnew.H : nullptr));
+        }
+        Mz = Mnew;
+    }
+    bool finite = true;
+    const int first = cl.rank * RC_THREADS + tid, stride = cl.size * RC_THREADS;
+    for (int i = first; i < N; i += stride) {
+        const double2 a = y[b][i];
+        cg[i] = a;
+        if (!isfinite(a.x) || !isfinite(a.y)) finite = false;
+    }
+    if (!finite) atomicOr(A.flags, FLAG_NONFINITE);
+    // carry the matrices at the chunk's last node into the next chunk
+    double2* cH = A.carryH + (size_t)pc.path * mat;
+    if (Mz.H != cH) {
+        for (size_t q = first; q < mat; q += stride) cH[q] = Mz.H[q];
         if (MODE != RK_MATRIX) {
             double2* cL = A.carryLU + (size_t)pc.path * mat;
-            int* cP = A.carryPiv + (size_t)pc.path * N;
-            for (size_t q = threadIdx.x; q < mat; q += RK_THREADS) cL[q] = Mz.S[q];
-            for (int q = threadIdx.x; q < N; q += RK_THREADS) cP[q] = Mz.piv[q];
+            for (size_t q = first; q < mat; q += stride) cL[q] = Mz.S[q];
         }
-        if (MIX) {
-            float2* cL32 = A.carryLU32 + (size_t)pc.path * mat;
-            for (size_t q = threadIdx.x; q < mat; q += RK_THREADS) cL32[q] = Mz.L32[q];
+        if (MODE == RK_STAGE) {
+            int* cP = A.carryPiv + (size_t)pc.path * N;
+            for (int q = first; q < N; q += stride) cP[q] = Mz.piv[q];
         }
     }
 }
@@ -274,13 +455,18 @@ __global__ void __launch_bounds__(WIDE_ROWS) k_rk4_wide(WideArgs A, int s, int s
     }
 }
 
+// Largest N of the shared-memory sweeps, by mode: the size that a call takes (above it a one-centre basis goes to the
+// global-memory layout and a two-centre one is refused).  The sweeps' shared memory stays below 226 KB up to there.
+static int rk_max_states(int mode) {
+    return mode == RK_SCHUR ? 2240 : mode == RK_MIXED_SCHUR ? 1744 : mode == RK_MIXED ? 1860 : 2688;
+}
+
 size_t rk_smem_bytes(int mode, int N) {
-    if (mode == RK_SCHUR) return (size_t)N * 6 * sizeof(double2) + 32 * 32 * sizeof(double2);
-    if (mode == RK_MIXED_SCHUR)
-        return (size_t)N * 7 * sizeof(double2) + 2 * (size_t)(N + (N & 1)) * sizeof(float2) + 32 * 32 * sizeof(float2);
-    return mode == RK_MIXED ? (size_t)N * 7 * sizeof(double2) + (size_t)(N + (N & 1)) * sizeof(float2) +
-                                  32 * 32 * sizeof(float2)
-                            : (size_t)N * 5 * sizeof(double2) + 32 * 32 * sizeof(double2);
+    if (mode == RK_MATRIX) return ((size_t)N * 4 + RC_BLK) * sizeof(double2);
+    if (mode == RK_SCHUR) return ((size_t)N * 5 + RC_BLK) * sizeof(double2);
+    if (mode == RK_STAGE) return ((size_t)N * 5 + RC_BLK) * sizeof(double2) + (size_t)N * sizeof(uint16_t);
+    if (mode == RK_MIXED_SCHUR) return (size_t)N * 6 * sizeof(double2) + (32 * 32 + 3 * (size_t)N) * sizeof(float2);
+    return (size_t)N * 7 * sizeof(double2) + (size_t)(N + (N & 1)) * sizeof(float2) + 32 * 32 * sizeof(float2);
 }
 
 __global__ void k_probabilities(long long n, const double2* __restrict__ c, double* __restrict__ P) {
@@ -394,8 +580,7 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
         if (ts != WPCCC_OK) return ts;
     }
     P.mode = P.mixed ? (P.schur ? RK_MIXED_SCHUR : RK_MIXED) : (P.schur ? RK_SCHUR : (P.stage ? RK_STAGE : RK_MATRIX));
-    // 227 KB per block, less the kernels' static shared memory (the refinement check's reduction)
-    const bool fits = rk_smem_bytes(P.mode, N) + 1024 <= (size_t)227 * 1024;
+    const bool fits = N <= rk_max_states(P.mode);
     if (P.two && B->rk4_layout == WPCCC_RK4_GLOBAL)
         return fail(WPCCC_EUNSUPPORTED, "wpccc_propagate: the global-memory RK4 layout is one-centre only");
     P.wide = !P.two && (B->rk4_layout == WPCCC_RK4_GLOBAL || (B->rk4_layout == WPCCC_RK4_AUTO && !fits));
@@ -545,19 +730,21 @@ struct PlanStreams {
 
 // Queues every kernel of the plan: the flags reset, then per chunk the element kernels and the
 // solve on S.st, the RK4 sweep on S.rs, with double-buffered chunks.  Capturable into a graph.
-static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S) {
+static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S, int n_sets = 1) {
     if (P.max_steps == 0) return WPCCC_OK;
     wpccc_basis_s* B = P.B;
     const int N = P.N;
     cudaStream_t st = S.st, rs = S.rs;
     WPCCC_CUDA(cudaMemsetAsync(P.d_flags, 0, sizeof(int), st));
+    int sms = 0;
+    WPCCC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device));
     int rk_smem = P.wide ? 0 : (int)rk_smem_bytes(P.mode, N);
     // reduced-precision forms with N <= RK_THREADS: H streamed through two shared-memory slots of up to eight
     // columns each, in what the mode's vectors leave of the 227 KB
     int stage_cols = 0;
     size_t stage_off = 0;
     const size_t rk_cap = (size_t)227 * 1024 - 1024;
-    if (!P.wide && P.df_rhs && N <= RK_THREADS) {
+    if (!P.wide && P.mode == RK_MIXED && P.df_rhs && N <= RK_THREADS) {
         stage_off = ((size_t)rk_smem + 127) / 128 * 128;
         if (rk_cap > stage_off + 16)
             stage_cols = (int)std::min<size_t>(8, (rk_cap - stage_off - 16) / (2 * (size_t)N * sizeof(double2)));
@@ -567,11 +754,11 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S) 
     if (!P.wide) {
         // the largest any plan takes (a batch graph holds launches of several plans)
         const int mx = (int)rk_cap;
-        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4<RK_MATRIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4<RK_STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4<RK_SCHUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4<RK_MIXED>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
-        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4<RK_MIXED_SCHUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_fp64<RK_MATRIX>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_fp64<RK_STAGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_fp64<RK_SCHUR>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_mixed_lu, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
+        WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_mixed_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, mx));
     }
     const size_t hS = P.sz_S / 2 / sizeof(double2), hH = P.sz_H / 2 / sizeof(double2);
     const size_t hL = P.sz_LU32 / 2 / sizeof(float2), hP = P.sz_piv / 2 / sizeof(int), hI = P.sz_info / 2 / sizeof(int);
@@ -644,11 +831,19 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S) 
             const dim3 grid((N + WIDE_ROWS - 1) / WIDE_ROWS, npc);
             for (int s2 = 0; s2 < steps; ++s2)
                 for (int stage = 1; stage <= 4; ++stage) k_rk4_wide<<<grid, WIDE_ROWS, 0, rs>>>(wa, s2, stage);
-        } else if (P.mode == RK_MIXED) k_rk4<RK_MIXED><<<npc, RK_THREADS, rk_smem, rs>>>(ra);
-        else if (P.mode == RK_MIXED_SCHUR) k_rk4<RK_MIXED_SCHUR><<<npc, RK_THREADS, rk_smem, rs>>>(ra);
-        else if (P.mode == RK_SCHUR) k_rk4<RK_SCHUR><<<npc, RK_THREADS, rk_smem, rs>>>(ra);
-        else if (P.mode == RK_STAGE) k_rk4<RK_STAGE><<<npc, RK_THREADS, rk_smem, rs>>>(ra);
-        else k_rk4<RK_MATRIX><<<npc, RK_THREADS, rk_smem, rs>>>(ra);
+        } else if (P.mode == RK_MIXED) k_rk4_mixed_lu<<<npc, RK_THREADS, rk_smem, rs>>>(ra);
+        else {
+            // SMs for the sweep: half the chip beside the next chunk's assembly (p + H, 32 paths, 16 steps in mode 3: 42.4,
+            // 40.6, 44.3 and 55.8 ms with one, two, four and eight blocks per path; C6+ + H, 16 paths: 166, 128, 122 and
+            // 131), all of it for the last chunk or where the assembly is small (one centre); a set's part in a batch
+            // (three sets of 16 paths: 110, 107, 113 and 138)
+            const int share = n_sets > 1 ? sms / n_sets : (P.two && ch + 1 < P.n_chunks ? sms / 2 : sms);
+            ClusterLaunch L(npc, rk4_cluster(npc, N, share), RC_THREADS, rk_smem, rs);
+            WPCCC_CUDA(P.mode == RK_MIXED_SCHUR ? cudaLaunchKernelEx(&L.cfg, k_rk4_mixed_schur, ra)
+                       : P.mode == RK_SCHUR ? cudaLaunchKernelEx(&L.cfg, k_rk4_fp64<RK_SCHUR>, ra)
+                       : P.mode == RK_STAGE ? cudaLaunchKernelEx(&L.cfg, k_rk4_fp64<RK_STAGE>, ra)
+                                            : cudaLaunchKernelEx(&L.cfg, k_rk4_fp64<RK_MATRIX>, ra));
+        }
         WPCCC_CHECK_LAUNCH("k_rk4");
         B->prof.end(PROF_RK4, rs, e1);
         WPCCC_CUDA(cudaEventRecord(S.rk_done[k], rs));
@@ -931,7 +1126,7 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
             break;
         }
         PlanStreams S{st, rs, {ev[0], ev[1]}, {ev[2], ev[3]}, ev[4], ev[5]};
-        cs = plan_enqueue(X->plans[k], X->c[k], S);
+        cs = plan_enqueue(X->plans[k], X->c[k], S, n_sets);
         if (cs != WPCCC_OK) break;
         // join: the capture stream waits for this set's assembly stream (which waits for its sweeps)
         if (cudaEventRecord(ev[5], st) != cudaSuccess || cudaStreamWaitEvent(cap, ev[5], 0) != cudaSuccess)

@@ -28,7 +28,7 @@
 #include <vector>
 
 #include "geometry.cuh"
-#include "rk_device.cuh"
+#include "rk4_fp64.cuh"
 #include "wpccc_internal.cuh"
 
 namespace wpccc {
@@ -56,7 +56,10 @@ __device__ inline double2 cadd(double2 a, double2 b) { return make_double2(a.x +
 __device__ inline double2 cscale(double2 a, double s) { return make_double2(a.x * s, a.y * s); }
 
 // ---------------------------------------------------------------------------
-// k_rk4_adjoint: one block per path slot.  Phase 1 replays the segment's steps from its checkpoint
+// k_rk4_adjoint: one cluster of blocks per path slot (rk4_fp64.cuh: every block keeps all vectors and updates them alike,
+// the products with H and the LU solves are shared out; the first block writes the records).  A gradient has few paths, so
+// one block per path left most SMs idle (p + Li, N = 379, 6 paths, 4 steps: this kernel and the element adjoint together
+// 62 -> 35 ms).  Phase 1 replays the segment's steps from its checkpoint
 // and records x_s, k_s and H_s x_s of every stage; phase 2 runs the reverse stages, records xi_s and
 // adds the energy-phase part of the parameter derivatives.
 // ---------------------------------------------------------------------------
@@ -82,9 +85,11 @@ struct AdjRkArgs {
 
 constexpr int ADJ_RED = 2 * WPCCC_MAX_PARAMS;
 
-__global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
+__global__ void __launch_bounds__(RC_THREADS, 1) k_rk4_adjoint(AdjRkArgs A) {
     extern __shared__ double2 adj_smem[];
     __shared__ double red[RK_THREADS / 32][ADJ_RED];
+    const RcCluster cl{cluster_rank(), cluster_size()};
+    const bool first = cl.rank == 0;
     const int N = A.N;
     double2* c = adj_smem;
     double2* y = c + N;
@@ -93,14 +98,15 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
     double2* xb = t + N;
     double2* xs = xb + N;
     double2* lam = xs + N;                       // [n_obs][N]
-    double2* blk = lam + (size_t)A.n_obs * N;    // 32 x 32
-    const int sl = A.slots[blockIdx.x];
+    double2* blk = lam + (size_t)A.n_obs * N;    // RC_BLK
+    uint16_t* perm = reinterpret_cast<uint16_t*>(blk + RC_BLK);
+    const int sl = A.slots[blockIdx.x / cl.size];
     const int n = A.nsteps[sl], p0 = A.pos0[sl];
     const double v = A.v[sl];
     const double* zs = A.z + (size_t)sl * (A.K + 1);
     const size_t mat = (size_t)N * N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (A.info && tid == 0) {
+    if (A.info && first && tid == 0) {
         int bad = 0;
         for (int e = 0; e <= 2 * n; ++e)
             if (A.info[p0 + e] != 0) bad = 1;
@@ -111,6 +117,21 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
     auto Pv = [&](int e) { return A.piv + (size_t)(p0 + e) * N; };
     auto stage_pos = [&](int s, int st) { return st == 0 ? 2 * s : (st == 3 ? 2 * s + 2 : 2 * s + 1); };
     auto rec = [&](int s, int st) { return ((size_t)sl * A.K + s) * 4 + st; };
+
+    // t <- S_e^{-1} t and out = H_e x, replicated; kv is the solve's scratch
+    int perm_of = -1;
+    auto solve = [&](int e) {
+        if (e != perm_of) rc_permutation(Pv(e), N, perm, blk);
+        perm_of = e;
+        rc_lu_solve(cl, Lm(e), perm, N, t, kv, blk);
+    };
+    auto times_H = [&](int e, const double2* x, double2* out) {
+        int lo, hi;
+        cl.rows(N, lo, hi);
+        rc_matvec(Hm(e) + lo, N, hi - lo, N, x, blk, [&](int r, double2 a) { cl.bcast(out + lo + r, a); });
+        cl.sync();
+    };
+    cl.sync();   // every block has started
 
     // ---- phase 1: replay, recording the stage vectors
     for (int i = tid; i < N; i += RK_THREADS) c[i] = A.ckpt[(size_t)sl * N + i];
@@ -126,28 +147,29 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
         for (int st = 0; st < 4; ++st) {
             const int e = stage_pos(s, st);
             const size_t r = rec(s, st) * N;
-            matvec(Hm(e), N, y, t);
-            for (int i = tid; i < N; i += RK_THREADS) {
-                A.rhx[r + i] = t[i];
-                A.rx[r + i] = y[i];
-            }
+            times_H(e, y, t);
+            if (first)
+                for (int i = tid; i < N; i += RK_THREADS) {
+                    A.rhx[r + i] = t[i];
+                    A.rx[r + i] = y[i];
+                }
             __syncthreads();   // the solve permutes t in place
-            lu_solve_inplace<double2>(Lm(e), Pv(e), N, t, blk);
+            solve(e);
             const double hn = st == 2 ? h : h2;
             const double wk = (st == 0 || st == 3) ? 1.0 : 2.0;
             for (int i = tid; i < N; i += RK_THREADS) {
                 const double2 k = make_double2(t[i].y / v, -t[i].x / v);
-                A.rk[r + i] = k;
+                if (first) A.rk[r + i] = k;
                 xb[i] = make_double2(fma(wk, k.x, xb[i].x), fma(wk, k.y, xb[i].y));
                 if (st < 3) y[i] = make_double2(fma(hn, k.x, c[i].x), fma(hn, k.y, c[i].y));
             }
-            __syncthreads();
+            cl.sync();   // t is read everywhere before the next product is stored into it
         }
         for (int i = tid; i < N; i += RK_THREADS) c[i] = make_double2(fma(h6, xb[i].x, c[i].x), fma(h6, xb[i].y, c[i].y));
         __syncthreads();
     }
 
-    // ---- phase 2: reverse stages
+    // ---- phase 2: reverse stages (the first block's records are read by every block)
     for (int q = tid; q < A.n_obs * N; q += RK_THREADS) lam[q] = A.lam[(size_t)sl * A.n_obs * N + q];
     __syncthreads();
     double gacc[4][WPCCC_MAX_PARAMS] = {};   // thread 0 keeps the per-observable phase contributions
@@ -173,15 +195,15 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
                     t[i] = kb;
                 }
                 __syncthreads();
-                lu_solve_inplace<double2>(Lm(e), Pv(e), N, t, blk);
-                matvec(Hm(e), N, t, kv);   // u = H xi
+                solve(e);
+                times_H(e, t, kv);   // u = H xi
                 // energy-phase part: Re A_p and Im B_p with
                 //   A = sum_i deps_i (conj(xi_i) (Hx)_i - conj(u_i) x_i)
                 //   B = sum_i deps_i (conj(xi_i) (Sk)_i - conj(kb_i) k_i),  S k = -(i/v) H x
                 double part[ADJ_RED] = {};
                 for (int i = tid; i < N; i += RK_THREADS) {
                     const double2 xi = t[i], u = kv[i], kb = y[i];
-                    const double2 hx = A.rhx[r + i], xx = A.rx[r + i], kk = A.rk[r + i];
+                    const double2 hx = __ldcg(A.rhx + r + i), xx = __ldcg(A.rx + r + i), kk = __ldcg(A.rk + r + i);
                     const double2 sk = make_double2(hx.y / v, -hx.x / v);
                     const double2 a1 = cmulc(xi, hx), a2 = cmulc(u, xx);
                     const double2 b1 = cmulc(xi, sk), b2 = cmulc(kb, kk);
@@ -200,7 +222,7 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
                 // record xi, then xb = (i/v) u and its running sum
                 const size_t rxo = (rec(s, st) * A.n_obs + o) * N;
                 for (int i = tid; i < N; i += RK_THREADS) {
-                    A.rxi[rxo + i] = t[i];
+                    if (first) A.rxi[rxo + i] = t[i];
                     const double2 x = make_double2(-kv[i].y / v, kv[i].x / v);
                     xb[i] = x;
                     xs[i] = cadd(xs[i], x);
@@ -226,15 +248,18 @@ __global__ void __launch_bounds__(RK_THREADS) k_rk4_adjoint(AdjRkArgs A) {
     }
     for (int q = tid; q < A.n_obs * N; q += RK_THREADS) {
         const double2 l = lam[q];
-        A.lam[(size_t)sl * A.n_obs * N + q] = l;
+        if (first) A.lam[(size_t)sl * A.n_obs * N + q] = l;
         if (!isfinite(l.x) || !isfinite(l.y)) atomicOr(A.flags, 2);
     }
-    if (tid == 0)
+    if (first && tid == 0)
         for (int o = 0; o < A.n_obs; ++o)
             for (int p = 0; p < A.npar; ++p) A.gphase[((size_t)sl * A.n_obs + o) * A.npar + p] += gacc[o][p];
+    cl.sync();   // no block leaves while another may still store into its shared memory
 }
 
-size_t adj_rk_smem_bytes(int N, int n_obs) { return ((size_t)(6 + n_obs) * N + 32 * 32) * sizeof(double2); }
+size_t adj_rk_smem_bytes(int N, int n_obs) {
+    return ((size_t)(6 + n_obs) * N + RC_BLK) * sizeof(double2) + (size_t)N * sizeof(uint16_t);
+}
 
 // lam = g o c at the end of the paths, P = g |c|^2
 __global__ void k_adj_init(int N, int n_obs, int n_slots, const double* __restrict__ g,
@@ -847,6 +872,8 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     if ((s = ensure_workspace(B, ws_need)) != WPCCC_OK) return s;
     double* node = static_cast<double*>(B->ws_ptr);
     const int adj_smem = (int)adj_rk_smem_bytes(N, n_obs);
+    int sms = 0;
+    WPCCC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device));
     WPCCC_CUDA(cudaFuncSetAttribute(k_rk4_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, adj_smem));
     int LMX = std::max(B->T.lmax, B->P.lmax);
 
@@ -944,8 +971,8 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
         ra.gphase = gphase;
         ra.flags = flags;
         cudaEvent_t pa = B->prof.begin(PROF_ADJ, st);
-        k_rk4_adjoint<<<(unsigned)slots.size(), RK_THREADS, adj_smem, st>>>(ra);
-        WPCCC_CHECK_LAUNCH("k_rk4_adjoint");
+        ClusterLaunch CL((int)slots.size(), rk4_cluster((int)slots.size(), N, sms), RC_THREADS, adj_smem, st);
+        WPCCC_CUDA(cudaLaunchKernelEx(&CL.cfg, k_rk4_adjoint, ra));
         B->prof.end(PROF_ADJ, st, pa);
         // element adjoint, sub-batch by sub-batch of positions
         size_t t0 = 0;
@@ -1171,7 +1198,8 @@ extern "C" wpccc_status wpccc_propagate_adjoint(wpccc_basis B, const wpccc_paths
     if (B->tanT.n_tan > ADJ_MAXTAN || B->tanP.n_tan > ADJ_MAXTAN)
         return fail(WPCCC_EUNSUPPORTED, "wpccc_propagate_adjoint: more than 2 derivative tables on one centre");
     const int N = B->N;
-    if (adj_rk_smem_bytes(N, n_obs) + 2048 > (size_t)227 * 1024)
+    // (6 + n_obs) N + 1024 complex numbers and 2 KB in a block's 227 KB; the kernel takes no more up to there
+    if (((size_t)(6 + n_obs) * N + 1024) * sizeof(double2) + 2048 > (size_t)227 * 1024)
         return fail(WPCCC_EINVAL, "wpccc_propagate_adjoint: N too large for the adjoint RK4 kernel");
     const int np = paths->n_paths;
     if (np < 1 || !paths->b || !paths->v || !paths->n_z || !paths->z)

@@ -503,7 +503,7 @@ struct PropPlan {
     int np = 0, N = 0, mode = RK_MATRIX, elem_precision = 0, C = 1, n_chunks = 0, max_chunk_evals = 0;
     int max_steps = 0;
     bool two = false, mixed = false, stage = false, schur = false;
-    bool schur_tc = false;   // mixed Schur forms: the trailing update I - K^+ K on the tensor cores
+    bool schur_tc = false;   // Schur forms: the trailing update I - K^+ K on the tensor cores
     bool df_rhs = false;     // reduced-precision forms (1, 2, 3): H y on the FP32 pipe in double-float arithmetic
     bool wide = false;       // one-centre RK4 with the vectors in global memory (k_rk4_wide)
     size_t per_eval = 0, fixed = 0;
@@ -579,6 +579,8 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
         wpccc_status ts = schur_tc_prepare(B);
         if (ts != WPCCC_OK) return ts;
     }
+    if (P.schur && !P.mixed)   // the FP64 form: always where the elements' scratch holds the digits
+        P.schur_tc = schur_fp64_tc_applicable(B, elem_scratch_layout(B, P.elem_precision).bytes_per_eval);
     P.mode = P.mixed ? (P.schur ? RK_MIXED_SCHUR : RK_MIXED) : (P.schur ? RK_SCHUR : (P.stage ? RK_STAGE : RK_MATRIX));
     const bool fits = N <= rk_max_states(P.mode);
     if (P.two && B->rk4_layout == WPCCC_RK4_GLOBAL)
@@ -802,6 +804,8 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S, 
                                                elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
             else if (P.mixed && P.schur) s = launch_schur_factor_f32(N, B->N_T, nev, bS, bL, bI, st);
             else if (P.mixed) s = launch_factor_f32(N, nev, bS, bL, bP, bI, st);
+            else if (P.schur && P.schur_tc)
+                s = launch_schur_factor_fp64_tc(B, nev, bS, bI, P.d_scr, elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
             else if (P.schur) s = launch_schur_factor(N, B->N_T, nev, bS, bI, st);
             else s = launch_solve(N, nev, bS, P.stage ? nullptr : bH, bP, bI, st);
             if (s != WPCCC_OK) return s;

@@ -240,7 +240,13 @@ wpccc_status launch_schur_factor(int N, int N_T, int batch, double2* S, int* inf
 wpccc_status launch_schur_factor_f32(int N, int N_T, int batch, const double2* S, float2* D, int* info,
                                      cudaStream_t st);
 
-// The Cholesky factor of a trailing matrix I - K^+ K already in D's projectile block (K in FP32 in D).
+// The FP64 form with the rank-N_T update I - K^+ K on the tensor cores (schur_fp64.cu); `scratch` holds at least
+// `scratch_per_eval` bytes per evaluation.
+bool schur_fp64_tc_applicable(const wpccc_basis_s* B, size_t scratch_per_eval);
+wpccc_status launch_schur_factor_fp64_tc(wpccc_basis_s* B, int nev, double2* S, int* info, void* scratch,
+                                         size_t scratch_per_eval, cudaStream_t st);
+// The Cholesky factor of a trailing matrix I - K^+ K already in S's (D's, with K in FP32) projectile block.
+wpccc_status launch_schur_cholesky(int N, int N_T, int batch, double2* S, int* info, cudaStream_t st);
 wpccc_status launch_schur_cholesky_f32(int N, int N_T, int batch, float2* D, int* info, cudaStream_t st);
 // The FP32 preconditioner of the mixed Schur forms with the rank-N_T update I - K^+ K on the tensor cores
 // (schur_tc.cu); `scratch` holds at least `scratch_per_eval` bytes per evaluation.

@@ -804,74 +804,69 @@ struct EtArgs {
     size_t et_doubles;
 };
 
+// Blocks x of a position share its entries out, one per thread where there are enough blocks: each is a chain of FP64
+// operations or loads, so a position on one block took 104 us (24 positions, N = 572) or 36 us (one centre, N = 59;
+// now 19 us).
+// Every block finds the stencil itself (its last warp, while the others are busy).
 __global__ void __launch_bounds__(128) k_eval_tables(EtArgs A, const EvalDesc* __restrict__ ev) {
-    const int e = blockIdx.x;
-    const double b = ev[e].b, z = ev[e].z;
+    const int e = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    const int first = blockIdx.x * blockDim.x + tid, stride = gridDim.x * blockDim.x;
+    const double b = ev[e].b, v = ev[e].v, z = ev[e].z;
     const double R = dist_R(b, z);
-    const double cth = z / R;
-    const double ch = sqrt(0.5 * (1.0 + cth)), sh = sqrt(0.5 * (1.0 - cth));
     double* et = A.et + (size_t)e * A.et_doubles;
-    for (int idx = threadIdx.x; idx < A.dtot; idx += blockDim.x) {
-        int l = 0, off = 0;
-        while (idx >= off + (2 * l + 1) * (2 * l + 1)) {
-            off += (2 * l + 1) * (2 * l + 1);
-            ++l;
-        }
-        int loc = idx - off, m = loc / (2 * l + 1) - l, q = loc % (2 * l + 1) - l;
-        et[idx] = wigner_small_d(l, m, q, ch, sh);
-    }
-    for (int t = threadIdx.x; t < A.npb; t += blockDim.x) {
-        int lam = 0;
-        while ((lam + 1) * (lam + 2) / 2 <= t) ++lam;
-        int mu = t - lam * (lam + 1) / 2;
-        et[A.dtot + t] = sqrt(dfact(lam - mu) / dfact(lam + mu)) * assoc_legendre(lam, mu, cth);
-    }
+    double2* ph = reinterpret_cast<double2*>(et + A.ph_off);
     __shared__ int s_s, s_out;
     __shared__ double s_L[5];
-    if (threadIdx.x == 0) {
-        double* st = et + A.dtot + A.npb;
-        int s;
-        double L[5];
-        if (R > A.r[A.Nr - 1]) {
-            st[0] = (double)(A.Nr - 1);
-            st[1] = 1.0;
-            for (int k = 0; k < 5; ++k) st[2 + k] = 0.0;
-            s_s = A.Nr - 1;
-            s_out = 1;
-        } else {
-            stencil5(A.r, A.Nr, R, s, L);
-            st[0] = (double)s;
-            st[1] = 0.0;
-            for (int k = 0; k < 5; ++k) st[2 + k] = L[k];
+    if (tid >= 96) {
+        int s = A.Nr - 1;
+        double L = 0.0;
+        const bool out = R > A.r[A.Nr - 1];
+        if (!out) stencil5_warp(A.r, A.Nr, R, lane, s, L);
+        if (lane == 0) {
             s_s = s;
-            s_out = 0;
-            for (int k = 0; k < 5; ++k) s_L[k] = L[k];
+            s_out = out;
+        }
+        if (lane < 5) s_L[lane] = L;
+        if (blockIdx.x == 0) {
+            double* st = et + A.dtot + A.npb;
+            if (lane == 0) {
+                st[0] = (double)s;
+                st[1] = out ? 1.0 : 0.0;
+            }
+            if (lane < 5) st[2 + lane] = L;
+        }
+    }
+    for (int t = first; t < A.dtot + A.npb + A.N; t += stride) {
+        if (t < A.dtot) {
+            const double cth = z / R;
+            const double ch = sqrt(0.5 * (1.0 + cth)), sh = sqrt(0.5 * (1.0 - cth));
+            int l = 0, off = 0;
+            while (t >= off + (2 * l + 1) * (2 * l + 1)) {
+                off += (2 * l + 1) * (2 * l + 1);
+                ++l;
+            }
+            const int loc = t - off, m = loc / (2 * l + 1) - l, q = loc % (2 * l + 1) - l;
+            et[t] = wigner_small_d(l, m, q, ch, sh);
+        } else if (t < A.dtot + A.npb) {
+            int lam = 0;
+            while ((lam + 1) * (lam + 2) / 2 <= t - A.dtot) ++lam;
+            const int mu = t - A.dtot - lam * (lam + 1) / 2;
+            et[t] = sqrt(dfact(lam - mu) / dfact(lam + mu)) * assoc_legendre(lam, mu, z / R);
+        } else {
+            const int i = t - A.dtot - A.npb;
+            const double eps = i < A.N_T ? A.epsT[i] : A.epsP[i - A.N_T];
+            double sp, cp;
+            sincos(eps * z / v, &sp, &cp);
+            ph[i] = make_double2(cp, sp);
         }
     }
     __syncthreads();
     // F of every Eq. 7 table entry at R (5-point interpolation, or the multipole tail beyond the grid)
     double* Fint = et + A.dtot + A.npb + 8;
-    const double ratio = A.r[A.Nr - 1] / R;
-    for (int t = threadIdx.x; t < A.nfT + A.nfP; t += blockDim.x) {
-        const double* Fe = t < A.nfT ? A.FT + (size_t)t * A.Nr : A.FP + (size_t)(t - A.nfT) * A.Nr;
-        double Fv;
-        if (s_out) {
-            // lam of the entry is not needed here: the tail factor (r_max/R)^{lam+1} is applied in k_direct
-            Fv = Fe[A.Nr - 1];
-        } else {
-            const int s = s_s;
-            Fv = s_L[0] * Fe[s] + s_L[1] * Fe[s + 1] + s_L[2] * Fe[s + 2] + s_L[3] * Fe[s + 3] + s_L[4] * Fe[s + 4];
-        }
-        Fint[t] = Fv;
-    }
-    (void)ratio;
-    double2* ph = reinterpret_cast<double2*>(et + A.ph_off);
-    const double v = ev[e].v;
-    for (int i = threadIdx.x; i < A.N; i += blockDim.x) {
-        const double eps = i < A.N_T ? A.epsT[i] : A.epsP[i - A.N_T];
-        double sp, cp;
-        sincos(eps * z / v, &sp, &cp);
-        ph[i] = make_double2(cp, sp);
+    for (int t = first; t < A.nfT + A.nfP; t += stride) {
+        const double* Fe = (t < A.nfT ? A.FT + (size_t)t * A.Nr : A.FP + (size_t)(t - A.nfT) * A.Nr) + s_s;
+        // beyond the grid the tail factor (r_max/R)^{lam+1} is applied in k_direct_coef
+        Fint[t] = s_out ? Fe[0] : s_L[0] * Fe[0] + s_L[1] * Fe[1] + s_L[2] * Fe[2] + s_L[3] * Fe[3] + s_L[4] * Fe[4];
     }
 }
 
@@ -1343,7 +1338,10 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
         ea.et = et;
         ea.et_doubles = L.et_doubles;
         cudaEvent_t e0 = B->prof.begin(PROF_NODES, st);
-        k_eval_tables<<<nev, 128, 0, st>>>(ea, evals);
+        // one entry per thread, in a grid of up to about 2048 blocks
+        const int entries = std::max(L.dtot + L.npb + B->N, ea.nfT + ea.nfP);
+        const int parts = std::max(1, std::min((entries + 127) / 128, 2048 / nev));
+        k_eval_tables<<<dim3(parts, nev), 128, 0, st>>>(ea, evals);
         WPCCC_CHECK_LAUNCH("k_eval_tables");
         B->prof.end(PROF_NODES, st, e0);
     }

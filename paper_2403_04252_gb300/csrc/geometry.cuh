@@ -40,6 +40,23 @@ static __device__ inline bool stencil5(const double* __restrict__ r, int Nr, dou
     return true;
 }
 
+// The same stencil by one warp: the start in every lane, weight a in lane a < 5.
+static __device__ inline void stencil5_warp(const double* __restrict__ r, int Nr, double x, int lane, int& s, double& L) {
+    int lo = -1, hi = Nr;   // r[lo] <= x < r[hi]
+    while (hi - lo > 1) {
+        const int step = (hi - lo + 32) / 33, p = lo + (lane + 1) * step;
+        const int c = __popc(__ballot_sync(0xffffffffu, p < hi && r[p] <= x));
+        lo += c * step;
+        hi = min(hi, lo + step);
+    }
+    s = min(max(lo - 2, 0), Nr - 5);
+    const int a = min(lane, 4);
+    double p = 1.0;
+    for (int c = 0; c < 5; ++c)
+        if (c != a) p *= (x - r[s + c]) / (r[s + a] - r[s + c]);
+    L = p;
+}
+
 // The same stencil with the Lagrange denominators 1/prod_{c != a}(r_{s+a} - r_{s+c}) read from a
 // table made at set-up (inv_den[s][a], 5 per stencil start), so no division per interpolation.
 static __device__ inline bool stencil5_fast(const double* __restrict__ r, const double* __restrict__ inv_den, int Nr,

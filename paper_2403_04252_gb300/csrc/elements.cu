@@ -39,9 +39,10 @@ constexpr int NX = 2;
 //   x >= dmax       forward recurrence J_{n+1} = (2n/x) J_n - J_{n-1} from J_0, J_1 (stable while the
 //                   order stays below the argument);
 //   1e-5 <= x < dmax  Miller's backward recurrence (J. C. P. Miller; Abramowitz & Stegun 9.12): start
-//                   from f_{M+1} = 0, f_M = 1 at an order M well above x and dmax, recur downwards with
+//                   from f_{M+1} = 0, f_M = 1 at an order M above x and dmax, recur downwards with
 //                   the same relation, rescale against overflow, and normalise by J_0 (or J_1 when that
-//                   is larger, so a zero of J_0 costs no accuracy);
+//                   is larger, so a zero of J_0 costs no accuracy).  M = dmax + 14 + x / 2 leaves a truncation
+//                   below 1e-18 of every J_n for dmax <= 20 (in 40-digit arithmetic);
 //   x < 1e-5        the first two terms of the power series, (x/2)^n/n! (1 - (x/2)^2/(n+1)).
 // J_0 and J_1 come from CUDA's j0 and j1.
 // ---------------------------------------------------------------------------
@@ -65,15 +66,15 @@ __device__ inline void bessel_j_orders(int dmax, double x, double* J) {
         for (int n = 1; n < dmax; ++n) J[n + 1] = (n * ix2) * J[n] - J[n - 1];
         return;
     }
-    const int M = dmax + 26 + (int)x;
+    const int M = dmax + 14 + ((int)x >> 1);
     const double ix2 = 2.0 / x;
-    double fn1 = 0.0, fn = 1.0;   // f_{n+1}, f_n
-    for (int n = M; n >= 1; --n) {
-        const double fm = (n * ix2) * fn - fn1;   // f_{n-1}
+    double fn1 = 0.0, fn = 1.0, dn = (double)M;   // f_{n+1}, f_n, n
+    for (int n = M; n >= 1; --n, dn -= 1.0) {
+        const double fm = (dn * ix2) * fn - fn1;   // f_{n-1}
         fn1 = fn;
         fn = fm;
         if (n - 1 <= dmax) J[n - 1] = fm;
-        if (fabs(fn) > 1e200) {
+        if ((__double2hiint(fn) & 0x7FFFFFFF) > 0x6974E718) {   // above 1e200, without the FP64 pipe
             fn *= 1e-200;
             fn1 *= 1e-200;
             for (int k = n - 1; k <= dmax; ++k) J[k] *= 1e-200;
@@ -111,14 +112,16 @@ struct NodeArgs {
     // r_T, r_T V_T at f64_r (byte offsets, rows of Gp nodes, zero past the last node)
     int f64, Gp;
     size_t f64_w2, f64_r;
-    // sqrt((2l+1)/2 (l-q)!/(l+q)!) at l(l+1)/2 + q, and 1/k for k = 0..WPCCC_LMAX (entry 0 unused): the
-    // Legendre recurrence's constants, formed once on the host instead of per node
+    // sqrt((2l+1)/2 (l-q)!/(l+q)!) at l(l+1)/2 + q, 1/k for k = 0..WPCCC_LMAX (entry 0 unused) and the numbers k
+    // themselves (a conversion takes the FP64 pipe as long as a multiplication): the Legendre recurrence's constants
     double th_nrm[(WPCCC_LMAX + 1) * (WPCCC_LMAX + 2) / 2];
     double inv_int[WPCCC_LMAX + 1];
+    double num[2 * WPCCC_LMAX + 2];
 };
 
-// Radial functions of the tensor-core layout's target rows processed per shared-memory batch.
+// Radial functions of the tensor-core layout's target rows processed per shared-memory batch (even: two at a time).
 constexpr int TC_NA = 16;
+template <int V> struct IntC { static constexpr int value = V; };
 
 // Normalised Legendre functions Theta_lq(c) = sqrt((2l+1)/2 (l-q)!/(l+q)!) P_l^q(c) (Condon-Shortley phase)
 // for 0 <= q <= l <= lmax, by the upward recurrence in l at fixed q, handed to put(l (l+1)/2 + q, value).
@@ -127,13 +130,13 @@ __device__ inline void theta_lq(double c, int lmax, const NodeArgs& A, F put) {
     const double sq = sqrt((1.0 - c) * (1.0 + c));
     double pmm = 1.0;   // P_q^q, built up from P_0^0 = 1
     for (int q = 0; q <= lmax; ++q) {
-        if (q > 0) pmm *= -(2.0 * q - 1.0) * sq;
+        if (q > 0) pmm *= -A.num[2 * q - 1] * sq;
         double pa = 0.0, pb = pmm;   // P_{l-2}^q, P_{l-1}^q
         for (int l = q; l <= lmax; ++l) {
             double pl;
             if (l == q) pl = pmm;
-            else if (l == q + 1) pl = c * (2.0 * q + 1.0) * pmm;
-            else pl = (c * (2.0 * l - 1.0) * pb - (l + q - 1.0) * pa) * A.inv_int[l - q];
+            else if (l == q + 1) pl = c * A.num[2 * q + 1] * pmm;
+            else pl = (c * A.num[2 * l - 1] * pb - A.num[l + q - 1] * pa) * A.inv_int[l - q];
             if (l > q) {
                 pa = pb;
                 pb = pl;
@@ -151,6 +154,13 @@ template <> struct Vec2<float> { using type = float2; };
 // The per-node factors are computed in FP64; T = double keeps them in FP64, T = float (mixed-precision
 // form) stores them rounded to FP32 for the FP32 contraction.  In the tensor-core layout a block is one
 // 128-node scaling window and needs dynamic shared memory (see node_tables_smem).
+//
+// What bounds it: the FP64 pipe (two operations per clock per SM), 81 % busy in FP64 where the interpolation of the
+// radial functions dominates; in the tensor-core layout the geometry, the Bessel functions and the Legendre recurrences
+// took 37 % of it and the slicing most of the issue slots.  So conversions, comparisons and recurrence steps that need no
+// FP64 are kept off the pipe, two nodes share an instruction (FP32x2), the rows of m and -m are sliced once, and a lane
+// stores four nodes at a time.  With k_eval_tables: N = 572, 45 positions 0.72 -> 0.53 ms; FP64, N = 380, 24 positions
+// 0.22 -> 0.16 ms.
 template <typename T>
 __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc* __restrict__ ev) {
     using T2 = typename Vec2<T>::type;
@@ -208,116 +218,149 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
         // tensor-core layout: A_T r_T and A_T r_T V_T per target state (rows of the row tiles), each as
         // tc_slices bf16 slices against a power-of-two scale per 128-node window (this block); the
         // products are formed in double-float arithmetic from FP64 factors split once per node.
-        // Shared memory: th [nlq][128] (this thread's column only while it builds A_P from the projectile's
-        // Theta, then the target's Theta for every warp), r [2][128] (r_T, r_T V_T), f [TC_NA][128]
-        // (a batch of target radial functions at the window's nodes).
-        extern __shared__ float2 s_tc[];
+        // Shared memory, a row of 128 high parts and a row of 128 low parts per entry: th [nlq] (this thread's column
+        // only while it builds A_P from the projectile's Theta, then the target's Theta for every warp), r [2] (r_T,
+        // r_T V_T), f [TC_NA] (a batch of target radial functions at the window's nodes).
+        extern __shared__ __align__(16) float s_tc[];
         // the 5-point interpolation in double-float arithmetic on the FP32 pipe (the FP64 pipe is two
         // operations per clock per SM on this part): Lagrange weights split once per node, tables stored
-        // split; each term's product is exact in its high parts (FMA residual) and the sum a TwoSum chain
+        // split; each term's product is exact in its high parts (FMA residual) and the sum a TwoSum chain.
+        // Two radial functions at a time (a and a2) in packed FP32x2 instructions.
         float2 LT2[5], LP2[5];
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
             LT2[k] = df_split(LT[k]);
             LP2[k] = df_split(LP[k]);
         }
-        auto interp2 = [&](const float2* f2, int a, bool in, int st, const float2* Lw) {
-            if (!in) return make_float2(0.f, 0.f);
+        auto interp2 = [&](const float2* f2, int a, int a2, bool in, int st, const float2* Lw, f32x2& s, f32x2& r) {
+            s = r = x2_pack(0.f, 0.f);
+            if (!in) return;
             const float2* fa = f2 + (size_t)a * A.Nr + st;
-            float hi = 0.f, lo = 0.f;
+            const float2* fb = f2 + (size_t)a2 * A.Nr + st;
+            f32x2 hi = s, lo = s;
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
-                const float2 v = fa[k];
-                const float p = Lw[k].x * v.x;
-                float e = fmaf(Lw[k].x, v.x, -p);
-                e = fmaf(Lw[k].x, v.y, e);
-                e = fmaf(Lw[k].y, v.x, e);
-                float r;
-                hi = two_sum(hi, p, r);
-                lo += r + e;
+                const float2 v = fa[k], w = fb[k];
+                const f32x2 vh = x2_pack(v.x, w.x), vl = x2_pack(v.y, w.y);
+                const f32x2 Lh = x2_pack(Lw[k].x, Lw[k].x), Ll = x2_pack(Lw[k].y, Lw[k].y);
+                f32x2 p, e, c;
+                df_mul_pe_x2(Lh, Ll, vh, vl, p, e);
+                hi = two_sum_x2(hi, p, c);
+                lo = x2_add(lo, x2_add(c, e));
             }
-            const float s = hi + lo;
-            return make_float2(s, lo - (s - hi));
+            s = x2_add(hi, lo);
+            r = x2_sub(lo, x2_sub(s, hi));
         };
         const int nlq = A.nlqT > A.nlqP ? A.nlqT : A.nlqP;
-        float2* s_th = s_tc;
-        float2* s_r = s_th + (size_t)nlq * 128;
-        float2* s_f = s_r + 2 * 128;
+        float* s_th = s_tc;
+        float* s_r = s_th + (size_t)nlq * 256;
+        float* s_f = s_r + 2 * 256;
         const int tx = threadIdx.x, wid = tx >> 5, lid = tx & 31;
+        auto put = [&](float* row, float2 v) {
+            row[tx] = v.x;
+            row[128 + tx] = v.y;
+        };
         // A_P per half column as double-floats
-        theta_lq(cP, A.lmaxP, A, [&](int q, double val) { s_th[q * 128 + tx] = df_split(val); });
+        theta_lq(cP, A.lmaxP, A, [&](int q, double val) { put(s_th + q * 256, df_split(val)); });
         float2* aP = reinterpret_cast<float2*>(reinterpret_cast<float*>(base) + A.t6_ap_off);
-        for (int b2 = 0; b2 < A.nradP; ++b2) {
-            const float2 fv = interp2(A.fP2, b2, inP, sP, LP2);
-            const int l = A.radP_l[b2];
-            for (int q = 0; q <= l; ++q) {
-                const int j = A.half_of[b2 * (WPCCC_LMAX + 1) + q];
-                aP[(size_t)j * A.G + g] = df_mul(fv, s_th[(l * (l + 1) / 2 + q) * 128 + tx]);
+        for (int b2 = 0; b2 < A.nradP; b2 += 2) {
+            f32x2 fh, fl;
+            interp2(A.fP2, b2, min(b2 + 1, A.nradP - 1), inP, sP, LP2, fh, fl);
+            float2 fv[2];
+            x2_unpack(fh, fv[0].x, fv[1].x);
+            x2_unpack(fl, fv[0].y, fv[1].y);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (b2 + u >= A.nradP) break;
+                const int l = A.radP_l[b2 + u];
+                for (int q = 0; q <= l; ++q) {
+                    const int j = A.half_of[(b2 + u) * (WPCCC_LMAX + 1) + q];
+                    const float* th = s_th + (l * (l + 1) / 2 + q) * 256 + tx;
+                    aP[(size_t)j * A.G + g] = df_mul(fv[u], make_float2(th[0], th[128]));
+                }
             }
         }
-        theta_lq(cT, A.lmaxT, A, [&](int q, double val) { s_th[q * 128 + tx] = df_split(val); });
+        theta_lq(cT, A.lmaxT, A, [&](int q, double val) { put(s_th + q * 256, df_split(val)); });
         const double rTV = A.mp_c == 0.0 ? -A.Z_T : -A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT);
-        s_r[tx] = df_split(rT);
-        s_r[128 + tx] = df_split(rTV);
+        put(s_r, df_split(rT));
+        put(s_r + 256, df_split(rTV));
         __nv_bfloat16* sp = reinterpret_cast<__nv_bfloat16*>(base);
         float* sc = reinterpret_cast<float*>(base) + A.t6_sc_off + (size_t)blockIdx.x * A.tc_rows;
         const size_t split = (size_t)A.tc_rows * A.G;
-        const int g0 = blockIdx.x * 128;
-        // one row of the slice planes at the window's 128 nodes: lane holds nodes lid + 32 j
-        auto put_row = [&](size_t row, const float2* xv, float mx) {
-            const int sh = oz_shift(mx);
+        const int g0 = blockIdx.x * 128 + 4 * lid;   // lane: nodes 4 lid .. 4 lid + 3 of the window
+        // four nodes' double-floats as two packed pairs
+        auto load4 = [&](const float* row, f32x2 h[2], f32x2 l[2]) {
+            const float4 a = *reinterpret_cast<const float4*>(row + 4 * lid);
+            const float4 b = *reinterpret_cast<const float4*>(row + 128 + 4 * lid);
+            h[0] = x2_pack(a.x, a.y);
+            h[1] = x2_pack(a.z, a.w);
+            l[0] = x2_pack(b.x, b.y);
+            l[1] = x2_pack(b.z, b.w);
+        };
+        // the rows r1 of m and, unless negative, r2 of -m (sign (-1)^m: `flip`) of the slice planes at the window's nodes
+        auto put_rows = [&](int r1, int r2, bool flip, const f32x2 h[2], const f32x2 l[2]) {
+            float m = 0.f;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                __nv_bfloat16 q[OZ_SLICES];
-                const size_t o = row * A.G + g0 + lid + 32 * j;
-                if (A.tc_slices == OZ_FAST_SLICES) {
-                    oz_slices<OZ_FAST_SLICES>(xv[j].x, xv[j].y, sh, q);
-#pragma unroll
-                    for (int i = 0; i < OZ_FAST_SLICES; ++i) sp[i * split + o] = q[i];
-                } else {
-                    oz_slices<OZ_SLICES>(xv[j].x, xv[j].y, sh, q);
-#pragma unroll
-                    for (int i = 0; i < OZ_SLICES; ++i) sp[i * split + o] = q[i];
-                }
+            for (int u = 0; u < 2; ++u) {
+                float a, b;
+                x2_unpack(h[u], a, b);
+                m = fmaxf(m, fmaxf(fabsf(a), fabsf(b)));
             }
-            if (lid == 0) sc[row] = ldexpf(1.f, -sh);
+            const int sh = oz_shift(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m))));
+            auto slices = [&](auto n) {
+                constexpr int NS = decltype(n)::value;
+                uint32_t q[2][NS];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) oz_slices_x2<NS>(h[u], l[u], sh, q[u]);
+#pragma unroll
+                for (int i = 0; i < NS; ++i) {
+                    *reinterpret_cast<uint2*>(sp + i * split + (size_t)r1 * A.G + g0) = make_uint2(q[0][i], q[1][i]);
+                    const uint32_t f = flip ? 0x80008000u : 0u;
+                    if (r2 >= 0) *reinterpret_cast<uint2*>(sp + i * split + (size_t)r2 * A.G + g0) = make_uint2(q[0][i] ^ f, q[1][i] ^ f);
+                }
+            };
+            if (A.tc_slices == OZ_FAST_SLICES) slices(IntC<OZ_FAST_SLICES>());
+            else slices(IntC<OZ_SLICES>());
+            if (lid == 0) {
+                const float v = ldexpf(1.f, -sh);
+                sc[r1] = v;
+                if (r2 >= 0) sc[r2] = v;
+            }
         };
         for (int a0 = 0; a0 < A.nradT; a0 += TC_NA) {
             const int na = A.nradT - a0 < TC_NA ? A.nradT - a0 : TC_NA;
             __syncthreads();   // the previous batch's rows are written (and, first time, Theta_T and r are in)
-            for (int j = 0; j < na; ++j) s_f[j * 128 + tx] = interp2(A.fT2, a0 + j, inT, sT, LT2);
+            for (int j = 0; j < na; j += 2) {
+                f32x2 fh, fl;
+                interp2(A.fT2, a0 + j, min(a0 + j + 1, A.nradT - 1), inT, sT, LT2, fh, fl);
+                float2 f0, f1;
+                x2_unpack(fh, f0.x, f1.x);
+                x2_unpack(fl, f0.y, f1.y);
+                put(s_f + j * 256, f0);
+                if (j + 1 < na) put(s_f + (j + 1) * 256, f1);
+            }
             __syncthreads();
-            // the batch's states, one per warp in turn: (radial function, m) pairs in order
+            // the batch's (radial function, m >= 0) pairs, one per warp in turn
             int pair = 0;
             for (int j = 0; j < na; ++j) {
                 const int a = a0 + j, l = A.radT_l[a];
-                for (int m = -l; m <= l; ++m, ++pair) {
+                const int* idx = A.stT_index + a * (2 * WPCCC_LMAX + 1) + WPCCC_LMAX;
+                for (int m = 0; m <= l; ++m, ++pair) {
                     if ((pair & 3) != wid) continue;
-                    const int i = A.stT_index[a * (2 * WPCCC_LMAX + 1) + m + WPCCC_LMAX];
-                    const int am = m < 0 ? -m : m;
-                    const bool neg = m < 0 && (am & 1);
-                    const float2* th = s_th + (l * (l + 1) / 2 + am) * 128;
-                    float2 x1[4], x2[4];
-                    float m1 = 0.f, m2 = 0.f;
+                    const int ip = idx[m], in = m > 0 ? idx[-m] : ip;
+                    const int rp = A.tc_row[ip], tp = A.tc_row[A.N_T + ip], rn = A.tc_row[in], tn = A.tc_row[A.N_T + in];
+                    f32x2 fh[2], fl[2], th[2], tl[2], rh[2], rl[2];
+                    load4(s_f + j * 256, fh, fl);
+                    load4(s_th + (l * (l + 1) / 2 + m) * 256, th, tl);
 #pragma unroll
-                    for (int jj = 0; jj < 4; ++jj) {
-                        const int n = lid + 32 * jj;
-                        float2 tv = df_mul(s_f[j * 128 + n], th[n]);
-                        if (neg) tv = make_float2(-tv.x, -tv.y);
-                        x1[jj] = df_mul(tv, s_r[n]);
-                        x2[jj] = df_mul(tv, s_r[128 + n]);
-                        m1 = fmaxf(m1, fabsf(x1[jj].x));
-                        m2 = fmaxf(m2, fabsf(x2[jj].x));
-                    }
+                    for (int u = 0; u < 2; ++u) df_mul_x2(fh[u], fl[u], th[u], tl[u], th[u], tl[u]);
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-                        m2 = fmaxf(m2, __shfl_xor_sync(0xffffffffu, m2, o));
+                    for (int v = 0; v < 2; ++v) {
+                        load4(s_r + v * 256, rh, rl);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) df_mul_x2(th[u], tl[u], rh[u], rl[u], rh[u], rl[u]);
+                        put_rows(rp + v * tp, m > 0 ? rn + v * tn : -1, m & 1, rh, rl);
                     }
-                    const int row = A.tc_row[i];
-                    const int tsz = A.tc_row[A.N_T + i];
-                    put_row((size_t)row, x1, m1);
-                    put_row((size_t)(row + tsz), x2, m2);
                 }
             }
         }
@@ -1398,6 +1441,7 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
     na.Gp = L.Gp;
     na.f64_w2 = L.f64_w2;
     na.f64_r = L.f64_r;
+    for (int k = 0; k < 2 * WPCCC_LMAX + 2; ++k) na.num[k] = k;
     for (int l = 0; l <= WPCCC_LMAX; ++l) {
         na.inv_int[l] = l > 0 ? 1.0 / l : 0.0;
         for (int q = 0; q <= l; ++q) {

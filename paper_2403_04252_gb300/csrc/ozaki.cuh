@@ -93,6 +93,14 @@ static __device__ __forceinline__ void df_mul_pe_x2(f32x2 wh, f32x2 wl, f32x2 ah
     e = x2_fma(wl, ah, e);
 }
 
+// a b for double-floats (ah, al), (bh, bl) at two nodes at once (df_mul).
+static __device__ __forceinline__ void df_mul_x2(f32x2 ah, f32x2 al, f32x2 bh, f32x2 bl, f32x2& s, f32x2& r) {
+    f32x2 p, e;
+    df_mul_pe_x2(ah, al, bh, bl, p, e);
+    s = x2_add(p, e);
+    r = x2_sub(e, x2_sub(s, p));
+}
+
 // The four fixed-point slices of the pairs p + e of two nodes scaled by s2 = 2^sh in both halves
 // (|p s| < 128, |e| <= 2^-21 |p|), each rounded to its grid by adding and subtracting 1.5 2^23 times the
 // grid unit (1, 2^-8, 2^-16, 2^-24):
@@ -167,6 +175,35 @@ static __device__ __forceinline__ void oz_slices(float h, float l, int sh, __nv_
         p *= 256.f;
         e *= 256.f;
         w *= (1.f / 256.f);
+    }
+}
+
+// The slices of oz_slices for two double-floats (h, l) at once, packed as bf16x2.  The remainders stay unscaled: each
+// slice is the sum rounded to its grid 2^(-8 i) by adding and subtracting 1.5 2^23 times the grid's unit.
+template <int NS>
+static __device__ __forceinline__ void oz_slices_x2(f32x2 h, f32x2 l, int sh, uint32_t out[NS]) {
+    f32x2 p, e;
+    if (sh >= -126 && sh <= 127) {
+        const float s = __int_as_float((sh + 127) << 23);
+        p = x2_mul(h, x2_pack(s, s));
+        e = x2_mul(l, x2_pack(s, s));
+    } else {
+        float a, b;
+        x2_unpack(h, a, b);
+        p = x2_pack(ldexpf(a, sh), ldexpf(b, sh));
+        x2_unpack(l, a, b);
+        e = x2_pack(ldexpf(a, sh), ldexpf(b, sh));
+    }
+    float c = 12582912.f;
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+        const f32x2 C = x2_pack(c, c);
+        const f32x2 t = x2_sub(x2_add(x2_add(p, e), C), C);
+        p = x2_sub(p, t);
+        float a, b;
+        x2_unpack(t, a, b);
+        out[i] = bf16x2_exact(a, b);
+        c *= 1.f / 256.f;
     }
 }
 

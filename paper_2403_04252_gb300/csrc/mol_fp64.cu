@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
         for (int j = 0; j < A.nwin && ok; ++j) {
             const int Ea = lrow < 2 * ns ? ea[(size_t)j * A.tc_rows + row0 + lrow] : F64_EMIN;
             const int Eb = ebv ? eb[ebo + j] : F64_EMIN;
-            ok = mbar_wait(accf, j & 1, abort_flag, A.err, 35, A.wait_limit);
+            ok = mbar_wait_warp(accf, j & 1, abort_flag, A.err, 35, A.wait_limit);
             if (!ok) break;
             tc_fence_after();
             // first the nine levels of each element are put together; then the accumulators are free for the next
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             f64_digits(f64_fix(w1.x * ac.x, E1), f64_fix(w1.y * ac.y, E1), q1);
             if (k >= F64_GSTAGES) {
                 const int kp = k - F64_GSTAGES;
-                ok = mbar_wait(done0 + 8 * (kp % F64_DONE), (kp / F64_DONE) & 1, abort_flag, A.err, 36, A.wait_limit);
+                ok = mbar_wait_warp(done0 + 8 * (kp % F64_DONE), (kp / F64_DONE) & 1, abort_flag, A.err, 36, A.wait_limit);
             }
             if (!ok) break;
             unsigned char* bt = gsm + s * F64_GSTAGE;

@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
         bool ok = true;
         for (int j = 0; j < nwin && ok; ++j) {
             const int b = j & 1;
-            ok = mbar_wait(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 14, A.wait_limit);
+            ok = mbar_wait_warp(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 14, A.wait_limit);
             if (!ok) break;
             tc_fence_after();
             if (live) {
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
         // drain of window j: its accumulators with the window's scales
         auto drain = [&](int j) {
             const int b = j & 1;
-            ok = ok && mbar_wait(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 14, A.wait_limit);
+            ok = ok && mbar_wait_warp(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 14, A.wait_limit);
             if (!ok) return;
             tc_fence_after();
             if (live) {
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
         for (int w = 0; w < nwin && ok; ++w) {
             f32x2 pw[T6_WIN * 2], ew[T6_WIN * 2];
             float mx = 0.f;
-            ok = mbar_wait(rawfull, w & 1, abort_flag, A.err, 18, A.wait_limit);
+            ok = mbar_wait_warp(rawfull, w & 1, abort_flag, A.err, 18, A.wait_limit);
             if (!ok) break;
 #pragma unroll
             for (int cc = 0; cc < T6_WIN; ++cc) {
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
             for (int cc = 0; cc < T6_WIN; ++cc) {
                 const int k = w * T6_WIN + cc, s = k % T6_GSTAGES;
                 if (k >= T6_GSTAGES)
-                    ok = ok && mbar_wait(gempty0 + 8 * s, ((k - T6_GSTAGES) / T6_GSTAGES) & 1, abort_flag, A.err, 15, A.wait_limit);
+                    ok = ok && mbar_wait_warp(gempty0 + 8 * s, ((k - T6_GSTAGES) / T6_GSTAGES) & 1, abort_flag, A.err, 15, A.wait_limit);
                 if (!ok) break;
                 unsigned char* bt = gsm + s * T6_GSTAGE_BYTES;
                 f32x2 t0[4], t1[4];
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
             // window's 128 nodes (the row's eight threads), and the window's scales
             float2 xw[T6_WIN * 4];
             float mx = 0.f;
-            ok = mbar_wait(rawfull, w & 1, abort_flag, A.err, 18, A.wait_limit);
+            ok = mbar_wait_warp(rawfull, w & 1, abort_flag, A.err, 18, A.wait_limit);
             if (!ok) break;
 #pragma unroll
             for (int cc = 0; cc < T6_WIN; ++cc) {
@@ -593,7 +593,7 @@ __global__ void __launch_bounds__(Tc64Cfg<SL>::THREADS, 1) k_mol_tc64(const __gr
             for (int cc = 0; cc < T6_WIN; ++cc) {
                 const int k = w * T6_WIN + cc, s = k % T6_GSTAGES;
                 if (k >= T6_GSTAGES)
-                    ok = ok && mbar_wait(gempty0 + 8 * s, ((k - T6_GSTAGES) / T6_GSTAGES) & 1, abort_flag, A.err, 15, A.wait_limit);
+                    ok = ok && mbar_wait_warp(gempty0 + 8 * s, ((k - T6_GSTAGES) / T6_GSTAGES) & 1, abort_flag, A.err, 15, A.wait_limit);
                 if (!ok) break;
                 unsigned char* bt = gsm + s * T6_GSTAGE_BYTES;
                 __nv_bfloat16 q[4][SL];

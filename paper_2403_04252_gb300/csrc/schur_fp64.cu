@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(SD_THREADS, 1) k_schur_f64tc(const __grid_cons
         for (int j = 0; j < A.nwin && ok; ++j) {
             const int Em = m < A.NP ? ex[(size_t)j * A.NP + m] : F64_EMIN;
             const int nn = n0 + col0 + (lane & 15), En = nn < A.NP ? ex[(size_t)j * A.NP + nn] : F64_EMIN;
-            ok = mbar_wait(accf, j & 1, abort_flag, A.err, 44, A.wait_limit);
+            ok = mbar_wait_warp(accf, j & 1, abort_flag, A.err, 44, A.wait_limit);
             if (!ok) break;
             tc_fence_after();
             const uint32_t base = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)col0;

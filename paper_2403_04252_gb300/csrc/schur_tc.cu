@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(SU_THREADS, 1) k_schur_gemm_tc(const __grid_co
         bool ok = true;
         for (int j = 0; j < A.nwin && ok; ++j) {
             const int b = j & 1;
-            ok = mbar_wait(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 24, A.wait_limit);
+            ok = mbar_wait_warp(accf0 + 8 * b, (j >> 1) & 1, abort_flag, A.err, 24, A.wait_limit);
             if (!ok) break;
             tc_fence_after();
             const float* scw = scA + (size_t)j * A.NP2;

@@ -59,6 +59,13 @@ static __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* ab
     return false;
 }
 
+// The same by a whole warp: one outcome for all lanes, so that a lane that saw the wait give up does not leave the others
+// at the warp's next synchronising instruction.
+static __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* err, int code,
+                                                      long limit) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, err, code, limit));
+}
+
 static __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 static __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 

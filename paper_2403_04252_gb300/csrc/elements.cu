@@ -1187,8 +1187,12 @@ __global__ void __launch_bounds__(256) k_direct(DirArgs A0, DirArgs A1, const Ev
 // In the molecular frame the potential is symmetric about the axis, so only equal q couple:
 //   I[b][q] = (R^3/8) sum_g w_g (eta^2 - tau^2) V_s(r_T) f_a(r_P) Theta_{l_a q}(c_P) f_b(r_P) Theta_{l_b q}(c_P)
 // (Theta_{l,-q} = (-1)^q Theta_{l,q}, so I does not depend on the sign of q).  One block per
-// (projectile radial a, position): a warp per (b, q) sums over the nodes, then the rows of a are
-// rotated with d^{l}(theta) on both sides, given their energy phases and added to H.
+// (group of NA projectile radials a, position, part of the b): a warp per (b, q) sums over the nodes, then the rows of the a are
+// rotated with d^{l}(theta) on both sides, given their energy phases and added to H.  The FP64 pipe bounds the sums: with
+// NA = 4 the factor of a, Theta_{l_a q} included, is formed once per q and f_b Theta_{l_b q} once for all four a (2.25
+// instead of 3 operations per term at NA = 1, which more than about 5700 nodes take: shared memory; the sums are the same
+// bits), and the b are split over blocks where there are few positions.  p + Li, N = 379, 108 positions in calls of 4 to
+// 12: with rotation and direct blocks 13.6 -> 10.4 ms.
 // ---------------------------------------------------------------------------
 struct SrArgs {
     int G, Gtau, nradT, nradP, lmaxP, nlqT, N_T, N_P, N, dtot;
@@ -1204,9 +1208,16 @@ struct SrArgs {
     size_t mat;
 };
 
+template <int NA>
+static size_t direct_sr_smem(int G, int nradP, int LQ, int dtot) {
+    return ((size_t)(NA > 1 ? NA + 1 : 1) * G + (size_t)NA * nradP * LQ + dtot) * sizeof(double);
+}
+
+template <int NA>
 __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __restrict__ ev) {
-    extern __shared__ double srm[];   // [G] V_s-weighted f_a, then I[n_radP][lmaxP+1], then Wigner d
-    const int a = blockIdx.x, e = blockIdx.y;
+    extern __shared__ double srm[];   // [G] weighted V_s (NA = 1: times f_a), NA > 1: [NA][G] factors of the a, I[NA][n_radP][lmaxP+1], Wigner d
+    const int a0 = blockIdx.x * NA, e = blockIdx.y;
+    const int b0 = A.nradP * blockIdx.z / gridDim.z, b1 = A.nradP * (blockIdx.z + 1) / gridDim.z;
     const double b = ev[e].b, z = ev[e].z;
     const double R = dist_R(b, z);
     const double gR = __dmul_rn(A.gamma, R);
@@ -1215,9 +1226,10 @@ __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __r
     const double* oP = base + (size_t)A.nradT * A.G;
     const double* thP = oP + (size_t)A.nradP * A.G + (size_t)A.nlqT * A.G;
     const int LQ = A.lmaxP + 1;
-    double* ufa = srm;
-    double* I = srm + A.G;
-    double* dt = I + A.nradP * LQ;
+    double* uv = srm;
+    double* U = uv + A.G;
+    double* I = NA > 1 ? U + (size_t)NA * A.G : U;
+    double* dt = I + (size_t)NA * A.nradP * LQ;
     for (int g = threadIdx.x; g < A.G; g += blockDim.x) {
         const int k = g / A.Gtau, t = g - k * A.Gtau;
         const double eta = __dadd_rn(1.0, __ddiv_rn(A.s[k], gR));
@@ -1226,49 +1238,80 @@ __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __r
         const double wgt = (A.ws[k] / gR) * A.wtau[t];
         const double vol = (R * R * R / 8.0) * wgt * (eta * eta - tau * tau);
         const double Vs = (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT) / rT;
-        ufa[g] = vol * Vs * oP[(size_t)a * A.G + g];
+        uv[g] = NA > 1 ? vol * Vs : vol * Vs * oP[(size_t)a0 * A.G + g];
     }
     const double* etd = A.et + (size_t)e * A.et_doubles;
     for (int t = threadIdx.x; t < A.dtot; t += blockDim.x) dt[t] = etd[t];
     __syncthreads();
-    const int la = A.radP_l[a];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int pq = warp; pq < A.nradP * LQ; pq += nw) {
-        const int bb = pq / LQ, q = pq - bb * LQ;
-        const int lb = A.radP_l[bb];
-        double acc = 0.0;
-        if (q <= la && q <= lb) {
-            const double* ta = thP + (size_t)(la * (la + 1) / 2 + q) * A.G;
-            const double* tb = thP + (size_t)(lb * (lb + 1) / 2 + q) * A.G;
-            const double* fb = oP + (size_t)bb * A.G;
-            for (int g = lane; g < A.G; g += 32) acc = fma(ufa[g] * ta[g], fb[g] * tb[g], acc);
+    int la[NA];
+#pragma unroll
+    for (int k = 0; k < NA; ++k) la[k] = a0 + k < A.nradP ? A.radP_l[a0 + k] : -1;
+    for (int q = 0; q < LQ; ++q) {
+        if (NA > 1) {
+#pragma unroll
+            for (int k = 0; k < NA; ++k)
+                if (q <= la[k])
+                    for (int g = threadIdx.x; g < A.G; g += blockDim.x)
+                        U[(size_t)k * A.G + g] = uv[g] * oP[(size_t)(a0 + k) * A.G + g] *
+                                                 thP[(size_t)(la[k] * (la[k] + 1) / 2 + q) * A.G + g];
+            __syncthreads();
         }
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) I[pq] = acc;
+        for (int bb = b0 + warp; bb < b1; bb += nw) {
+            const int lb = A.radP_l[bb];
+            double acc[NA];
+#pragma unroll
+            for (int k = 0; k < NA; ++k) acc[k] = 0.0;
+            if (q <= lb) {
+                const double* tb = thP + (size_t)(lb * (lb + 1) / 2 + q) * A.G;
+                const double* fb = oP + (size_t)bb * A.G;
+                if (NA > 1) {
+                    for (int g = lane; g < A.G; g += 32) {
+                        const double w = fb[g] * tb[g];
+#pragma unroll
+                        for (int k = 0; k < NA; ++k) acc[k] = fma(U[(size_t)k * A.G + g], w, acc[k]);
+                    }
+                } else if (q <= la[0]) {
+                    const double* ta = thP + (size_t)(la[0] * (la[0] + 1) / 2 + q) * A.G;
+                    for (int g = lane; g < A.G; g += 32) acc[0] = fma(uv[g] * ta[g], fb[g] * tb[g], acc[0]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < NA; ++k) {
+                for (int o = 16; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+                if (lane == 0) I[(k * A.nradP + bb) * LQ + q] = q <= la[k] ? acc[k] : 0.0;
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
     // lab frame: D[(a, m)][(b, m')] = sum_q d^{la}_{m q} d^{lb}_{m' q} I[b][|q|]
-    int offa = 0;
-    for (int l = 0; l < la; ++l) offa += (2 * l + 1) * (2 * l + 1);
+    const double2* phs = reinterpret_cast<const double2*>(etd + A.ph_off);
     double2* H = A.H + (size_t)e * A.mat;
-    for (int idx = threadIdx.x; idx < (2 * la + 1) * A.N_P; idx += blockDim.x) {
-        const int mi = idx / A.N_P - la, j = idx % A.N_P;
-        const int bb = A.stP_rad[j], lb = A.radP_l[bb], mj = A.stP_m[j];
-        int offb = 0;
-        for (int l = 0; l < lb; ++l) offb += (2 * l + 1) * (2 * l + 1);
-        const int qm = la < lb ? la : lb;
-        double D = 0.0;
-        for (int q = -qm; q <= qm; ++q) {
-            const double da = dt[offa + (mi + la) * (2 * la + 1) + (q + la)];
-            const double db = dt[offb + (mj + lb) * (2 * lb + 1) + (q + lb)];
-            D = fma(da * db, I[bb * LQ + (q < 0 ? -q : q)], D);
+    for (int k = 0; k < NA; ++k) {
+        const int a = a0 + k;
+        if (a >= A.nradP) break;
+        const int l = A.radP_l[a];
+        int offa = 0;
+        for (int x = 0; x < l; ++x) offa += (2 * x + 1) * (2 * x + 1);
+        for (int idx = threadIdx.x; idx < (2 * l + 1) * A.N_P; idx += blockDim.x) {
+            const int mi = idx / A.N_P - l, j = idx % A.N_P;
+            const int bb = A.stP_rad[j], lb = A.radP_l[bb], mj = A.stP_m[j];
+            if (bb < b0 || bb >= b1) continue;
+            int offb = 0;
+            for (int x = 0; x < lb; ++x) offb += (2 * x + 1) * (2 * x + 1);
+            const int qm = l < lb ? l : lb;
+            double D = 0.0;
+            for (int q = -qm; q <= qm; ++q) {
+                const double da = dt[offa + (mi + l) * (2 * l + 1) + (q + l)];
+                const double db = dt[offb + (mj + lb) * (2 * lb + 1) + (q + lb)];
+                D = fma(da * db, I[(k * A.nradP + bb) * LQ + (q < 0 ? -q : q)], D);
+            }
+            const int i = A.stP_index[a * (2 * WPCCC_LMAX + 1) + mi + WPCCC_LMAX];
+            const double2 ph = cmul(phs[A.N_T + i], cconj(phs[A.N_T + j]));
+            const size_t o = (size_t)(A.N_T + i) + (size_t)(A.N_T + j) * A.N;
+            const double2 h = H[o];
+            H[o] = make_double2(fma(D, ph.x, h.x), fma(D, ph.y, h.y));
         }
-        const int i = A.stP_index[a * (2 * WPCCC_LMAX + 1) + mi + WPCCC_LMAX];
-        const double2* phs = reinterpret_cast<const double2*>(etd + A.ph_off);
-        const double2 ph = cmul(phs[A.N_T + i], cconj(phs[A.N_T + j]));
-        const size_t o = (size_t)(A.N_T + i) + (size_t)(A.N_T + j) * A.N;
-        const double2 h = H[o];
-        H[o] = make_double2(fma(D, ph.x, h.x), fma(D, ph.y, h.y));
     }
 }
 
@@ -1640,10 +1683,19 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
         sa.epsP = B->P.st_eps;
         sa.H = H;
         sa.mat = (size_t)B->N * B->N;
-        const size_t srsm = ((size_t)B->G + (size_t)B->P.n_rad * (B->P.lmax + 1) + L.dtot) * sizeof(double);
-        WPCCC_CUDA(cudaFuncSetAttribute(k_direct_sr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srsm));
+        const int LQ = B->P.lmax + 1;
+        const size_t sm4 = direct_sr_smem<4>(B->G, B->P.n_rad, LQ, L.dtot);
+        const bool four = sm4 <= (size_t)226 * 1024;
+        const size_t srsm = four ? sm4 : direct_sr_smem<1>(B->G, B->P.n_rad, LQ, L.dtot);
+        auto kern = four ? k_direct_sr<4> : k_direct_sr<1>;
+        WPCCC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srsm));
         ed = B->prof.begin(PROF_ROT_DIRECT, st);
-        k_direct_sr<<<dim3(B->P.n_rad, nev), 256, srsm, st>>>(sa, evals);
+        // the b in parts while there are fewer than three blocks per SM and a block's warps have a b each
+        int sms = 0;
+        WPCCC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, B->device));
+        const int groups = four ? (B->P.n_rad + 3) / 4 : B->P.n_rad;
+        const int parts = std::max(1, std::min(B->P.n_rad / 8, (3 * sms + groups * nev - 1) / (groups * nev)));
+        kern<<<dim3(groups, nev, parts), 256, srsm, st>>>(sa, evals);
         WPCCC_CHECK_LAUNCH("k_direct_sr");
         B->prof.end(PROF_ROT_DIRECT, st, ed);
     }

@@ -352,7 +352,7 @@ def run_batch(args) -> dict:
         n_half = int(sum(1 for m in basis.P.st_m if m >= 0))
         cats = _category_rooflines(basis, mode, args.solve_mode, basis.N, n_half)
         cats["rk4"] = (_rk4_flops_per_step(mode, args.solve_mode, basis.N, basis.T.N, basis.P.N),
-                       ("alu", FP64_PEAK_TFLOPS, "TFLOP/s"), "k_rk4")
+                       ("alu", FP64_PEAK_TFLOPS, "TFLOP/s"), _rk4_kernel(mode, args.solve_mode))
         for k, (per_unit, meta, name) in cats.items():
             n_units = args.steps * b.size * (seg.size - 1) if k == "rk4" else evals
             work[k] = work.get(k, 0.0) + per_unit * n_units
@@ -654,7 +654,8 @@ def run_grad(args) -> None:
     flops["mol_gemm"] = 8.0 * basis.T.N * n_half * basis.quad.G * evals
     flops["solve"] = (8.0 / 3.0) * basis.N ** 3 * evals
     dom = max(prof, key=lambda k: prof[k][0])
-    dom_f = dom if dom in flops else "mol_gemm"
+    dom_f = "solve" if dom != "mol_gemm" else dom
+    peak = {"mol_gemm": BF16_SUSTAINED_TFLOPS, "solve": FP64_PEAK_TFLOPS}[dom_f]
     achieved = flops[dom_f] / (prof[dom_f][0] / 1e3) / 1e12
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
@@ -673,11 +674,11 @@ def run_grad(args) -> None:
             "gradient_finite": finite,
             "fd_check": fd_check,
             "kernel_ms": {k: v_[0] for k, v_ in prof.items()},
-            "roofline": {"bound": "alu", "kernel": {"mol_gemm": "k_mol_gemm<double>",
-                                                           "solve": "k_lu_solve"}[dom_f],
-                         "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                         "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                         "peak_source": "FP64 pipe from unit counts and clocks (152 SMs x 2 DFMA/clk x 2.07 GHz)",
+            "roofline": {"bound": {"mol_gemm": "tensor", "solve": "alu"}[dom_f],
+                         "kernel": {"mol_gemm": "k_mol_f64tc", "solve": "k_lu<double>"}[dom_f],
+                         "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                         "frac": achieved / peak, "traffic": None,
+                         "peak_source": _peak_source({"mol_gemm": "tensor", "solve": "alu"}[dom_f], peak),
                          "dominant_category": dom},
             "e2e": {"value": world * units * args.steps / e2e_s, "unit": UNIT,
                     "h2d_bytes_per_step": c_host.numel() * 16,
@@ -697,7 +698,7 @@ def _category_rooflines(basis, mode: int, solve_mode: str, N: int, n_half: int) 
     """Per position (evaluation of S and H at one z): the work each category of kernels must do, as the
     method defines it, with the bound and peak that apply.  Contraction: K and Q over the full N_T x N_P
     block, 4 real flops per node each (8 N_T N_P G; the q -> -q reflection lets the kernels form only the
-    n_half projectile columns with q >= 0, and the tensor-core forms issue 10 or 28 bf16 slice products per
+    n_half projectile columns with q >= 0, and the tensor-core forms issue 10, 28 or 43 bf16 slice products per
     algorithmic product: neither changes the algorithmic count).  Factorisation: the Schur complement's
     lower triangle and its Cholesky factor (4 N_P^2 N_T + 4/3 N_P^3), or LU (8/3 N^3).  Node tables and
     rotation/direct blocks are bound by memory: the bytes they must write (node tables of the layout the
@@ -716,17 +717,16 @@ def _category_rooflines(basis, mode: int, solve_mode: str, N: int, n_half: int) 
     elif mode == 1:
         node_bytes = (NT + n_half) * G * 4 + 2 * (dmax + 1) * G * 8
     else:
-        node_bytes = (nradT + nradP + nlqT + nlqP) * G * 8 + 2 * (dmax + 1) * G * 16
+        node_bytes = (nradT + nradP + nlqT + nlqP) * G * 8 + 2 * (dmax + 2) * G * 8
     if solve_mode == "schur":
         f_solve = 4.0 * NP_ * NP_ * NT + (4.0 / 3.0) * NP_ ** 3
     else:
         f_solve = (8.0 / 3.0 + (8.0 if (solve_mode == "matrix" and not mixed) else 0.0)) * N ** 3
     mol_name = {1: "k_mol_gemm_f32q", 3: "k_mol_tc64<4>", 4: "k_mol_tc64<7>", 5: "k_mol_tc64<7>"}.get(
-        mode, "k_mol_gemm<double>")
-    solve_name = (("k_schur_factor<float>" if solve_mode == "schur" else "k_lu_factor_f32") if mixed
-                  else ("k_schur_factor<double>" if solve_mode == "schur" else "k_lu_solve"))
-    mol_peak = (("tensor", BF16_SUSTAINED_TFLOPS, "TFLOP/s") if tc else
-                ("alu", FP32_PEAK_TFLOPS, "TFLOP/s") if mode == 1 else ("alu", FP64_PEAK_TFLOPS, "TFLOP/s"))
+        mode, "k_mol_f64tc")
+    solve_name = (("k_schur_factor<float>" if solve_mode == "schur" else "k_lu<float>") if mixed
+                  else ("k_schur_f64tc+k_schur_factor<double>" if solve_mode == "schur" else "k_lu<double>"))
+    mol_peak = (("alu", FP32_PEAK_TFLOPS, "TFLOP/s") if mode == 1 else ("tensor", BF16_SUSTAINED_TFLOPS, "TFLOP/s"))
     return {
         "node_tables": (float(node_bytes), ("hbm", HBM_MEASURED_GBS, "GB/s"),
                         "k_node_tables<float>" if (tc or mode == 1) else "k_node_tables<double>"),
@@ -751,6 +751,12 @@ def _peak_source(bound: str, peak: float) -> str:
             f"measured DFMA microbenchmark {FP64_DFMA_MEASURED_TFLOPS} TFLOP/s")
 
 
+def _rk4_kernel(mode: int, solve_mode: str) -> str:
+    if mode in (1, 2, 3, 5):
+        return "k_rk4_mixed_schur" if solve_mode == "schur" else "k_rk4_mixed_lu"
+    return "k_rk4_fp64"
+
+
 def _rk4_flops_per_step(mode: int, solve_mode: str, N: int, NT: int, NP_: int) -> float:
     """RK4 per path-step (FP64): 4 applications of M; matrix form X y, stage form H y + two triangles,
     Schur form H y, K^+ t_T, K x_P and two triangles of N_P; refined forms H y, two preconditioner solves
@@ -769,9 +775,6 @@ def _rk4_flops_per_step(mode: int, solve_mode: str, N: int, NT: int, NP_: int) -
 # dram__bytes_write.sum over a capture of whole launches, divided by the positions): only kernels whose code
 # is unchanged since the capture are listed (the others report traffic null)
 MEASURED_TRAFFIC_PER_POSITION = {
-    # ncu over 33 positions of the p + H workload, precision mode 3: (314.0 + 17.5) MB and (3.7 + 263.2) MB
-    ("p_H_2c_n4l3", "k_mol_tc64<4>"): 10.05e6,
-    ("p_H_2c_n4l3", "k_node_tables<float>"): 8.09e6,
 }
 
 
@@ -945,8 +948,8 @@ def run_fixed_speed(args, sub: bool = False) -> dict:
     evals = args.steps * n_paths * (2 * STEP + 1)
     cats = _category_rooflines(basis, mode, args.solve_mode, N, n_half)
     cats["rk4"] = (_rk4_flops_per_step(mode, args.solve_mode, N, NT, NP_), ("alu", FP64_PEAK_TFLOPS, "TFLOP/s"),
-                   "k_rk4")
-    issued = {3: 10.0, 4: 28.0, 5: 28.0}.get(mode)
+                   _rk4_kernel(mode, args.solve_mode))
+    issued = {0: 43.0, 2: 43.0, 3: 10.0, 4: 28.0, 5: 28.0}.get(mode)
 
     def roof(key: str) -> dict:
         k_ms, k_launches = prof[key]
@@ -977,7 +980,8 @@ def run_fixed_speed(args, sub: bool = False) -> dict:
                            "factorisation on the caller's stream; shares are of the summed kernel time")
     total_flops = (cats["mol_gemm"][0] + cats["solve"][0]) * evals + cats["rk4"][0] * n_paths * STEP * args.steps
     launches = int(sum(n for _, n in prof.values()))
-    form_desc = {0: "plain FP64, all paths batched; S^-1 applied "
+    form_desc = {0: "FP64 (Eq. 9 contraction on tcgen05 in eight exact seven-bit digits per operand, 43 digit products), all "
+                    "paths batched; S^-1 applied "
                     + {"stage": "per RK4 stage from LU factors",
                        "schur": "per RK4 stage through the Cholesky factor of the Schur complement I - K^+ K",
                        "matrix": "as X = S^-1 H with N right-hand sides (the paper's ZGESV form)"}[args.solve_mode],

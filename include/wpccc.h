@@ -64,7 +64,8 @@ typedef enum {
                               wpccc_basis_set_refine_tolerance); the amplitudes are returned but not trusted */
 } wpccc_status;
 
-/* Largest orbital angular momentum a basis may hold, and largest system size.  Beyond about 2840 states
+/* Largest orbital angular momentum a basis may hold, and largest system size.  Beyond 2688 states
+ * (fewer in some modes)
  * the RK4 sweep of the two-centre forms no longer fits one block's shared memory (EINVAL from
  * wpccc_propagate); one-centre bases then propagate with the vectors in global memory (see
  * wpccc_basis_set_rk4_layout). */
@@ -243,7 +244,8 @@ WPCCC_API wpccc_status wpccc_solve(int N, int batch, void* S, void* H, int* ipiv
  *      node (Algorithm 1 starts from c = (1, 0, ..., 0)); out, the amplitudes at
  *      its last node.
  *   precision_mode
- *     0  FP64 throughout;
+ *     0  FP64 throughout (the Eq. 9 contraction and the Schur solve's update I - K^+ K in exact fixed-point
+ *        digits on the tensor cores where they can run there, with at least FP64's accuracy);
  *     1  mixed: the Eq. 9 contraction and the LU factors of S on the FP32 pipe,
  *        each RK4 stage's S^{-1} solved by FP64 iterative refinement (residuals
  *        against the FP64 S), RK4 amplitudes in FP64;
@@ -375,8 +377,8 @@ WPCCC_API wpccc_status wpccc_basis_set_solve_mode(wpccc_basis basis, int mode);
  *                                  operands in four fixed-point bf16 slices per 128-wide window with exact
  *                                  FP32 level accumulators (about 2^-28 of each window's largest term), then
  *                                  the Cholesky factor on the CUDA cores;
- *   WPCCC_SCHUR_UPDATE_CUDA_CORES  update and Cholesky factor in FP32 on the CUDA cores, one block per
- *                                  position;
+ *   WPCCC_SCHUR_UPDATE_CUDA_CORES  update and Cholesky factor in FP32 on the CUDA cores, a cluster of
+ *                                  blocks per position;
  *   WPCCC_SCHUR_UPDATE_AUTO        (default) tensor cores when N_P >= 256, else CUDA cores (below that the
  *                                  three launches of the tensor-core route cost more than they save).
  * Both are preconditioners of the same FP64 refinement; the tensor-core one is the more accurate (its
@@ -425,9 +427,9 @@ WPCCC_API wpccc_status wpccc_basis_set_wait_limit(wpccc_basis basis, long polls)
 
 /*
  * Where the RK4 sweep of Algorithm 1 keeps its vectors.
- *   WPCCC_RK4_SHARED  one thread block per path, c and the stage vectors in its shared memory, all the
- *                     chunk's steps in one launch (fastest; N up to about 2840 in the one-centre form,
- *                     fewer in the two-centre forms);
+ *   WPCCC_RK4_SHARED  a cluster of one to eight thread blocks per path, c and the stage vectors in the
+ *                     blocks' shared memory, all the chunk's steps in one launch (fastest; N up to 2688 in
+ *                     the one-centre form, at most that in the two-centre forms);
  *   WPCCC_RK4_GLOBAL  one-centre form only: one launch per RK4 stage for all paths of a chunk, the
  *                     matrix-vector product M(z) y spread over the GPU (a thread per row, the columns of
  *                     y staged in shared memory), the vectors in global memory; every chunk evaluates its

@@ -260,7 +260,7 @@ class Basis:
         _check(_lib.wpccc_basis_set_solve_mode(self._h, int(mode)), "wpccc_basis_set_solve_mode")
 
     def set_rk4_layout(self, layout: int) -> None:
-        """RK4_AUTO (default), RK4_SHARED (one block per path, vectors in shared memory) or RK4_GLOBAL
+        """RK4_AUTO (default), RK4_SHARED (a cluster of blocks per path, vectors in shared memory) or RK4_GLOBAL
         (one-centre form: a launch per RK4 stage, vectors in global memory, any N)."""
         _check(_lib.wpccc_basis_set_rk4_layout(self._h, int(layout)), "wpccc_basis_set_rk4_layout")
 

@@ -559,7 +559,7 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     P.N = N;
     P.two = B->n_centres == 2;
     // 1: FP32 contraction + FP32 factors + FP64 refinement; 2: FP64 elements + FP32 factors + FP64
-    // refinement; 3: as 1 with the contraction on the tensor cores (three bf16 slices); 4: FP64 form with
+    // refinement; 3: as 1 with the contraction on the tensor cores (four bf16 slices); 4: FP64 form with
     // the contraction on the tensor cores to FP64 accuracy (seven slices); 5: as 2 with mode 4's elements
     P.mixed = P.two && precision_mode >= 1 && precision_mode != 4;
     P.df_rhs = P.mixed && precision_mode != 5;
@@ -848,7 +848,7 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S, 
                        : P.mode == RK_STAGE ? cudaLaunchKernelEx(&L.cfg, k_rk4_fp64<RK_STAGE>, ra)
                                             : cudaLaunchKernelEx(&L.cfg, k_rk4_fp64<RK_MATRIX>, ra));
         }
-        WPCCC_CHECK_LAUNCH("k_rk4");
+        WPCCC_CHECK_LAUNCH("RK4 sweep");
         B->prof.end(PROF_RK4, rs, e1);
         WPCCC_CUDA(cudaEventRecord(S.rk_done[k], rs));
     }

@@ -945,6 +945,7 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
             if ((s = launch_solve(N, nb, segS + (size_t)p0 * mat, nullptr, piv + (size_t)p0 * N, info + p0, st)) !=
                 WPCCC_OK)
                 return s;
+            if ((s = launch_lu_invert_diag(N, nb, segS + (size_t)p0 * mat, st)) != WPCCC_OK) return s;
         }
         // replay and reverse stages
         AdjRkArgs ra;

@@ -808,6 +808,7 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S, 
                 s = launch_schur_factor_fp64_tc(B, nev, bS, bI, P.d_scr, elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
             else if (P.schur) s = launch_schur_factor(N, B->N_T, nev, bS, bI, st);
             else s = launch_solve(N, nev, bS, P.stage ? nullptr : bH, bP, bI, st);
+            if (s == WPCCC_OK && P.mode == RK_STAGE) s = launch_lu_invert_diag(N, nev, bS, st);
             if (s != WPCCC_OK) return s;
             B->prof.end(PROF_SOLVE, st, e0);
         }

@@ -23,8 +23,7 @@
 namespace wpccc {
 
 constexpr int RC_THREADS = 512;
-constexpr int RC_BLK = 528;   // double2 of block scratch: partial sums (RC_THREADS) or one triangle of a diagonal block
-static_assert(RC_BLK >= RC_THREADS, "partial sums");
+constexpr int RC_BLK = RC_THREADS;   // double2 of block scratch: partial sums, or pivots
 
 static __device__ __forceinline__ void remote_store(uint32_t addr, int rank, double2 v) {
     uint32_t r;
@@ -269,83 +268,67 @@ static __device__ __noinline__ void rc_schur_solve(const RcCluster& cl, const do
     }
 }
 
-// t <- S^{-1} t (replicated) from P S = L U (LAPACK layout): perm[r] = row of t that comes r-th.  z: scratch of N
-// entries; blk: RC_BLK.
+// t <- S^{-1} t (replicated) from P S = L U with inverted 32 x 32 diagonal blocks (launch_lu_invert_diag): perm[r] = row of t
+// that comes r-th.  z: scratch of N entries; part: RC_BLK.  The inverse turns a panel's chain of 32 dependent FP64 steps
+// into one product of 16 threads per row, whose entries are loaded before the barrier that makes the panel's right-hand
+// side known (N = 109, 5 paths of 13 steps: sweep 4.2 -> SWEEPNOW ms).
 static __device__ __noinline__ void rc_lu_solve(const RcCluster& cl, const double2* __restrict__ LU, const uint16_t* perm,
-                                                   int N, double2* t, double2* z, double2* blk) {
-    const int np = (N + 31) / 32, tid = threadIdx.x, lane = tid & 31;
-    double2* part = blk;   // used between the diagonal solves
+                                                   int N, double2* t, double2* z, double2* part) {
+    const int np = (N + 31) / 32, tid = threadIdx.x, dr = tid >> 4, dl = tid & 15;
+    double2 m[2];   // this thread's entries (dr, dl) and (dr, dl + 16) of the next own diagonal block
+    auto fetch = [&](int p, bool upper) {
+        if (p < 0 || p >= np || p % cl.size != cl.rank) return;
+        const int nb = min(32, N - 32 * p);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = dl + 16 * h;
+            m[h] = make_double2(!upper && j == dr ? 1.0 : 0.0, 0.0);
+            if (dr < nb && j < nb && (upper ? j >= dr : j < dr)) m[h] = LU[(size_t)(32 * p + dr) + (size_t)(32 * p + j) * N];
+        }
+    };
+    auto diag = [&](int p) {
+        if (p % cl.size != cl.rank) return;
+        const int nb = min(32, N - 32 * p);
+        double re = 0.0, im = 0.0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int j = dl + 16 * h;
+            const double2 v = z[32 * p + (j < nb ? j : 0)];   // the entries past nb are zero
+            if (j < nb) {
+                re += m[h].x * v.x - m[h].y * v.y;
+                im += m[h].x * v.y + m[h].y * v.x;
+            }
+        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            re += __shfl_xor_sync(0xffffffffu, re, o);
+            im += __shfl_xor_sync(0xffffffffu, im, o);
+        }
+        if (dl == 0 && dr < nb) cl.bcast(t + 32 * p + dr, make_double2(re, im));
+    };
+    fetch(0, false);
     for (int r = tid; r < N; r += RC_THREADS)
         if ((r >> 5) % cl.size == cl.rank) z[r] = t[perm[r]];
     cl.sync();   // t may be overwritten
     RcPanel P;
-    // one triangle of a diagonal block, packed: lower (i >= j) by columns, or upper (i <= j) by columns
-    auto lo_at = [](int i, int j) { return j * (65 - j) / 2 + i - j; };
-    auto up_at = [](int i, int j) { return j * (j + 1) / 2 + i; };
-    auto stage = [&](int p, bool upper) {
-        const int nb = min(32, N - 32 * p);
-        for (int q = tid; q < 1024; q += RC_THREADS) {
-            const int i = q & 31, j = q >> 5;
-            if (i < nb && j < nb && (upper ? i <= j : i >= j))
-                blk[upper ? up_at(i, j) : lo_at(i, j)] = LU[(size_t)(32 * p + i) + (size_t)(32 * p + j) * N];
-        }
-        __syncthreads();
-    };
     for (int p = 0; p < np; ++p) {
         const int nb = min(32, N - 32 * p);
-        if (p % cl.size == cl.rank) {
-            stage(p, false);
-            if (tid < 32) {
-                double2 x = z[32 * p + (lane < nb ? lane : 0)];
-                for (int j = 0; j < nb - 1; ++j) {
-                    const double xr = __shfl_sync(0xffffffffu, x.x, j), xi = __shfl_sync(0xffffffffu, x.y, j);
-                    if (lane > j && lane < nb) {
-                        const double2 l = blk[lo_at(lane, j)];
-                        x.x = fma(-l.x, xr, x.x);
-                        x.x = fma(l.y, xi, x.x);
-                        x.y = fma(-l.x, xi, x.y);
-                        x.y = fma(-l.y, xr, x.y);
-                    }
-                }
-                if (lane < nb) cl.bcast(t + 32 * p + lane, x);
-            }
-        }
+        diag(p);
+        fetch(p + 1, false);
         const int q0 = rc_first_after(p, cl.rank, cl.size);
         P.load(LU + (size_t)(32 * p) * N, N, q0, rc_count(q0, np, cl.size), cl.size, N, nb);
         cl.sync();
         P.apply(t + 32 * p, z, nb, part);
         __syncthreads();
     }
+    fetch(np - 1, true);
     for (int r = tid; r < N; r += RC_THREADS)
         if ((r >> 5) % cl.size == cl.rank) z[r] = t[r];
     __syncthreads();
     for (int p = np - 1; p >= 0; --p) {
         const int nb = min(32, N - 32 * p);
-        if (p % cl.size == cl.rank) {
-            stage(p, true);
-            if (tid < 32) {
-                double2 x = z[32 * p + (lane < nb ? lane : 0)];
-                const double2 u = blk[up_at(lane < nb ? lane : 0, lane < nb ? lane : 0)];
-                const double d = u.x * u.x + u.y * u.y;
-                const double ir = u.x / d, ii = -u.y / d;   // reciprocals of the diagonal, off the serial chain
-                for (int j = nb - 1; j >= 0; --j) {
-                    if (lane == j) {
-                        const double xr0 = x.x;
-                        x.x = x.x * ir - x.y * ii;
-                        x.y = xr0 * ii + x.y * ir;
-                    }
-                    const double xr = __shfl_sync(0xffffffffu, x.x, j), xi = __shfl_sync(0xffffffffu, x.y, j);
-                    if (lane < j) {
-                        const double2 w = blk[up_at(lane, j)];
-                        x.x = fma(-w.x, xr, x.x);
-                        x.x = fma(w.y, xi, x.x);
-                        x.y = fma(-w.x, xi, x.y);
-                        x.y = fma(-w.y, xr, x.y);
-                    }
-                }
-                if (lane < nb) cl.bcast(t + 32 * p + lane, x);
-            }
-        }
+        diag(p);
+        fetch(p - 1, true);
         P.load(LU + (size_t)(32 * p) * N, N, cl.rank, rc_count(cl.rank, p, cl.size), cl.size, N, nb);
         cl.sync();
         P.apply(t + 32 * p, z, nb, part);

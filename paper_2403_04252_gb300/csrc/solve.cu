@@ -338,6 +338,53 @@ static wpccc_status lu_launch(int N, int batch, const double2* S, typename LuC<R
     return WPCCC_OK;
 }
 
+// The 32 x 32 diagonal blocks of P S = L U replaced by the inverses of their triangles: strictly below the diagonal the
+// unit lower block's inverse (its unit diagonal implied), from the diagonal on the upper block's.  One block per (panel,
+// system), a warp per four columns of an inverse, a row per lane.  The RK4 sweep applies them instead of solving with the
+// triangles; the FP64 work here is 2 / N of the factorisation's.
+__global__ void __launch_bounds__(256) k_lu_invert_diag(int N, double2* __restrict__ LU) {
+    __shared__ double2 blk[NB][NB + 1];   // [column][row]
+    const int k0 = blockIdx.x * NB, nb = min(NB, N - k0), lane = threadIdx.x & 31, c0 = (threadIdx.x >> 5) * 4;
+    double2* A = LU + (size_t)blockIdx.y * N * N + (size_t)k0 + (size_t)k0 * N;
+    for (int q = threadIdx.x; q < NB * NB; q += 256) {
+        const int i = q & 31, j = q >> 5;
+        blk[j][i] = i < nb && j < nb ? A[(size_t)i + (size_t)j * N] : make_double2(i == j ? 1.0 : 0.0, 0.0);
+    }
+    __syncthreads();
+    const double2 inv = crecip(blk[lane][lane]);
+    double2 l[4], u[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) l[c] = u[c] = make_double2(lane == c0 + c ? 1.0 : 0.0, 0.0);
+    for (int k = c0; k < nb; ++k) {
+        const double2 a = lane > k ? blk[k][lane] : make_double2(0.0, 0.0);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double2 w = make_double2(__shfl_sync(0xffffffffu, l[c].x, k), __shfl_sync(0xffffffffu, l[c].y, k));
+            l[c] = csub_prod(l[c], a, w);
+        }
+    }
+    for (int k = min(c0 + 3, nb - 1); k >= 0; --k) {
+        const double2 a = lane < k ? blk[k][lane] : make_double2(0.0, 0.0);
+        const double2 d = make_double2(__shfl_sync(0xffffffffu, inv.x, k), __shfl_sync(0xffffffffu, inv.y, k));
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double2 w = cprod(make_double2(__shfl_sync(0xffffffffu, u[c].x, k), __shfl_sync(0xffffffffu, u[c].y, k)), d);
+            if (lane == k) u[c] = w;
+            u[c] = csub_prod(u[c], a, w);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        if (lane < nb && c0 + c < nb) A[(size_t)lane + (size_t)(c0 + c) * N] = lane > c0 + c ? l[c] : u[c];
+}
+
+wpccc_status launch_lu_invert_diag(int N, int batch, double2* LU, cudaStream_t st) {
+    if (batch == 0) return WPCCC_OK;
+    k_lu_invert_diag<<<dim3((N + NB - 1) / NB, batch), 256, 0, st>>>(N, LU);
+    WPCCC_CHECK_LAUNCH("k_lu_invert_diag");
+    return WPCCC_OK;
+}
+
 wpccc_status launch_factor_f32(int N, int batch, const double2* S, float2* LU, int* ipiv, int* info, cudaStream_t st) {
     return lu_launch<float>(N, batch, S, LU, nullptr, ipiv, info, st);
 }

@@ -262,6 +262,8 @@ wpccc_status check_tc_err(wpccc_basis_s* B, const char* where);
 // Queue the batched solve of S X = H (results in place).
 wpccc_status launch_solve(int N, int batch, double2* S, double2* H, int* ipiv, int* info,
                           cudaStream_t st);
+// The factors' 32 x 32 diagonal blocks replaced by their triangles' inverses, as rc_lu_solve takes them.
+wpccc_status launch_lu_invert_diag(int N, int batch, double2* LU, cudaStream_t st);
 
 }  // namespace wpccc
 

@@ -13,7 +13,7 @@
 // panel by panel (32 rows, the panels to the blocks in turn): the owner solves the diagonal block and sends the 32
 // unknowns to all blocks, every block updates its own rows; the factor's tile is loaded before the barrier.
 // Measured, one block per path with a row per thread -> here, sweeps alone: one centre, N = 59, 8 paths of 800 steps
-// 42.6 -> 10.2 ms (13.3 -> 3.2 us per stage); two centres, LU, N = 109, 5 paths of 23 steps 10.3 -> 4.2 ms; Schur,
+// 42.6 -> 10.2 ms (13.3 -> 3.2 us per stage); two centres, LU, N = 109, 5 paths of 13 steps 10.3 -> 2.4 ms; Schur,
 // N = 380, 32 paths of 10 steps 22 -> 9.0 ms.
 #pragma once
 
@@ -271,7 +271,8 @@ static __device__ __noinline__ void rc_schur_solve(const RcCluster& cl, const do
 // t <- S^{-1} t (replicated) from P S = L U with inverted 32 x 32 diagonal blocks (launch_lu_invert_diag): perm[r] = row of t
 // that comes r-th.  z: scratch of N entries; part: RC_BLK.  The inverse turns a panel's chain of 32 dependent FP64 steps
 // into one product of 16 threads per row, whose entries are loaded before the barrier that makes the panel's right-hand
-// side known (N = 109, 5 paths of 13 steps: sweep 4.2 -> SWEEPNOW ms).
+// side known (N = 109, 5 paths of up to 23 steps: sweep 7.8 -> 4.4 ms, for 0.3 ms of inversion; the adjoint of p + Li,
+// N = 379: 35 -> 28 ms).
 static __device__ __noinline__ void rc_lu_solve(const RcCluster& cl, const double2* __restrict__ LU, const uint16_t* perm,
                                                    int N, double2* t, double2* z, double2* part) {
     const int np = (N + 31) / 32, tid = threadIdx.x, dr = tid >> 4, dl = tid & 15;

@@ -108,22 +108,29 @@ __device__ __forceinline__ C2 csub_prod(C2 x, C2 l, C2 u) {
     return x;
 }
 
+// Order of |re| + |im| as an integer: the bits of a number >= 0; -1 for NaN, which is never a pivot while there is another.
+__device__ __forceinline__ long long pivot_key(double v) { return v == v ? __double_as_longlong(v) : -1; }
+__device__ __forceinline__ long long pivot_key(float v) { return v == v ? (long long)__float_as_int(v) : -1; }
+
 // Unblocked LU with partial pivoting of the panel's nb columns from k0 (rows k0..N-1), by one block; pivots (1-based)
-// to ipiv, the first zero pivot to *info.
+// to ipiv, the first zero pivot to *info.  An FP64 instruction holds its quarter of the SM's pipe for 64 cycles per warp, so
+// the search for the pivot compares integers, and two lanes of one warp form the pivot's reciprocal (a division is some 30
+// instructions) while the other warps interchange the rows.  Against the division in every warp and FP64 comparisons:
+// N = 109, 200 factorisations 2.9 -> 2.4 ms; N = 380 with N right-hand sides, 24 systems 24.8 -> 24.2 ms.
 template <typename C2>
 __device__ void panel_lu(C2* __restrict__ A, int N, int k0, int nb, int* __restrict__ ipiv, int* info) {
     using R = decltype(C2().x);
-    __shared__ R red_v[LU_THREADS / 32];
+    __shared__ long long red_v[LU_THREADS / 32];
     __shared__ int red_i[LU_THREADS / 32];
-    __shared__ int s_piv;
+    __shared__ R s_inv[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int kk = 0; kk < nb; ++kk) {
         const int k = k0 + kk;
-        R best = R(-1);
+        long long best = -1;
         int bi = N;
         for (int i = k + tid; i < N; i += LU_THREADS) {
             const C2 a = A[(size_t)i + (size_t)k * N];
-            const R v = fabs(a.x) + fabs(a.y);
+            const long long v = pivot_key(fabs(a.x) + fabs(a.y));
             if (v > best) {
                 best = v;
                 bi = i;
@@ -131,7 +138,7 @@ __device__ void panel_lu(C2* __restrict__ A, int N, int k0, int nb, int* __restr
         }
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
-            const R ov = __shfl_down_sync(0xffffffffu, best, off);
+            const long long ov = __shfl_down_sync(0xffffffffu, best, off);
             const int oi = __shfl_down_sync(0xffffffffu, bi, off);
             if (ov > best || (ov == best && oi < bi)) {
                 best = ov;
@@ -143,31 +150,37 @@ __device__ void panel_lu(C2* __restrict__ A, int N, int k0, int nb, int* __restr
             red_i[warp] = bi;
         }
         __syncthreads();
+        best = red_v[0];
+        bi = red_i[0];
+        for (int w = 1; w < LU_THREADS / 32; ++w)
+            if (red_v[w] > best || (red_v[w] == best && red_i[w] < bi)) {
+                best = red_v[w];
+                bi = red_i[w];
+            }
+        const int p = bi < N ? bi : k;
         if (tid == 0) {
-            R bv = red_v[0];
-            int bix = red_i[0];
-            for (int w = 1; w < LU_THREADS / 32; ++w)
-                if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
-                    bv = red_v[w];
-                    bix = red_i[w];
-                }
-            if (bix >= N) bix = k;
-            s_piv = bix;
-            ipiv[k] = bix + 1;
-            if (bv == R(0) && *info == 0) *info = k + 1;
+            ipiv[k] = p + 1;
+            if (best == 0 && *info == 0) *info = k + 1;
         }
-        __syncthreads();
-        const int p = s_piv;
-        if (p != k && tid < nb) {
-            const int c = k0 + tid;
+        // the first warp: the pivot's reciprocal and this column's interchange; the next: the other columns'
+        if (tid < 2) {
+            const C2 piv = A[(size_t)p + (size_t)k * N];
+            const R d = piv.x * piv.x + piv.y * piv.y;
+            s_inv[tid] = (tid == 0 ? piv.x : -piv.y) / d;
+            __syncwarp(3u);
+            if (tid == 0 && p != k) {
+                A[(size_t)p + (size_t)k * N] = A[(size_t)k + (size_t)k * N];
+                A[(size_t)k + (size_t)k * N] = piv;
+            }
+        } else if (p != k && warp == 1 && lane < nb && lane != kk) {
+            const int c = k0 + lane;
             const C2 t = A[(size_t)k + (size_t)c * N];
             A[(size_t)k + (size_t)c * N] = A[(size_t)p + (size_t)c * N];
             A[(size_t)p + (size_t)c * N] = t;
         }
         __syncthreads();
-        const C2 piv = A[(size_t)k + (size_t)k * N];
-        if (piv.x != R(0) || piv.y != R(0)) {
-            const C2 inv = crecip(piv);
+        if (best != 0) {
+            const C2 inv = C2{s_inv[0], s_inv[1]};
             for (int i = k + 1 + tid; i < N; i += LU_THREADS) {
                 C2* q = A + (size_t)i + (size_t)k * N;
                 *q = cprod(*q, inv);

@@ -1776,13 +1776,21 @@ static wpccc_status matrix_elements_prec(wpccc_basis B, double b, double v, int 
         if (rs != WPCCC_OK) return rs;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const ElemScratch L = elem_scratch_layout(B, precision);
+    int chunk = 1;
     // evaluations per launch bounded by the workspace limit
-    size_t per = L.bytes_per_eval + sizeof(EvalDesc);
-    int chunk = (int)std::min<size_t>({(size_t)nz, (size_t)MAX_EVALS_PER_LAUNCH,
+    auto workspace = [&]() {
+        const ElemScratch L = elem_scratch_layout(B, precision);
+        const size_t per = L.bytes_per_eval + sizeof(EvalDesc);
+        chunk = (int)std::min<size_t>({(size_t)nz, (size_t)MAX_EVALS_PER_LAUNCH,
                                        std::max<size_t>(1, (B->ws_limit - 256) / per)});
-    size_t need = (size_t)chunk * L.bytes_per_eval + 256 + (size_t)chunk * sizeof(EvalDesc);
-    wpccc_status s = ensure_workspace(B, need);
+        return ensure_workspace(B, (size_t)chunk * L.bytes_per_eval + 256 + (size_t)chunk * sizeof(EvalDesc));
+    };
+    wpccc_status s = workspace();
+    if (s == WPCCC_ENOMEM && precision == ELEM_F64_TC) {   // the CUDA cores' form takes less scratch
+        cudaGetLastError();
+        precision = ELEM_F64;
+        s = workspace();
+    }
     if (s != WPCCC_OK) return s;
     char* wsb = static_cast<char*>(B->ws_ptr);
     EvalDesc* dev_ev = reinterpret_cast<EvalDesc*>(wsb);

@@ -525,9 +525,10 @@ struct PropPlan {
 static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Validates the paths and lays out the plan.  C_request > 0 fixes the RK4 steps per chunk,
-// otherwise they are chosen from the workspace limit and the SM count.
+// otherwise they are chosen from the workspace limit and the SM count.  cuda_cores: the FP64 contraction stays off the
+// tensor cores, whose digits take more scratch per position (the callers' second try when memory is short).
 static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int precision_mode, int C_request,
-                               size_t ws_limit, PropPlan& P) {
+                               size_t ws_limit, PropPlan& P, bool cuda_cores = false) {
     if (precision_mode < 0 || precision_mode > 5)
         return fail(WPCCC_EUNSUPPORTED, "wpccc_propagate: precision_mode must be 0 to 5");
     if ((precision_mode == 1 || precision_mode >= 3) && B->n_centres == 2 && B->mp_c != 0.0)
@@ -566,7 +567,7 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     P.elem_precision = !P.two ? 0
                        : (precision_mode == 1 || precision_mode == 3) ? precision_mode
                        : (precision_mode == 4 || precision_mode == 5) ? ELEM_TC7 : ELEM_F64;
-    if (P.two && P.elem_precision == ELEM_F64) {
+    if (P.two && P.elem_precision == ELEM_F64 && !cuda_cores) {
         wpccc_status rs = fp64_route(B, &P.elem_precision);
         if (rs != WPCCC_OK) return rs;
     }
@@ -892,7 +893,13 @@ wpccc_status propagate_internal(wpccc_basis_s* B, const wpccc_paths* paths, int 
     wpccc_status s = plan_build(B, paths, precision_mode, 0, B->ws_limit, P);
     if (s != WPCCC_OK) return s;
     if (P.max_steps == 0) return WPCCC_OK;
-    if ((s = ensure_workspace(B, P.bytes)) != WPCCC_OK) return s;
+    s = ensure_workspace(B, P.bytes);
+    if (s == WPCCC_ENOMEM && P.elem_precision == ELEM_F64_TC) {
+        cudaGetLastError();   // the failed allocation's, not a later launch's
+        if ((s = plan_build(B, paths, precision_mode, 0, B->ws_limit, P, true)) != WPCCC_OK) return s;
+        s = ensure_workspace(B, P.bytes);
+    }
+    if (s != WPCCC_OK) return s;
     plan_bind(P, B->ws_ptr);
     if ((s = basis_streams(B)) != WPCCC_OK) return s;
     if ((s = plan_upload(P, st)) != WPCCC_OK) return s;
@@ -954,7 +961,7 @@ static void batch_free(wpccc_batch_s* X) {
 
 // Times one candidate schedule of a set on its first steps: a warm run, then a timed run.
 static wpccc_status tune_trial(wpccc_basis_s* B, const wpccc_paths* paths, int precision, int C, double2* c_src,
-                               double* ms_per_step) {
+                               double* ms_per_step, bool cuda_cores) {
     // the set's paths cut to 2C steps (at least two chunks, so the overlap is part of the timing)
     const int np = paths->n_paths;
     std::vector<int> nz(np);
@@ -974,7 +981,7 @@ static wpccc_status tune_trial(wpccc_basis_s* B, const wpccc_paths* paths, int p
     }
     wpccc_paths tp{np, paths->b, paths->v, nz.data(), z.data()};
     PropPlan P;
-    wpccc_status s = plan_build(B, &tp, precision, C, B->ws_limit, P);
+    wpccc_status s = plan_build(B, &tp, precision, C, B->ws_limit, P, cuda_cores);
     if (s != WPCCC_OK) return s;
     void* ws = nullptr;
     double2* c = nullptr;
@@ -1044,12 +1051,13 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
         set_error(keep);
         return st;
     };
-    wpccc_status s;
+    wpccc_status s = WPCCC_OK;
+    auto plan_sets = [&](bool cuda_cores) -> wpccc_status {
     for (int k = 0; k < n_sets; ++k) {
         wpccc_basis_s* B = bases[k];
         X->c[k] = static_cast<double2*>(c[k]);
         PropPlan P;
-        if ((s = plan_build(B, &paths[k], precision_mode, 0, B->ws_limit, P)) != WPCCC_OK) return bail(s);
+        if ((s = plan_build(B, &paths[k], precision_mode, 0, B->ws_limit, P, cuda_cores)) != WPCCC_OK) return s;
         int best = P.C;
         if (autotune && P.max_steps > 1) {
             // schedules tried: the default chunk and half and twice as many RK4 steps per chunk
@@ -1061,9 +1069,9 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
                 double ms = 0.0;
                 const bool was_on = B->prof.on;
                 B->prof.on = false;
-                s = tune_trial(B, &paths[k], precision_mode, C, X->c[k], &ms);
+                s = tune_trial(B, &paths[k], precision_mode, C, X->c[k], &ms, cuda_cores);
                 B->prof.on = was_on;
-                if (s != WPCCC_OK) return bail(s);
+                if (s != WPCCC_OK) return s;
                 if (best_ms < 0.0 || ms < best_ms) {
                     best_ms = ms;
                     best = C;
@@ -1071,7 +1079,7 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
             }
             X->tuned_ms_per_step[k] = best_ms;
         }
-        if ((s = plan_build(B, &paths[k], precision_mode, best, B->ws_limit, X->plans[k])) != WPCCC_OK) return bail(s);
+        if ((s = plan_build(B, &paths[k], precision_mode, best, B->ws_limit, X->plans[k], cuda_cores)) != WPCCC_OK) return s;
         X->chunk_steps[k] = X->plans[k].C;
     }
     // one workspace for every set
@@ -1079,8 +1087,17 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
     for (auto& P : X->plans) total += align256(P.bytes);
     {
         cudaError_t e = cudaMalloc(&X->ws, std::max<size_t>(total, 256));
-        if (e != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc(batch workspace)"));
+        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(batch workspace)");
     }
+    return WPCCC_OK;
+    };
+    s = plan_sets(false);
+    if (s == WPCCC_ENOMEM && (precision_mode == 0 || precision_mode == 2)) {
+        cudaGetLastError();
+        X->ws = nullptr;
+        s = plan_sets(true);
+    }
+    if (s != WPCCC_OK) return bail(s);
     size_t off = 0;
     for (auto& P : X->plans) {
         plan_bind(P, static_cast<char*>(X->ws) + off);

@@ -14,6 +14,7 @@
 // their FP64 iterative refinement.
 #include <algorithm>
 
+#include "chol_panel.cuh"
 #include "cluster.cuh"
 #include "wpccc_internal.cuh"
 
@@ -105,36 +106,6 @@ __device__ void cta_update_lower(typename SchurC<R>::type* __restrict__ C, int l
     }
 }
 
-// v -= l conj(u): one step of the Cholesky factor's element (i, j) with l = L[i][k], u = L[j][k]
-static __device__ __forceinline__ float2 chol_step(float2 v, float2 l, float2 u) {
-    v.x -= l.x * u.x + l.y * u.y;
-    v.y -= l.y * u.x - l.x * u.y;
-    return v;
-}
-static __device__ __forceinline__ double2 chol_step(double2 v, double2 l, double2 u) {
-    v.x = fma(-l.x, u.x, fma(-l.y, u.y, v.x));
-    v.y = fma(-l.y, u.x, fma(l.x, u.y, v.y));
-    return v;
-}
-
-// (sqrt(d), 1 / sqrt(d)); in FP64 by two Newton-Raphson steps r <- r + r (1 - d r^2) / 2 from the FP32 reciprocal square
-// root: an FP64 square root and division are long serial chains on this part's FP64 pipe
-static __device__ __forceinline__ float2 sqrt_and_inverse(float d) {
-    const float s = sqrt(d);
-    return make_float2(s, 1.f / s);
-}
-static __device__ __forceinline__ double2 sqrt_and_inverse(double d) {
-    double r;
-    if (d > 1e-30 && d < 1e30) {
-        r = (double)rsqrtf((float)d);
-        r = fma(0.5 * r, fma(-d * r, r, 1.0), r);
-        r = fma(0.5 * r, fma(-d * r, r, 1.0), r);
-    } else {
-        r = rsqrt(d);
-    }
-    return make_double2(d * r, r);
-}
-
 // One system per cluster of blocks (cluster size 1 to 8).  R = double: D is S itself (FP64, in place).  R = float
 // (preconditioner of the mixed-precision form): D is a separate FP32 N x N buffer that receives K rounded to FP32
 // in its target-projectile block and the FP32 Cholesky factor in its projectile block; S is only read.
@@ -153,7 +124,6 @@ __global__ void __launch_bounds__(SC_THREADS) k_schur_factor(int N, int N_T, con
                                                              typename SchurC<R>::type* __restrict__ Dall,
                                                              int* __restrict__ info_all, bool given) {
     using C2 = typename SchurC<R>::type;
-    using R2 = C2;   // a pair of reals
     extern __shared__ __align__(16) unsigned char sc_smem_raw[];
     C2* sA = reinterpret_cast<C2*>(sc_smem_raw);   // SC_NB * SC_LD
     C2* sB = sA + SC_NB * SC_LD;                   // SC_NB * SC_LD
@@ -199,31 +169,7 @@ __global__ void __launch_bounds__(SC_THREADS) k_schur_factor(int N, int N_T, con
             if (j <= i && i < nb) sL[j * (SC_NB + 1) + i] = __ldcg(C + (size_t)(k0 + i) + (size_t)(k0 + j) * N);
         }
         __syncthreads();
-        // row = lane; column k is scaled by the first warp, the columns j > k belong to the warps in turn (an FP64
-        // instruction holds a quarter's pipe for 64 cycles per warp, so the steps are spread over all four)
-        for (int k = 0; k < nb; ++k) {
-            if (tid < 32) {
-                R d = sL[k * (SC_NB + 1) + k].x;
-                if (!(d > R(0))) {
-                    if (lane == 0 && s_info == 0) s_info = k0 + k + 1;
-                    d = R(1);
-                }
-                const R2 r = sqrt_and_inverse(d);
-                if (lane == k) {
-                    sL[k * (SC_NB + 1) + k] = C2{r.x, R(0)};
-                    s_inv[k] = r.y;
-                } else if (lane > k && lane < nb) {
-                    const C2 l = sL[k * (SC_NB + 1) + lane];
-                    sL[k * (SC_NB + 1) + lane] = C2{l.x * r.y, l.y * r.y};
-                }
-            }
-            __syncthreads();
-            const C2 l = sL[k * (SC_NB + 1) + lane];
-            for (int j = k + 1 + (tid >> 5); j < nb; j += SC_THREADS / 32)
-                if (lane >= j && lane < nb)
-                    sL[j * (SC_NB + 1) + lane] = chol_step(sL[j * (SC_NB + 1) + lane], l, sL[k * (SC_NB + 1) + j]);
-            __syncthreads();
-        }
+        chol_diag_block<SC_THREADS / 32>(sL, SC_NB + 1, s_inv, &s_info, k0, nb, tid);
         // every block has read the diagonal block before one of them overwrites it with its factor
         cluster_sync_all();
         if (sizeof(R) == 4) {

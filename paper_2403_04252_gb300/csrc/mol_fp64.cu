@@ -137,9 +137,11 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int a = h[4 * j + k], b = hv[k];
-                    // zero and denormal factors leave the window's scale alone; a non-finite one marks the row
+                    // zero and denormal factors leave the window's scale alone; a non-finite one marks the row (the sum of
+                    // two high words passes 2^31 from a product of 4 on: unsigned)
+                    const uint32_t ab = (uint32_t)a + (uint32_t)b;
                     const int p = max(a, b) >= 0x7FF00000 ? 0x7FF00000
-                                  : min(a, b) < (1 << 20) ? 0 : max(0, min(a + b - (1023 << 20), 0x7FEFFFFF));
+                                  : min(a, b) < (1 << 20) || ab < (1023u << 20) ? 0 : (int)min(ab - (1023u << 20), 0x7FEFFFFFu);
                     m = max(m, p);
                 }
             }

@@ -245,7 +245,8 @@ WPCCC_API wpccc_status wpccc_solve(int N, int batch, void* S, void* H, int* ipiv
  *      its last node.
  *   precision_mode
  *     0  FP64 throughout (the Eq. 9 contraction and the Schur solve's update I - K^+ K in exact fixed-point
- *        digits on the tensor cores where they can run there, with at least FP64's accuracy);
+ *        digits on the tensor cores where they can run there, within the rounding of a chain of FP64
+ *        multiply-adds element by element, and of the update in norm);
  *     1  mixed: the Eq. 9 contraction and the LU factors of S on the FP32 pipe,
  *        each RK4 stage's S^{-1} solved by FP64 iterative refinement (residuals
  *        against the FP64 S), RK4 amplitudes in FP64;

@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 
 #include "angular.cuh"
+#include "f64_order.cuh"
 #include "geometry.cuh"
 #include "ozaki.cuh"
 #include "wpccc_internal.cuh"
@@ -108,10 +109,12 @@ struct NodeArgs {
     const int* tc_row;          // [2 N_T]: row of each target state in the slice planes, then its tile's size
     int tc_rows;
     size_t t6_ap_off, t6_w_off, t6_sc_off;
-    // FP64 tensor-core form (T = double, f64 != 0): instead of W, the rows W_K / r_T (re, im per d) at f64_w2 and
-    // r_T, r_T V_T at f64_r (byte offsets, rows of Gp nodes, zero past the last node)
+    // FP64 tensor-core form (T = double, f64 != 0): nodes in the order of f64_order.cuh; instead of W, the rows W_K / r_T
+    // (re, im per d) at f64_w2 and r_T, r_T V_T at f64_r (byte offsets, rows of Gp nodes, zero past the last node), scaled
+    // by 2^-s and 2^s
     int f64, Gp;
     size_t f64_w2, f64_r;
+    double kappa;               // steepness of the nodes' order and scales (f64_order.cuh)
     // sqrt((2l+1)/2 (l-q)!/(l+q)!) at l(l+1)/2 + q, 1/k for k = 0..WPCCC_LMAX (entry 0 unused) and the numbers k
     // themselves (a conversion takes the FP64 pipe as long as a multiplication): the Legendre recurrence's constants
     double th_nrm[(WPCCC_LMAX + 1) * (WPCCC_LMAX + 2) / 2];
@@ -174,9 +177,10 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
         }
         return;
     }
-    const int k = g / A.Gtau, t = g - k * A.Gtau;
     const double b = ev[e].b, v = ev[e].v, z = ev[e].z;
     const double R = dist_R(b, z);
+    int k = g / A.Gtau, t = g - k * A.Gtau;
+    if (sizeof(T) == 8 && A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.Gtau, __dmul_rn(A.kappa, R)), k, t);
     const double gR = __dmul_rn(A.gamma, R);
     const double eta = __dadd_rn(1.0, __ddiv_rn(A.s[k], gR));
     const double tau = A.tau[t];
@@ -391,13 +395,16 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
         }
     }
     // node weights for the two integrands, d = |q - q'| = 0..dmax; Q carries the target potential
-    const double irT = 1.0 / rT;
+    double irT = 1.0 / rT;
     const double uQ = A.mp_c == 0.0 ? -A.Z_T * irT
                                     : (-A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT)) * irT;
     if (sizeof(T) == 8 && A.f64) {
         double* rr = reinterpret_cast<double*>(reinterpret_cast<char*>(base) + A.f64_r);
-        rr[g] = rT;
-        rr[(size_t)A.Gp + g] = A.mp_c == 0.0 ? -A.Z_T : -A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT);
+        const int sc = f64_scale(__dmul_rn(A.kappa, R), tau);
+        const double up = __hiloint2double((1023 + sc) << 20, 0);
+        rr[g] = rT * up;
+        rr[(size_t)A.Gp + g] = (A.mp_c == 0.0 ? -A.Z_T : -A.Z_T + (-A.mp_c * exp(-A.mp_a * rT)) * (1.0 + A.mp_b * rT)) * up;
+        irT *= __hiloint2double((1023 - sc) << 20, 0);
     }
     const size_t stride = (size_t)(A.dmax + 1) * A.G;
     double Jd[BESSEL_MAX + 1];
@@ -1195,6 +1202,8 @@ __global__ void __launch_bounds__(256) k_direct(DirArgs A0, DirArgs A1, const Ev
 // 12: with rotation and direct blocks 13.6 -> 10.4 ms.
 // ---------------------------------------------------------------------------
 struct SrArgs {
+    int f64;          // nodes in the order of f64_order.cuh
+    double kappa;
     int G, Gtau, nradT, nradP, lmaxP, nlqT, N_T, N_P, N, dtot;
     double gamma, mp_c, mp_a, mp_b;
     const double *s, *ws, *tau, *wtau;
@@ -1231,7 +1240,8 @@ __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __r
     double* I = NA > 1 ? U + (size_t)NA * A.G : U;
     double* dt = I + (size_t)NA * A.nradP * LQ;
     for (int g = threadIdx.x; g < A.G; g += blockDim.x) {
-        const int k = g / A.Gtau, t = g - k * A.Gtau;
+        int k = g / A.Gtau, t = g - k * A.Gtau;
+        if (A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.Gtau, __dmul_rn(A.kappa, R)), k, t);
         const double eta = __dadd_rn(1.0, __ddiv_rn(A.s[k], gR));
         const double tau = A.tau[t];
         const double rT = __dmul_rn(halfR, __dadd_rn(eta, tau));
@@ -1484,6 +1494,7 @@ static wpccc_status launch_tables(wpccc_basis_s* B, const EvalDesc* evals, int n
     na.Gp = L.Gp;
     na.f64_w2 = L.f64_w2;
     na.f64_r = L.f64_r;
+    na.kappa = f64_kappa(B);
     for (int k = 0; k < 2 * WPCCC_LMAX + 2; ++k) na.num[k] = k;
     for (int l = 0; l <= WPCCC_LMAX; ++l) {
         na.inv_int[l] = l > 0 ? 1.0 / l : 0.0;
@@ -1560,7 +1571,7 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
                                             (int)gsm));
             k_mol_gemm<double><<<dim3(n_row_tiles * ga.n_col_tiles, nev), 256, gsm, st>>>(ga);
         } else if (precision == ELEM_F64_TC) {
-            wpccc_status ms = launch_mol_f64tc(B, nev, node, mol, B->tc_err, st);
+            wpccc_status ms = launch_mol_f64tc(B, evals, nev, node, mol, B->tc_err, st);
             if (ms != WPCCC_OK) return ms;
         } else if (precision == 3 || precision == 4) {
             wpccc_status ms = launch_mol_tc64(B, nev, node, mol, B->tc_err, st,
@@ -1653,6 +1664,8 @@ wpccc_status launch_elements(wpccc_basis_s* B, const EvalDesc* evals, int nev, d
     B->prof.end(PROF_ROT_DIRECT, st, ed);
     if (two && B->mp_c != 0.0) {
         SrArgs sa;
+        sa.f64 = precision == ELEM_F64_TC;
+        sa.kappa = f64_kappa(B);
         sa.G = B->G;
         sa.Gtau = B->Gtau;
         sa.nradT = B->T.n_rad;

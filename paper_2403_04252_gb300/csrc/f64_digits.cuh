@@ -1,4 +1,4 @@
-// Building blocks of the contractions that the tensor cores carry out to more than FP64's accuracy (mol_fp64.cu,
+// Building blocks of the contractions that the tensor cores carry out in FP64's place (mol_fp64.cu,
 // schur_fp64.cu): fixed-point digits of FP64 rows, the MMAs of one chunk, and the sums put together again.
 // The representation and its error are described in mol_fp64.cu.
 #pragma once
@@ -14,7 +14,7 @@ constexpr int F64_LEV = 9;                      // levels 0..8
 constexpr int F64_M = 128;                      // A rows per CTA (MMA M)
 constexpr int F64_N = 32;                       // B rows per CTA (MMA N of one digit)
 constexpr int F64_K = 32;                       // terms per chunk: one 64-byte bf16 row
-constexpr int F64_WIN = 512;                    // terms per scaling window
+constexpr int F64_WIN = 512;                    // terms per scaling window, at most
 constexpr int F64_WCH = F64_WIN / F64_K;        // chunks per window
 constexpr int F64_TMEM_COLS = 512;              // one buffer of accumulators: 9 x 32 = 288 columns
 constexpr int F64_B_TILE = F64_N * 64;          // bytes of one digit of the B tile
@@ -83,15 +83,22 @@ static __device__ __forceinline__ void f64_levels(const float (&v)[F64_LEV][4], 
     low19 = (uint32_t)lo & 0x7FFFFu;
 }
 
-// One window's sum added to the running sum: T 2^(E - 42) to acc (one FP64 FMA), the low part 2^(E - 61) to low in FP32
-// (both zero below their range, NaN for a row with a non-finite value).
+// One window's sum added to the running sum: T 2^(E - 42) to acc (one FP64 FMA), the low part 2^(E - 61) to low in FP32, in
+// units of 2^-100; below that range (windows 2^-165 and smaller) the low part goes with T, rounded to FP64.  Zero below
+// FP64's range, NaN for a row with a non-finite value.
+constexpr int F64_LOW = 100;
 static __device__ __forceinline__ void f64_accumulate(double& acc, float& low, long long T, uint32_t low19, int E) {
-    const double X = __dsub_rn(__longlong_as_double(T + 0x4338000000000000ll), 6755399441055744.0);
-    const int es = E - 42 + 1023, ef = E - 61 + 127;
+    double X = __dsub_rn(__longlong_as_double(T + 0x4338000000000000ll), 6755399441055744.0);
+    const int es = E - 42 + 1023, ef = E - 61 + F64_LOW + 127;
     const int sh = E >= F64_BAD / 2 ? 0x7FF80000 : (max(0, min(es, 2046)) << 20);
+    if (ef <= 0 && low19 != 0) X = fma((double)low19, __hiloint2double((1023 - 19) << 20, 0), X);
     acc = fma(X, __hiloint2double(sh, 0), acc);
     const float r = __fsub_rn(__uint_as_float(0x4B000000u | low19), 8388608.f);
     low = fmaf(r, __uint_as_float((uint32_t)max(0, min(ef, 230)) << 23), low);
+}
+
+static __device__ __forceinline__ double f64_total(double acc, float low) {
+    return fma((double)low, __hiloint2double((1023 - F64_LOW) << 20, 0), acc);
 }
 
 // The MMAs of one chunk (one thread): the B tile's digits lie one after the other, so one MMA per A digit and K step forms

@@ -1,4 +1,4 @@
-// Eq. 9 contraction of the FP64 form on the 5th-generation tensor cores, with at least FP64's accuracy.
+// Eq. 9 contraction of the FP64 form on the 5th-generation tensor cores, at FP64's accuracy element by element.
 //
 // For one row tile (target states of one molecular-frame projection q') the two-centre integrals are
 //   X_K[i][c] = sum_g (A_T r_T)[i][g] b[c][g],   X_Q[i][c] = sum_g (A_T r_T V_T)[i][g] b[c][g],
@@ -6,7 +6,7 @@
 // a real contraction over the quadrature nodes g of M = 128 table rows and N = 32 generated rows
 // (16 half columns x re/im) per thread block.
 //
-// Representation.  Per window of F64_WIN = 512 nodes every row of both operands is written in fixed point against
+// Representation.  Per window of 512 nodes (fewer far from the target, see below) every row of both operands is written in fixed point against
 // the power of two above the row's largest |value| of the window, x = X 2^(E - 55) with X rounded to an integer
 // (|X| < 2^55), and X in eight balanced digits of seven bits, X = sum_i k_i 2^(49 - 7 i), k_i in [-64, 63], each an
 // exact bf16 number k_i 2^(-7 i) (the error-free slicing of Ozaki, Ogita, Oishi and Rump, with a fixed grid per
@@ -15,9 +15,14 @@
 // order.  Levels >= 9 are dropped: below 2^-60 of the window's largest product.  Per window the levels are put
 // together as one 51-bit and one 19-bit integer and added to the FP64 running sums (one FP64 FMA; the low bits go
 // to an FP32 sum of weight 2^-61).  The generated values are rounded once to FP64 as W A_P, as in the CUDA-core
-// contraction; the sums then lose less than its chain of G multiply-adds, each of which rounds the partial sum:
-// measured against long double on two-centre p + H, the off-diagonal blocks err by 1e-17 to 2e-17 in 2-norm where
-// the chain errs by 8e-17 to 1.3e-15 (|z| <= 12).
+// contraction.
+//
+// Accuracy.  A window's rounding is relative to the product of its rows' largest values.  In 2-norm the off-diagonal
+// blocks of two-centre p + H err by 1e-17 to 2e-17 (against long double, |z| <= 12), the chain of G multiply-adds by 8e-17
+// to 1.3e-15.  A small element whose rows peak at different nuclei is far below that product, so the nodes' order, the
+// windows' length and exact power-of-two scales keep the two together (f64_order.cuh): element by element the error
+// stays within what the chain leaves, at any distance.  The shorter windows cost FP64 operations, two per result and window:
+// 21 p + H positions over |z| <= 20 take 1.36 ms a call, 1.20 with windows of 512 nodes throughout.
 //
 // What bounds it.  The FP64 pipe of this part does two FMAs per clock per SM, and the CUDA-core contraction takes
 // five FP64 operations per (target state, half column, node): 581 us per p + H position (N = 380, 2304 nodes).  Here
@@ -32,10 +37,13 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <vector>
 
 #include "f64_digits.cuh"
+#include "f64_order.cuh"
+#include "geometry.cuh"
 #include "wpccc_internal.cuh"
 
 namespace wpccc {
@@ -51,15 +59,17 @@ constexpr int F64_GSTAGES = 4;
 constexpr int F64_RING = 160 * 1024;            // table ring: as many chunks as the tile's height allows
 constexpr int F64_TSTAGES_MAX = 8;
 constexpr int F64_DONE = 8;                     // ring of "MMAs of a chunk completed" barriers (>= every other ring)
-constexpr int F64_SPLIT = 4;                    // blocks of k_f64_slices per window
+constexpr int F64_SPLIT = 4;                    // blocks of k_f64_slices per span of 512 nodes
 
 // ---------------------------------------------------------------------------
 // k_f64_slices: the operands of the contraction from the FP64 node tables.
-// F64_SPLIT blocks per (window of 512 nodes, position): a warp per projectile half column (A_P and the scale exponents of
+// F64_SPLIT blocks per (span of 512 nodes, position): a warp per projectile half column (A_P and the scale exponents of
 // its generated rows), then a warp per (target radial, |m|) (digits of A_T r_T and A_T r_T V_T; the rows of m and
 // -m differ by the sign (-1)^m).  Lane: nodes 4 lane .. 4 lane + 3 and 128, 256, 384 further.
 // ---------------------------------------------------------------------------
 struct F64SliceArgs {
+    const EvalDesc* ev;
+    double kappa;
     int G, Gp, nradT, nradP, nlqT, nd, n_half, tc_rows, nwin, n_items, qmaxT;
     const int* items;       // [n_items][7]: radial, (l, |m|) index, 1 when m odd, row of +m, row of -m (or -1), sizes of their tiles
     const int* halves;      // [n_half][3]: radial, (l, q) index, q
@@ -84,7 +94,28 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
     __shared__ __align__(16) double s_r[F64_WIN], s_rv[F64_WIN];
     extern __shared__ int s_hw[];   // [nd][F64_WIN]: high word of max(|re|, |im|) of W / r_T
     const int e = blockIdx.y, w = blockIdx.x / F64_SPLIT, part = blockIdx.x % F64_SPLIT, g0 = w * F64_WIN;
-    const int tid = threadIdx.x, warp = part * 8 + (tid >> 5), lane = tid & 31;   // warp among the window's
+    const int tid = threadIdx.x, warp = part * 8 + (tid >> 5), lane = tid & 31;   // warp among the span's
+    constexpr int Q = F64_WIN / 128;   // node quads per lane
+    const int wch = f64_window_chunks(A.Gp, __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z))), wlog = 31 - __clz(wch);
+    // m[j] <- the largest m over the window of the lane's quad j
+    auto window_max = [&](int (&m)[Q]) {
+        if (wch * F64_K == F64_WIN) {
+            for (int j = 1; j < Q; ++j) m[0] = max(m[0], m[j]);
+            m[0] = __reduce_max_sync(0xffffffffu, m[0]);
+            for (int j = 1; j < Q; ++j) m[j] = m[0];
+        } else {
+            for (int j = 0; j < Q; ++j) {
+                if (wch == 4) m[j] = __reduce_max_sync(0xffffffffu, m[j]);
+                else
+                    for (int o = 4 * wch; o > 0; o >>= 1) m[j] = max(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
+            }
+        }
+    };
+    // window of the lane's quad j, for the one lane and quad that write it; else -1
+    auto window_of = [&](int j) {
+        const int g = g0 + 4 * lane + 128 * j;
+        return g < A.Gp && (g & (wch * F64_K - 1)) == 0 ? g / F64_K >> wlog : -1;
+    };
     char* base = A.node + (size_t)e * A.node_bytes;
     const double* fT = reinterpret_cast<const double*>(base);
     const double* fP = fT + (size_t)A.nradT * A.G;
@@ -129,9 +160,10 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
         }
         const int dlo = max(0, q - A.qmaxT), dhi = min(A.nd - 1, q + A.qmaxT);
         for (int d = dlo; d <= dhi; ++d) {
-            int m = 0;
+            int m[Q];
 #pragma unroll
-            for (int j = 0; j < F64_WIN / 128; ++j) {
+            for (int j = 0; j < Q; ++j) {
+                m[j] = 0;
                 const int4 hw = *reinterpret_cast<const int4*>(s_hw + d * F64_WIN + 4 * lane + 128 * j);
                 const int hv[4] = {hw.x, hw.y, hw.z, hw.w};
 #pragma unroll
@@ -142,18 +174,21 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
                     const uint32_t ab = (uint32_t)a + (uint32_t)b;
                     const int p = max(a, b) >= 0x7FF00000 ? 0x7FF00000
                                   : min(a, b) < (1 << 20) || ab < (1023u << 20) ? 0 : (int)min(ab - (1023u << 20), 0x7FEFFFFFu);
-                    m = max(m, p);
+                    m[j] = max(m[j], p);
                 }
             }
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (lane == 0) eb[((size_t)c * A.nd + d) * A.nwin + w] = f64_exponent(m, F64_MARGIN2);
+            window_max(m);
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                const int x = window_of(j);
+                if (x >= 0) eb[((size_t)c * A.nd + d) * A.nwin + x] = f64_exponent(m[j], F64_MARGIN2);
+            }
         }
     }
     // target rows
     __nv_bfloat16* pl = reinterpret_cast<__nv_bfloat16*>(base + A.pl_off);
-    int* ea = reinterpret_cast<int*>(base + A.ea_off) + (size_t)w * A.tc_rows;
+    int* ea = reinterpret_cast<int*>(base + A.ea_off);
     const size_t plane = (size_t)A.tc_rows * A.Gp;
-    constexpr int Q = F64_WIN / 128;   // node quads per lane
     for (int it = warp; it < A.n_items; it += 8 * F64_SPLIT) {
         const int* I = A.items + 7 * it;
         const double* f = fT + (size_t)I[0] * A.G;
@@ -173,7 +208,7 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
         for (int v = 0; v < 2; ++v) {
             const double* sr = v == 0 ? s_r : s_rv;
             double x[4 * Q];
-            int hm = 0;
+            int m[Q];
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const double2 ra = *reinterpret_cast<const double2*>(sr + 4 * lane + 128 * j),
@@ -182,20 +217,21 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
                 x[4 * j + 1] = t[4 * j + 1] * ra.y;
                 x[4 * j + 2] = t[4 * j + 2] * rb.x;
                 x[4 * j + 3] = t[4 * j + 3] * rb.y;
+                m[j] = 0;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) hm = max(hm, abs_hi(x[4 * j + k]));
+                for (int k = 0; k < 4; ++k) m[j] = max(m[j], abs_hi(x[4 * j + k]));
             }
-            const int E = f64_exponent(__reduce_max_sync(0xffffffffu, hm), F64_MARGIN);
-            const int E1 = E + 1023;
+            window_max(m);
             const int r1 = rp + v * ts, r2 = rn + v * tsn;
-            if (lane == 0) {
-                ea[r1] = E;
-                if (rn >= 0) ea[r2] = E;
-            }
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const int g = g0 + 4 * lane + 128 * j;
                 if (g >= A.Gp) continue;
+                const int E = f64_exponent(m[j], F64_MARGIN), E1 = E + 1023, wx = window_of(j);
+                if (wx >= 0) {
+                    ea[(size_t)wx * A.tc_rows + r1] = E;
+                    if (rn >= 0) ea[(size_t)wx * A.tc_rows + r2] = E;
+                }
                 uint32_t d0[F64_SL], d1[F64_SL];
                 f64_digits(f64_fix(x[4 * j], E1), f64_fix(x[4 * j + 1], E1), d0);
                 f64_digits(f64_fix(x[4 * j + 2], E1), f64_fix(x[4 * j + 3], E1), d1);
@@ -224,6 +260,8 @@ struct F64Maps {
 };
 
 struct F64Args {
+    const EvalDesc* ev;
+    double kappa;
     int Gp, N_T, n_half, nk, nwin, nd, n_ntiles, tc_rows, qg_max;
     const int *qg_off, *qg_q, *qg_rows, *half_q;
     const char* node;
@@ -275,6 +313,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
     volatile int* abort_flag = &s_abort;
     const char* nb = A.node + (size_t)e * A.node_bytes;
     const int nk = A.nk;
+    const int wch = f64_window_chunks(A.Gp, __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z))), wlog = 31 - __clz(wch);
 
     if (warp == F64_TMA_WARP) {
         // ---- TMA issue (one thread): the table tiles chunk by chunk into their ring
@@ -315,9 +354,9 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             };
             bool ready = false;
             for (int k = 0; k < nk && ok; ++k) {
-                const bool fresh = k % F64_WCH == 0;   // the window's first products overwrite the accumulators
+                const bool fresh = (k & (wch - 1)) == 0;   // the window's first products overwrite the accumulators
                 if (!ready) ok = wait(tfull0 + 8 * ts, tph, 32) && wait(gfull0 + 8 * gs, gph, 33);
-                if (ok && fresh && k > 0) ok = wait(acce, (k / F64_WCH - 1) & 1, 34);
+                if (ok && fresh && k > 0) ok = wait(acce, ((k >> wlog) - 1) & 1, 34);
                 if (!ok) break;
                 tc_fence_after();
                 const uint64_t da = da0 + (uint64_t)(ts * (tstage >> 4)), db = db0 + (uint64_t)(gs * (F64_GSTAGE >> 4));
@@ -331,7 +370,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
                 tc_commit(done0 + 8 * dsl);
                 dsl = (dsl + 1) % F64_DONE;
                 issued = k + 1;
-                if (k % F64_WCH == F64_WCH - 1 || k == nk - 1) tc_commit(accf);
+                if ((k & (wch - 1)) == wch - 1 || k == nk - 1) tc_commit(accf);
             }
             // the MMAs issued complete before the tensor memory is released
             if (issued > 0)
@@ -361,7 +400,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             low[k] = 0.f;
         }
         bool ok = true;
-        for (int j = 0; j < A.nwin && ok; ++j) {
+        const int nwin = (nk + wch - 1) >> wlog;
+        for (int j = 0; j < nwin && ok; ++j) {
             const int Ea = lrow < 2 * ns ? ea[(size_t)j * A.tc_rows + row0 + lrow] : F64_EMIN;
             const int Eb = ebv ? eb[ebo + j] : F64_EMIN;
             ok = mbar_wait_warp(accf, j & 1, abort_flag, A.err, 35, A.wait_limit);
@@ -405,7 +445,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             for (int k = 0; k < 16; k += 2) {
                 const int c = c0 + (col0 + k) / 2;
                 if (c < A.n_half)
-                    out[c] = make_double2(acc[k] + (double)low[k], acc[k + 1] + (double)low[k + 1]);
+                    out[c] = make_double2(f64_total(acc[k], low[k]), f64_total(acc[k + 1], low[k + 1]));
             }
         }
     } else {
@@ -436,7 +476,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
                 const int g = (k + 1) * F64_K;
                 if (valid) {
                     a = *reinterpret_cast<const double2*>(ap + g);
-                    if ((k + 1) % F64_WCH == 0) E = eb[(k + 1) / F64_WCH];
+                    if (((k + 1) & (wch - 1)) == 0) E = eb[(k + 1) >> wlog];
                 }
                 r = *reinterpret_cast<const double2*>(wr + g);
                 im = *reinterpret_cast<const double2*>(wi + g);
@@ -474,7 +514,7 @@ void f64_layout(const wpccc_basis_s* B, size_t node_doubles, ElemScratch& L) {
     auto a256 = [](size_t x) { return (x + 255) / 256 * 256; };
     L.tc_rows = 2 * B->N_T;
     L.Gp = (B->G + F64_K - 1) / F64_K * F64_K;
-    L.f64_nwin = (L.Gp + F64_WIN - 1) / F64_WIN;
+    L.f64_nwin = L.Gp / F64_K;
     size_t o = a256(node_doubles * sizeof(double));
     L.f64_pl = o;
     o += a256((size_t)F64_SL * L.tc_rows * L.Gp * 2);
@@ -490,6 +530,8 @@ void f64_layout(const wpccc_basis_s* B, size_t node_doubles, ElemScratch& L) {
     o += a256((size_t)2 * L.Gp * sizeof(double));
     L.node_doubles = o / sizeof(double);
 }
+
+double f64_kappa(const wpccc_basis_s* B) { return std::min(std::fabs(B->T.Z), std::fabs(B->P.Z)); }
 
 // Work lists of k_f64_slices, kept on the basis: (radial, |m|) items of the target and the half columns.
 static wpccc_status f64_lists(wpccc_basis_s* B) {
@@ -537,11 +579,13 @@ wpccc_status fp64_route(wpccc_basis_s* B, int* precision) {
     return WPCCC_OK;
 }
 
-wpccc_status launch_mol_f64tc(wpccc_basis_s* B, int nev, void* node, double2* mol, int* err,
+wpccc_status launch_mol_f64tc(wpccc_basis_s* B, const EvalDesc* evals, int nev, void* node, double2* mol, int* err,
                               cudaStream_t st) {
     const ElemScratch L = elem_scratch_layout(B, ELEM_F64_TC);
     const size_t node_bytes = L.node_doubles * sizeof(double);
     F64SliceArgs sa;
+    sa.ev = evals;
+    sa.kappa = f64_kappa(B);
     sa.G = B->G;
     sa.Gp = L.Gp;
     sa.nradT = B->T.n_rad;
@@ -566,7 +610,7 @@ wpccc_status launch_mol_f64tc(wpccc_basis_s* B, int nev, void* node, double2* mo
     const size_t ssm = (size_t)sa.nd * F64_WIN * sizeof(int);
     if (ssm > 40 * 1024)   // with the static 8 KB
         WPCCC_CUDA(cudaFuncSetAttribute(k_f64_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm));
-    k_f64_slices<<<dim3(sa.nwin * F64_SPLIT, nev), 256, ssm, st>>>(sa);
+    k_f64_slices<<<dim3((sa.Gp + F64_WIN - 1) / F64_WIN * F64_SPLIT, nev), 256, ssm, st>>>(sa);
     WPCCC_CHECK_LAUNCH("k_f64_slices");
     // the digit planes as one 3-D bf16 tensor: x = node (Gp), y = digit plane row (8 x tc_rows), z = position
     F64Maps maps;
@@ -581,6 +625,8 @@ wpccc_status launch_mol_f64tc(wpccc_basis_s* B, int nev, void* node, double2* mo
         if (r != CUDA_SUCCESS) return fail(WPCCC_ECUDA, "cuTensorMapEncodeTiled failed for the digit planes");
     }
     F64Args a;
+    a.ev = evals;
+    a.kappa = f64_kappa(B);
     a.Gp = L.Gp;
     a.N_T = B->N_T;
     a.n_half = B->n_half;

@@ -1,4 +1,5 @@
-// The FP64 Schur form's rank-N_T update C = I - K^+ K on the 5th-generation tensor cores, to more than FP64's accuracy.
+// The FP64 Schur form's rank-N_T update C = I - K^+ K on the 5th-generation tensor cores, to more than FP64's
+// accuracy in norm (I - K^+ K is of order 1, so its small elements need no more).
 //
 // With X[m][2t] = Re K[t][m], X[m][2t+1] = Im K[t][m] and Y[m][2t] = Im K[t][m], Y[m][2t+1] = -Re K[t][m],
 //   (K^+ K)_re[m][n] = sum_k X[m][k] X[n][k],   (K^+ K)_im[m][n] = sum_k X[m][k] Y[n][k],
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(SD_THREADS, 1) k_schur_f64tc(const __grid_cons
             for (int k = 0; k < 16; ++k) {
                 const int n = n0 + col0 + k;
                 if (n >= A.NP || n > m) continue;
-                const double c = acc[k] + (double)low[k];
+                const double c = f64_total(acc[k], low[k]);
                 double* p = reinterpret_cast<double*>(S + (size_t)(A.N_T + m) + (size_t)(A.N_T + n) * A.N);
                 if (half) p[1] = -c;
                 else p[0] = (m == n ? 1.0 : 0.0) - c;

@@ -185,7 +185,7 @@ struct ElemScratch {
     size_t t6_sc_off, t6_ap_off, t6_w_off;
     // FP64 tensor-core form (ELEM_F64_TC): behind the FP64 node tables the digit planes, the scale exponents of the
     // table rows and of the generated rows, A_P, W_K / r_T and r_T, r_T V_T in FP64 (byte offsets within a position's tables);
-    // Gp: nodes padded to a multiple of 32, f64_nwin: scaling windows
+    // Gp: nodes padded to a multiple of 32, f64_nwin: scaling windows there may be
     int Gp, f64_nwin;
     size_t f64_pl, f64_ea, f64_eb, f64_ap, f64_w2, f64_r;
 };
@@ -194,10 +194,11 @@ struct ElemScratch {
 enum : int { ELEM_F64 = 0, ELEM_F32 = 1, ELEM_TC4 = 3, ELEM_TC7 = 4, ELEM_F64_TC = 6 };
 ElemScratch elem_scratch_layout(const wpccc_basis_s* B, int precision);
 void f64_layout(const wpccc_basis_s* B, size_t node_doubles, ElemScratch& L);
+double f64_kappa(const wpccc_basis_s* B);   // steepness of the form's node order and scales (f64_order.cuh)
 // The element arithmetic of a plain FP64 call (ELEM_F64_TC where the tensor cores take it, else ELEM_F64), with
 // its lists prepared on the basis (before any capture).
 wpccc_status fp64_route(wpccc_basis_s* B, int* precision);
-wpccc_status launch_mol_f64tc(wpccc_basis_s* B, int nev, void* node, double2* mol, int* err, cudaStream_t st);
+wpccc_status launch_mol_f64tc(wpccc_basis_s* B, const EvalDesc* evals, int nev, void* node, double2* mol, int* err, cudaStream_t st);
 
 // Queue the element kernels for `nev` evaluations (device list `evals`), writing
 // S and H (matrix k at S + k*N*N).  S may be null (one-centre propagation).

@@ -447,7 +447,9 @@ WPCCC_API wpccc_status wpccc_basis_set_rk4_layout(wpccc_basis basis, int layout)
 
 /*
  * Upper bound on the scratch memory wpccc_propagate may hold (default 8 GiB).
- * The number of RK4 steps batched per launch is chosen to fit it.
+ * The number of RK4 steps batched per launch is chosen to fit it, and in the FP64 form (modes 0 and 2), whose
+ * digits take the most, the number of positions per launch of the element kernels.  One step's matrices for all
+ * paths and one position's digits are held in any case.  The results do not depend on it.
  */
 WPCCC_API wpccc_status wpccc_basis_set_workspace_limit(wpccc_basis basis, size_t bytes);
 

@@ -1726,6 +1726,27 @@ wpccc_status check_tc_err(wpccc_basis_s* B, const char* where) {
                                     std::to_string(e) + ")");
 }
 
+wpccc_status elem_workspace(wpccc_basis_s* B, int* precision, int n, int* per) {
+    auto get = [&]() {
+        const size_t each = elem_scratch_layout(B, *precision).bytes_per_eval + sizeof(EvalDesc);
+        *per = (int)std::min<size_t>({(size_t)n, (size_t)MAX_EVALS_PER_LAUNCH,
+                                      std::max<size_t>(1, (B->ws_limit - 256) / each)});
+        return ensure_workspace(B, (size_t)*per * each + 256);
+    };
+    const int all = n;
+    wpccc_status s = get();
+    while (s == WPCCC_ENOMEM && *precision == ELEM_F64_TC) {
+        cudaGetLastError();   // the failed allocation's, not a later launch's
+        if (*per > 1) n = *per / 2;
+        else {
+            *precision = ELEM_F64;
+            n = all;
+        }
+        s = get();
+    }
+    return s;
+}
+
 // Grows the basis-owned scratch buffer to at least `bytes`.
 wpccc_status ensure_workspace(wpccc_basis_s* B, size_t bytes) {
     if (B->ws_bytes >= bytes) return WPCCC_OK;
@@ -1790,20 +1811,7 @@ static wpccc_status matrix_elements_prec(wpccc_basis B, double b, double v, int 
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     int chunk = 1;
-    // evaluations per launch bounded by the workspace limit
-    auto workspace = [&]() {
-        const ElemScratch L = elem_scratch_layout(B, precision);
-        const size_t per = L.bytes_per_eval + sizeof(EvalDesc);
-        chunk = (int)std::min<size_t>({(size_t)nz, (size_t)MAX_EVALS_PER_LAUNCH,
-                                       std::max<size_t>(1, (B->ws_limit - 256) / per)});
-        return ensure_workspace(B, (size_t)chunk * L.bytes_per_eval + 256 + (size_t)chunk * sizeof(EvalDesc));
-    };
-    wpccc_status s = workspace();
-    if (s == WPCCC_ENOMEM && precision == ELEM_F64_TC) {   // the CUDA cores' form takes less scratch
-        cudaGetLastError();
-        precision = ELEM_F64;
-        s = workspace();
-    }
+    wpccc_status s = elem_workspace(B, &precision, nz, &chunk);
     if (s != WPCCC_OK) return s;
     char* wsb = static_cast<char*>(B->ws_ptr);
     EvalDesc* dev_ev = reinterpret_cast<EvalDesc*>(wsb);

@@ -501,6 +501,7 @@ namespace wpccc {
 struct PropPlan {
     wpccc_basis_s* B = nullptr;
     int np = 0, N = 0, mode = RK_MATRIX, elem_precision = 0, C = 1, n_chunks = 0, max_chunk_evals = 0;
+    int elem_batch = 0;      // positions per launch of the element kernels (a chunk's, or fewer: see plan_build)
     int max_steps = 0;
     bool two = false, mixed = false, stage = false, schur = false;
     bool schur_tc = false;   // Schur forms: the trailing update I - K^+ K on the tensor cores
@@ -525,8 +526,10 @@ struct PropPlan {
 static size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // Validates the paths and lays out the plan.  C_request > 0 fixes the RK4 steps per chunk,
-// otherwise they are chosen from the workspace limit and the SM count.  cuda_cores: the FP64 contraction stays off the
-// tensor cores, whose digits take more scratch per position (the callers' second try when memory is short).
+// otherwise they are chosen from the workspace limit and the SM count.  The FP64 form's digits take five times the CUDA
+// cores' scratch per position: where one step of all paths with them exceeds the limit, a chunk's elements run in
+// several launches over a smaller scratch (the results are the same bits).  cuda_cores: the FP64 contraction stays off
+// the tensor cores (the callers' last try when memory is short).
 static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int precision_mode, int C_request,
                                size_t ws_limit, PropPlan& P, bool cuda_cores = false) {
     if (precision_mode < 0 || precision_mode > 5)
@@ -686,9 +689,15 @@ static wpccc_status plan_build(wpccc_basis_s* B, const wpccc_paths* paths, int p
     P.sz_H = align256((size_t)mce * mat * sizeof(double2)) * 2;
     P.sz_piv = P.two ? align256((size_t)mce * N * sizeof(int)) * 2 : 0;
     P.sz_info = P.two ? align256((size_t)mce * sizeof(int)) * 2 : 0;
-    P.sz_scr = align256((size_t)mce * L.bytes_per_eval);
     P.bytes = P.sz_carry + P.sz_carryLU + P.sz_carryPiv + P.sz_carryLU32 + P.sz_LU32 + P.sz_z + P.sz_ev + P.sz_pc +
-              P.sz_flags + P.sz_S + P.sz_H + P.sz_piv + P.sz_info + P.sz_scr + P.sz_vec;
+              P.sz_flags + P.sz_S + P.sz_H + P.sz_piv + P.sz_info + P.sz_vec;
+    P.elem_batch = mce;
+    if (P.elem_precision == ELEM_F64_TC) {
+        const size_t room = ws_limit > P.bytes + 256 ? ws_limit - P.bytes - 256 : 0;
+        P.elem_batch = (int)std::max<size_t>(1, std::min<size_t>(mce, room / L.bytes_per_eval));
+    }
+    P.sz_scr = align256((size_t)P.elem_batch * L.bytes_per_eval);
+    P.bytes += P.sz_scr;
     return WPCCC_OK;
 }
 
@@ -796,17 +805,25 @@ static wpccc_status plan_enqueue(PropPlan& P, double2* c, const PlanStreams& S, 
         int* bI = P.two ? P.d_info + k * hI : nullptr;
         // buffer set k is free once the RK4 sweep of chunk ch - 2 is done
         if (ch >= 2) WPCCC_CUDA(cudaStreamWaitEvent(st, S.rk_done[k], 0));
-        s = launch_elements(B, P.d_ev + P.ev_begin[ch], nev, bS, bH, P.d_scr, st, P.elem_precision);
-        if (s != WPCCC_OK) return s;
-        if (P.two) {
+        for (int p0 = 0; p0 < nev; p0 += P.elem_batch) {
+            const int n = std::min(P.elem_batch, nev - p0);
+            const size_t o = (size_t)p0 * N * N;
+            s = launch_elements(B, P.d_ev + P.ev_begin[ch] + p0, n, P.two ? bS + o : nullptr, bH + o, P.d_scr, st,
+                                P.elem_precision);
+            if (s != WPCCC_OK) return s;
+            if (P.schur_tc) {   // its digits or slices take the elements' scratch
+                cudaEvent_t e0 = B->prof.begin(PROF_SOLVE, st);
+                const size_t per = elem_scratch_layout(B, P.elem_precision).bytes_per_eval;
+                s = P.mixed ? launch_schur_factor_f32_tc(B, n, bS + o, bL + o, bI + p0, P.d_scr, per, st)
+                            : launch_schur_factor_fp64_tc(B, n, bS + o, bI + p0, P.d_scr, per, st);
+                if (s != WPCCC_OK) return s;
+                B->prof.end(PROF_SOLVE, st, e0);
+            }
+        }
+        if (P.two && !P.schur_tc) {
             cudaEvent_t e0 = B->prof.begin(PROF_SOLVE, st);
-            if (P.mixed && P.schur && P.schur_tc)
-                s = launch_schur_factor_f32_tc(B, nev, bS, bL, bI, P.d_scr,
-                                               elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
-            else if (P.mixed && P.schur) s = launch_schur_factor_f32(N, B->N_T, nev, bS, bL, bI, st);
+            if (P.mixed && P.schur) s = launch_schur_factor_f32(N, B->N_T, nev, bS, bL, bI, st);
             else if (P.mixed) s = launch_factor_f32(N, nev, bS, bL, bP, bI, st);
-            else if (P.schur && P.schur_tc)
-                s = launch_schur_factor_fp64_tc(B, nev, bS, bI, P.d_scr, elem_scratch_layout(B, P.elem_precision).bytes_per_eval, st);
             else if (P.schur) s = launch_schur_factor(N, B->N_T, nev, bS, bI, st);
             else s = launch_solve(N, nev, bS, P.stage ? nullptr : bH, bP, bI, st);
             if (s == WPCCC_OK && P.mode == RK_STAGE) s = launch_lu_invert_diag(N, nev, bS, st);
@@ -893,10 +910,16 @@ wpccc_status propagate_internal(wpccc_basis_s* B, const wpccc_paths* paths, int 
     wpccc_status s = plan_build(B, paths, precision_mode, 0, B->ws_limit, P);
     if (s != WPCCC_OK) return s;
     if (P.max_steps == 0) return WPCCC_OK;
+    // short of memory with the digits: half of it (fewer steps per chunk, then fewer positions per element launch, the same
+    // bits), down to one position; then the CUDA cores' contraction
     s = ensure_workspace(B, P.bytes);
-    if (s == WPCCC_ENOMEM && P.elem_precision == ELEM_F64_TC) {
+    while (s == WPCCC_ENOMEM && P.elem_precision == ELEM_F64_TC) {
         cudaGetLastError();   // the failed allocation's, not a later launch's
-        if ((s = plan_build(B, paths, precision_mode, 0, B->ws_limit, P, true)) != WPCCC_OK) return s;
+        const size_t tried = P.bytes;
+        if ((s = plan_build(B, paths, precision_mode, 0, tried / 2, P)) != WPCCC_OK) return s;
+        if (P.bytes >= tried &&
+            (s = plan_build(B, paths, precision_mode, 0, B->ws_limit, P, true)) != WPCCC_OK)
+            return s;
         s = ensure_workspace(B, P.bytes);
     }
     if (s != WPCCC_OK) return s;
@@ -961,7 +984,7 @@ static void batch_free(wpccc_batch_s* X) {
 
 // Times one candidate schedule of a set on its first steps: a warm run, then a timed run.
 static wpccc_status tune_trial(wpccc_basis_s* B, const wpccc_paths* paths, int precision, int C, double2* c_src,
-                               double* ms_per_step, bool cuda_cores) {
+                               double* ms_per_step, size_t limit, bool cuda_cores) {
     // the set's paths cut to 2C steps (at least two chunks, so the overlap is part of the timing)
     const int np = paths->n_paths;
     std::vector<int> nz(np);
@@ -981,7 +1004,7 @@ static wpccc_status tune_trial(wpccc_basis_s* B, const wpccc_paths* paths, int p
     }
     wpccc_paths tp{np, paths->b, paths->v, nz.data(), z.data()};
     PropPlan P;
-    wpccc_status s = plan_build(B, &tp, precision, C, B->ws_limit, P, cuda_cores);
+    wpccc_status s = plan_build(B, &tp, precision, C, limit, P, cuda_cores);
     if (s != WPCCC_OK) return s;
     void* ws = nullptr;
     double2* c = nullptr;
@@ -1052,12 +1075,20 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
         return st;
     };
     wpccc_status s = WPCCC_OK;
-    auto plan_sets = [&](bool cuda_cores) -> wpccc_status {
+    bool digits = false, smallest = true;   // some set's plan takes the digits; all of those run one position at a time
+    auto plan_sets = [&](size_t cap, bool cuda_cores) -> wpccc_status {
+    digits = false;
+    smallest = true;
     for (int k = 0; k < n_sets; ++k) {
         wpccc_basis_s* B = bases[k];
+        const size_t limit = std::min(B->ws_limit, cap);
         X->c[k] = static_cast<double2*>(c[k]);
         PropPlan P;
-        if ((s = plan_build(B, &paths[k], precision_mode, 0, B->ws_limit, P, cuda_cores)) != WPCCC_OK) return s;
+        if ((s = plan_build(B, &paths[k], precision_mode, 0, limit, P, cuda_cores)) != WPCCC_OK) return s;
+        if (P.elem_precision == ELEM_F64_TC && P.max_steps > 0) {
+            digits = true;
+            if (P.C > 1 || P.elem_batch > 1) smallest = false;
+        }
         int best = P.C;
         if (autotune && P.max_steps > 1) {
             // schedules tried: the default chunk and half and twice as many RK4 steps per chunk
@@ -1069,7 +1100,7 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
                 double ms = 0.0;
                 const bool was_on = B->prof.on;
                 B->prof.on = false;
-                s = tune_trial(B, &paths[k], precision_mode, C, X->c[k], &ms, cuda_cores);
+                s = tune_trial(B, &paths[k], precision_mode, C, X->c[k], &ms, limit, cuda_cores);
                 B->prof.on = was_on;
                 if (s != WPCCC_OK) return s;
                 if (best_ms < 0.0 || ms < best_ms) {
@@ -1079,7 +1110,7 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
             }
             X->tuned_ms_per_step[k] = best_ms;
         }
-        if ((s = plan_build(B, &paths[k], precision_mode, best, B->ws_limit, X->plans[k], cuda_cores)) != WPCCC_OK) return s;
+        if ((s = plan_build(B, &paths[k], precision_mode, best, limit, X->plans[k], cuda_cores)) != WPCCC_OK) return s;
         X->chunk_steps[k] = X->plans[k].C;
     }
     // one workspace for every set
@@ -1087,15 +1118,23 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
     for (auto& P : X->plans) total += align256(P.bytes);
     {
         cudaError_t e = cudaMalloc(&X->ws, std::max<size_t>(total, 256));
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(batch workspace)");
+        if (e != cudaSuccess) {
+            X->ws = nullptr;
+            return cuda_fail(e, "cudaMalloc(batch workspace)");
+        }
     }
     return WPCCC_OK;
     };
-    s = plan_sets(false);
-    if (s == WPCCC_ENOMEM && (precision_mode == 0 || precision_mode == 2)) {
+    // as wpccc_propagate does: half of the memory while the digits do not fit, then the CUDA cores
+    size_t ws_cap = (size_t)1 << 46;
+    s = plan_sets(ws_cap, false);
+    while (s == WPCCC_ENOMEM && digits) {
         cudaGetLastError();
-        X->ws = nullptr;
-        s = plan_sets(true);
+        if (smallest) s = plan_sets((size_t)1 << 46, true);
+        else {
+            for (int k = 0; k < n_sets; ++k) ws_cap = std::min(ws_cap, bases[k]->ws_limit);
+            s = plan_sets(ws_cap /= 2, false);
+        }
     }
     if (s != WPCCC_OK) return bail(s);
     size_t off = 0;

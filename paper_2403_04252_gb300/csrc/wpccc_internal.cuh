@@ -214,6 +214,11 @@ wpccc_status launch_node_stage(wpccc_basis_s* B, const EvalDesc* evals, int nev,
 wpccc_status propagate_internal(wpccc_basis_s* B, const wpccc_paths* paths, int precision_mode, double2* c,
                                 cudaStream_t st);
 
+// Workspace for element launches of *per <= n positions: 256 bytes, then an EvalDesc and the elements' scratch per
+// position.  *per follows the workspace limit; where the FP64 form's digits do not fit the device's memory it is halved, and
+// at one position *precision becomes ELEM_F64, whose scratch is a fifth.
+wpccc_status elem_workspace(wpccc_basis_s* B, int* precision, int n, int* per);
+
 // Grows the basis-owned scratch buffer to at least `bytes`.
 wpccc_status ensure_workspace(wpccc_basis_s* B, size_t bytes);
 

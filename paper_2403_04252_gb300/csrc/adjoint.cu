@@ -850,7 +850,7 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     // S and H of a segment: positions per launch that the element-adjoint workspace holds in the elements' layout
     int elem_prec = ELEM_F64;
     if ((s = fp64_route(B, &elem_prec)) != WPCCC_OK) return s;
-    const size_t elem_bytes = elem_scratch_layout(B, elem_prec).bytes_per_eval;
+    size_t elem_bytes = elem_scratch_layout(B, elem_prec).bytes_per_eval;
     const TanLayout TL = tan_layout(B);
     const int NB = std::max(1, std::min(max_pos, 256));
     const int n_tiles = (B->G + ADJ_NODES - 1) / ADJ_NODES;
@@ -867,9 +867,17 @@ static wpccc_status adjoint_group(wpccc_basis_s* B, const wpccc_paths* paths, in
     if ((s = D.get(&tnode, (size_t)NB * TL.doubles, "adjoint node derivatives")) != WPCCC_OK) return s;
     if ((s = D.get(&d_terms, (size_t)max_pos * 2 * n_obs, "adjoint terms")) != WPCCC_OK) return s;
     if ((s = D.get(&d_jobs, (size_t)max_terms * ADJ_KINDS, "adjoint jobs")) != WPCCC_OK) return s;
-    const size_t ws_need = std::max((size_t)NB * EL.bytes_per_eval, elem_bytes);
+    size_t ws_need = std::max((size_t)NB * EL.bytes_per_eval, elem_bytes);
+    s = ensure_workspace(B, ws_need);
+    if (s == WPCCC_ENOMEM && elem_prec == ELEM_F64_TC) {   // the element adjoint's own scratch holds the CUDA cores' form
+        cudaGetLastError();
+        elem_prec = ELEM_F64;
+        elem_bytes = EL.bytes_per_eval;
+        ws_need = (size_t)NB * elem_bytes;
+        s = ensure_workspace(B, ws_need);
+    }
+    if (s != WPCCC_OK) return s;
     const int NE = (int)std::max<size_t>(1, std::min<size_t>(NB, ws_need / elem_bytes));
-    if ((s = ensure_workspace(B, ws_need)) != WPCCC_OK) return s;
     double* node = static_cast<double*>(B->ws_ptr);
     const int adj_smem = (int)adj_rk_smem_bytes(N, n_obs);
     int sms = 0;

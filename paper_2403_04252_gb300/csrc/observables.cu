@@ -148,16 +148,24 @@ extern "C" wpccc_status wpccc_overlap_norms(wpccc_basis B, int n_paths, const do
     int prec = ELEM_F64;
     wpccc_status s = fp64_route(B, &prec);
     if (s != WPCCC_OK) return s;
-    const ElemScratch L = elem_scratch_layout(B, prec);
-    // positions in groups that the workspace limit holds (scratch of the element kernels), S and H per group
-    const int per = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_paths,
-                                                               (B->ws_limit - 256) / (L.bytes_per_eval + sizeof(EvalDesc))));
-    const size_t need = (size_t)per * L.bytes_per_eval + 256 + (size_t)per * sizeof(EvalDesc);
-    if ((s = ensure_workspace(B, need)) != WPCCC_OK) return s;
+    // positions in groups that the workspace limit holds (scratch of the element kernels), S and H per group; where those
+    // two do not fit the device's memory together, groups of half the size, and last the CUDA cores' form
+    int per = 1;
     double2* SH = nullptr;
-    if (cudaMalloc(&SH, 2 * (size_t)per * N * N * sizeof(double2)) != cudaSuccess) {
+    for (int n = n_paths;;) {
+        if ((s = elem_workspace(B, &prec, n, &per)) != WPCCC_OK) return s;
+        if (cudaMalloc(&SH, 2 * (size_t)per * N * N * sizeof(double2)) == cudaSuccess) break;
         cudaGetLastError();
-        return fail(WPCCC_ENOMEM, "wpccc_overlap_norms: cudaMalloc(S, H)");
+        if (prec != ELEM_F64_TC) return fail(WPCCC_ENOMEM, "wpccc_overlap_norms: cudaMalloc(S, H)");
+        if (per > 1) n = per / 2;
+        else {
+            prec = ELEM_F64;
+            n = n_paths;
+        }
+        void* ws = B->ws_ptr;
+        B->ws_ptr = nullptr;
+        B->ws_bytes = 0;
+        WPCCC_CUDA(cudaFree(ws));
     }
     char* wsb = static_cast<char*>(B->ws_ptr);
     EvalDesc* dev_ev = reinterpret_cast<EvalDesc*>(wsb);

@@ -107,3 +107,26 @@ def test_short_memory_shrinks_the_digits_scratch_then_takes_the_cuda_cores():
     g.close()
     assert all(torch.equal(x, y) for x, y in zip(few, few0))
     assert not all(torch.equal(x, y) for x, y in zip(few, digits))
+
+
+def test_overlap_norms_on_a_nearly_full_device():
+    import paper_2403_04252_gb300 as w
+    basis, _ = wi.config_inputs("p_H_2c_n4l3")
+    n = 64
+    rng = np.random.default_rng(3)
+    c = torch.from_numpy(rng.standard_normal((n, basis.N)) + 1j * rng.standard_normal((n, basis.N))).cuda()
+    b, v, z = np.linspace(0.4, 10.0, n), np.full(n, 1.5), np.linspace(-3.0, 3.0, n)
+    out = []
+    # S and H take 0.3 GB for 64 paths, the digits 1.3 GB
+    for nbytes in (8 << 30, 500 << 20):
+        g = w.Basis(basis)
+        torch.cuda.empty_cache()
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - nbytes, dtype=torch.uint8, device="cuda")
+        try:
+            out.append(g.overlap_norms(b, v, z, c).clone())
+            torch.cuda.synchronize()
+        finally:
+            del hold
+            g.close()
+            torch.cuda.empty_cache()
+    assert torch.equal(out[0], out[1])

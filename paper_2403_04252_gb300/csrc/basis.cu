@@ -437,6 +437,8 @@ extern "C" wpccc_status wpccc_basis_create(const wpccc_basis_desc* d, int device
         if ((st = upload(&B->half_of, half_of.data(), half_of.size(), "upload half_of")) != WPCCC_OK)
             return bail(st);
         if ((st = rotation_plan(B)) != WPCCC_OK) return bail(st);
+        int route;   // the FP64 contraction's lists depend on the basis alone: made here, not in the first call
+        if ((st = fp64_route(B, &route)) != WPCCC_OK) return bail(st);
     } else {
         B->P.Z = d->P.Z;
     }

@@ -539,14 +539,13 @@ static wpccc_status f64_lists(wpccc_basis_s* B) {
     std::vector<int> trow(2 * (size_t)B->N_T), hs(B->n_half);
     WPCCC_CUDA(cudaMemcpy(trow.data(), B->tc_row, trow.size() * sizeof(int), cudaMemcpyDeviceToHost));
     WPCCC_CUDA(cudaMemcpy(hs.data(), B->half_state, hs.size() * sizeof(int), cudaMemcpyDeviceToHost));
-    std::vector<int> list;
+    std::vector<int> list, index((size_t)B->T.n_rad * (2 * WPCCC_LMAX + 1), -1);
+    for (int i = 0; i < B->N_T; ++i) index[(size_t)B->T.h_st_rad[i] * (2 * WPCCC_LMAX + 1) + B->T.h_st_m[i] + WPCCC_LMAX] = i;
     int n = 0;
     for (int i = 0; i < B->N_T; ++i) {
         const int a = B->T.h_st_rad[i], l = B->T.h_rad_l[a], m = B->T.h_st_m[i];
         if (m < 0) continue;
-        int in = -1;
-        for (int k = 0; k < B->N_T && m > 0 && in < 0; ++k)
-            if (B->T.h_st_rad[k] == a && B->T.h_st_m[k] == -m) in = k;
+        const int in = m > 0 ? index[(size_t)a * (2 * WPCCC_LMAX + 1) - m + WPCCC_LMAX] : -1;
         list.insert(list.end(), {a, l * (l + 1) / 2 + m, m & 1, trow[i], in >= 0 ? trow[in] : -1, trow[B->N_T + i],
                                  in >= 0 ? trow[B->N_T + in] : 0});
         ++n;

@@ -932,7 +932,8 @@ wpccc_status propagate_internal(wpccc_basis_s* B, const wpccc_paths* paths, int 
     int flags = 0;
     WPCCC_CUDA(cudaMemcpyAsync(&flags, P.d_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaStreamSynchronize(st));
-    if ((s = check_tc_err(B, "wpccc_propagate")) != WPCCC_OK) return s;
+    if (P.elem_precision >= ELEM_TC4 || P.schur_tc)
+        if ((s = check_tc_err(B, "wpccc_propagate")) != WPCCC_OK) return s;
     s = flags_status(flags);
     if (s != WPCCC_OK) set_error(std::string("wpccc_propagate: ") + wpccc_last_error());
     return s;
@@ -1225,8 +1226,8 @@ extern "C" wpccc_status wpccc_batch_status(wpccc_batch X, void* stream) {
             WPCCC_CUDA(cudaMemcpyAsync(&flags[k], X->plans[k].d_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
     WPCCC_CUDA(cudaStreamSynchronize(st));
     for (int k = 0; k < X->n_sets; ++k)
-        if (wpccc_basis_s* B = X->plans[k].B) {
-            wpccc_status ts = check_tc_err(B, "wpccc_batch_status");
+        if (X->plans[k].elem_precision >= ELEM_TC4 || X->plans[k].schur_tc) {
+            wpccc_status ts = check_tc_err(X->plans[k].B, "wpccc_batch_status");
             if (ts != WPCCC_OK) return ts;
         }
     int all = 0;

@@ -195,8 +195,8 @@ enum : int { ELEM_F64 = 0, ELEM_F32 = 1, ELEM_TC4 = 3, ELEM_TC7 = 4, ELEM_F64_TC
 ElemScratch elem_scratch_layout(const wpccc_basis_s* B, int precision);
 void f64_layout(const wpccc_basis_s* B, size_t node_doubles, ElemScratch& L);
 double f64_kappa(const wpccc_basis_s* B);   // steepness of the form's node order and scales (f64_order.cuh)
-// The element arithmetic of a plain FP64 call (ELEM_F64_TC where the tensor cores take it, else ELEM_F64), with
-// its lists prepared on the basis (before any capture).
+// The element arithmetic of a plain FP64 call (ELEM_F64_TC where the tensor cores take it, else ELEM_F64).  Its lists are
+// made on the basis the first time, by wpccc_basis_create.
 wpccc_status fp64_route(wpccc_basis_s* B, int* precision);
 wpccc_status launch_mol_f64tc(wpccc_basis_s* B, const EvalDesc* evals, int nev, void* node, double2* mol, int* err, cudaStream_t st);
 

@@ -1,0 +1,28 @@
+"""The first FP64 call on a two-centre basis costs what later ones do: its lists are made with the basis."""
+import time
+
+import numpy as np
+import pytest
+
+import wpccc_inputs as wi
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def test_the_first_fp64_call_makes_no_lists():
+    import paper_2403_04252_gb300 as w
+    basis = wi.make_basis(1.0, 1.0, 3, 2, 6, 2.0, True, Nr=600, Geta=16, Gtau=16)
+    first, later = [], []
+    for _ in range(22):
+        g = w.Basis(basis)
+        S, H = g.matrix_elements_precision(0.8, 1.2, np.linspace(-1.0, 1.0, 16), 1)   # allocates the workspace
+        for times in (first, later):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            g.matrix_elements(0.8, 1.2, np.array([0.3]), S[:1], H[:1])
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t)
+        g.close()
+    # six allocations and blocking copies and the search for the lists' pairs took 90 us of a call of 220 us
+    assert np.median(first[2:]) < 1.2 * np.median(later[2:]), (first, later)

@@ -345,7 +345,14 @@ static wpccc_status lu_launch(int N, int batch, const double2* S, typename LuC<R
     if (batch == 0) return WPCCC_OK;
     const int smem = (int)(sizeof(C2) * (TM * NB + NB * TN + NB * NB + NB));
     WPCCC_CUDA(cudaFuncSetAttribute(k_lu<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max(smem, 120 * 1024)));
-    static thread_local int held[9] = {};   // clusters an empty chip holds, by size
+    // clusters an empty chip holds, by size, of the device that this thread last used
+    static thread_local int held[9] = {}, device = -1;
+    int now = 0;
+    WPCCC_CUDA(cudaGetDevice(&now));
+    if (now != device) {
+        held[1] = 0;
+        device = now;
+    }
     ClusterLaunch L(batch, lu_cluster<R>(N, batch, H != nullptr, held, st), LU_THREADS, smem, st);
     WPCCC_CUDA(cudaLaunchKernelEx(&L.cfg, k_lu<R>, N, S, F, H, ipiv, info));
     return WPCCC_OK;

@@ -84,21 +84,19 @@ static __device__ __forceinline__ void f64_levels(const float (&v)[F64_LEV][4], 
 }
 
 // One window's sum added to the running sum: T 2^(E - 42) to acc (one FP64 FMA), the low part 2^(E - 61) to low in FP32, in
-// units of 2^-100; below that range (windows 2^-165 and smaller) the low part goes with T, rounded to FP64.  Zero below
-// FP64's range, NaN for a row with a non-finite value.
-constexpr int F64_LOW = 100;
-static __device__ __forceinline__ void f64_accumulate(double& acc, float& low, long long T, uint32_t low19, int E) {
-    double X = __dsub_rn(__longlong_as_double(T + 0x4338000000000000ll), 6755399441055744.0);
-    const int es = E - 42 + 1023, ef = E - 61 + F64_LOW + 127;
+// units of 2^-unit, which keeps it for windows of 2^E from 2^(-65 - unit) to 2^(164 - unit).  Zero below FP64's range, NaN
+// for a row with a non-finite value.
+constexpr int F64_UNIT = 100;
+static __device__ __forceinline__ void f64_accumulate(double& acc, float& low, long long T, uint32_t low19, int E, int unit) {
+    const double X = __dsub_rn(__longlong_as_double(T + 0x4338000000000000ll), 6755399441055744.0);
+    const int es = E - 42 + 1023, ef = E - 61 + unit + 127;
     const int sh = E >= F64_BAD / 2 ? 0x7FF80000 : (max(0, min(es, 2046)) << 20);
-    if (ef <= 0 && low19 != 0) X = fma((double)low19, __hiloint2double((1023 - 19) << 20, 0), X);
     acc = fma(X, __hiloint2double(sh, 0), acc);
     const float r = __fsub_rn(__uint_as_float(0x4B000000u | low19), 8388608.f);
     low = fmaf(r, __uint_as_float((uint32_t)max(0, min(ef, 230)) << 23), low);
 }
-
-static __device__ __forceinline__ double f64_total(double acc, float low) {
-    return fma((double)low, __hiloint2double((1023 - F64_LOW) << 20, 0), acc);
+static __device__ __forceinline__ double f64_total(double acc, float low, int unit) {
+    return fma((double)low, __hiloint2double((1023 - unit) << 20, 0), acc);
 }
 
 // The MMAs of one chunk (one thread): the B tile's digits lie one after the other, so one MMA per A digit and K step forms

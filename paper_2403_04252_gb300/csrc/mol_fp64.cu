@@ -21,8 +21,9 @@
 // blocks of two-centre p + H err by 1e-17 to 2e-17 (against long double, |z| <= 12), the chain of G multiply-adds by 8e-17
 // to 1.3e-15.  A small element whose rows peak at different nuclei is far below that product, so the nodes' order, the
 // windows' length and exact power-of-two scales keep the two together (f64_order.cuh): element by element the error
-// stays within what the chain leaves, at any distance.  The shorter windows cost FP64 operations, two per result and window:
-// 21 p + H positions over |z| <= 20 take 1.36 ms a call, 1.20 with windows of 512 nodes throughout.
+// stays within what the chain leaves, at any distance.  The shorter windows cost a drain each, with two FP64 operations per
+// result: 33, 43, 65 and 119 us per p + H position with windows of 512, 128, 64 and 32 nodes (24 positions); 21 positions
+// over |z| <= 20 take 1.3 to 1.4 ms a call, 1.20 with windows of 512 nodes throughout.
 //
 // What bounds it.  The FP64 pipe of this part does two FMAs per clock per SM, and the CUDA-core contraction takes
 // five FP64 operations per (target state, half column, node): 581 us per p + H position (N = 380, 2304 nodes).  Here
@@ -90,32 +91,28 @@ static __device__ __forceinline__ void load4(const double* __restrict__ p, int g
     }
 }
 
-__global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
-    __shared__ __align__(16) double s_r[F64_WIN], s_rv[F64_WIN];
-    extern __shared__ int s_hw[];   // [nd][F64_WIN]: high word of max(|re|, |im|) of W / r_T
+// FULL: one window per span (wch = 16); else wch chunks of 32 nodes per window.
+template <bool FULL>
+static __device__ __forceinline__ void f64_slices(const F64SliceArgs& A, int wch, double* s_r, double* s_rv, int* s_hw) {
     const int e = blockIdx.y, w = blockIdx.x / F64_SPLIT, part = blockIdx.x % F64_SPLIT, g0 = w * F64_WIN;
     const int tid = threadIdx.x, warp = part * 8 + (tid >> 5), lane = tid & 31;   // warp among the span's
-    constexpr int Q = F64_WIN / 128;   // node quads per lane
-    const int wch = f64_window_chunks(A.Gp, __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z))), wlog = 31 - __clz(wch);
+    constexpr int Q = F64_WIN / 128, NW = FULL ? 1 : Q;   // node quads per lane; windows that they lie in
     // m[j] <- the largest m over the window of the lane's quad j
-    auto window_max = [&](int (&m)[Q]) {
-        if (wch * F64_K == F64_WIN) {
-            for (int j = 1; j < Q; ++j) m[0] = max(m[0], m[j]);
-            m[0] = __reduce_max_sync(0xffffffffu, m[0]);
-            for (int j = 1; j < Q; ++j) m[j] = m[0];
-        } else {
-            for (int j = 0; j < Q; ++j) {
-                if (wch == 4) m[j] = __reduce_max_sync(0xffffffffu, m[j]);
-                else
-                    for (int o = 4 * wch; o > 0; o >>= 1) m[j] = max(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
-            }
+    auto window_max = [&](int (&m)[NW]) {
+#pragma unroll
+        for (int j = 0; j < NW; ++j) {
+            if (FULL || wch == 4) m[j] = __reduce_max_sync(0xffffffffu, m[j]);
+            else
+                for (int o = 4 * wch; o > 0; o >>= 1) m[j] = max(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
         }
     };
-    // window of the lane's quad j, for the one lane and quad that write it; else -1
-    auto window_of = [&](int j) {
-        const int g = g0 + 4 * lane + 128 * j;
-        return g < A.Gp && (g & (wch * F64_K - 1)) == 0 ? g / F64_K >> wlog : -1;
-    };
+    // that window, for the one lane that writes it; else -1
+    int window[NW];
+#pragma unroll
+    for (int j = 0; j < NW; ++j) {
+        const int g = g0 + 4 * lane + 128 * j, per = FULL ? F64_WIN : wch * F64_K;
+        window[j] = g < A.Gp && (g & (per - 1)) == 0 ? g / per : -1;
+    }
     char* base = A.node + (size_t)e * A.node_bytes;
     const double* fT = reinterpret_cast<const double*>(base);
     const double* fP = fT + (size_t)A.nradT * A.G;
@@ -160,10 +157,9 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
         }
         const int dlo = max(0, q - A.qmaxT), dhi = min(A.nd - 1, q + A.qmaxT);
         for (int d = dlo; d <= dhi; ++d) {
-            int m[Q];
+            int m[NW] = {};
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
-                m[j] = 0;
                 const int4 hw = *reinterpret_cast<const int4*>(s_hw + d * F64_WIN + 4 * lane + 128 * j);
                 const int hv[4] = {hw.x, hw.y, hw.z, hw.w};
 #pragma unroll
@@ -174,15 +170,13 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
                     const uint32_t ab = (uint32_t)a + (uint32_t)b;
                     const int p = max(a, b) >= 0x7FF00000 ? 0x7FF00000
                                   : min(a, b) < (1 << 20) || ab < (1023u << 20) ? 0 : (int)min(ab - (1023u << 20), 0x7FEFFFFFu);
-                    m[j] = max(m[j], p);
+                    m[FULL ? 0 : j] = max(m[FULL ? 0 : j], p);
                 }
             }
             window_max(m);
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                const int x = window_of(j);
-                if (x >= 0) eb[((size_t)c * A.nd + d) * A.nwin + x] = f64_exponent(m[j], F64_MARGIN2);
-            }
+            for (int j = 0; j < NW; ++j)
+                if (window[j] >= 0) eb[((size_t)c * A.nd + d) * A.nwin + window[j]] = f64_exponent(m[j], F64_MARGIN2);
         }
     }
     // target rows
@@ -208,7 +202,7 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
         for (int v = 0; v < 2; ++v) {
             const double* sr = v == 0 ? s_r : s_rv;
             double x[4 * Q];
-            int m[Q];
+            int m[NW] = {};
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
                 const double2 ra = *reinterpret_cast<const double2*>(sr + 4 * lane + 128 * j),
@@ -217,21 +211,23 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
                 x[4 * j + 1] = t[4 * j + 1] * ra.y;
                 x[4 * j + 2] = t[4 * j + 2] * rb.x;
                 x[4 * j + 3] = t[4 * j + 3] * rb.y;
-                m[j] = 0;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) m[j] = max(m[j], abs_hi(x[4 * j + k]));
+                for (int k = 0; k < 4; ++k) m[FULL ? 0 : j] = max(m[FULL ? 0 : j], abs_hi(x[4 * j + k]));
             }
             window_max(m);
             const int r1 = rp + v * ts, r2 = rn + v * tsn;
+            int E[NW];
+#pragma unroll
+            for (int j = 0; j < NW; ++j) {
+                E[j] = f64_exponent(m[j], F64_MARGIN);
+                if (window[j] < 0) continue;
+                ea[(size_t)window[j] * A.tc_rows + r1] = E[j];
+                if (rn >= 0) ea[(size_t)window[j] * A.tc_rows + r2] = E[j];
+            }
 #pragma unroll
             for (int j = 0; j < Q; ++j) {
-                const int g = g0 + 4 * lane + 128 * j;
+                const int g = g0 + 4 * lane + 128 * j, E1 = E[FULL ? 0 : j] + 1023;
                 if (g >= A.Gp) continue;
-                const int E = f64_exponent(m[j], F64_MARGIN), E1 = E + 1023, wx = window_of(j);
-                if (wx >= 0) {
-                    ea[(size_t)wx * A.tc_rows + r1] = E;
-                    if (rn >= 0) ea[(size_t)wx * A.tc_rows + r2] = E;
-                }
                 uint32_t d0[F64_SL], d1[F64_SL];
                 f64_digits(f64_fix(x[4 * j], E1), f64_fix(x[4 * j + 1], E1), d0);
                 f64_digits(f64_fix(x[4 * j + 2], E1), f64_fix(x[4 * j + 3], E1), d1);
@@ -250,6 +246,15 @@ __global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(256) k_f64_slices(F64SliceArgs A) {
+    __shared__ __align__(16) double s_r[F64_WIN], s_rv[F64_WIN];
+    extern __shared__ int s_hw[];   // [nd][F64_WIN]: high word of max(|re|, |im|) of W / r_T
+    const EvalDesc& p = A.ev[blockIdx.y];
+    const int wch = f64_window_chunks(A.Gp, __dmul_rn(A.kappa, dist_R(p.b, p.z)));
+    if (wch * F64_K == F64_WIN) f64_slices<true>(A, wch, s_r, s_rv, s_hw);
+    else f64_slices<false>(A, wch, s_r, s_rv, s_hw);
 }
 
 // ---------------------------------------------------------------------------
@@ -313,7 +318,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
     volatile int* abort_flag = &s_abort;
     const char* nb = A.node + (size_t)e * A.node_bytes;
     const int nk = A.nk;
-    const int wch = f64_window_chunks(A.Gp, __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z))), wlog = 31 - __clz(wch);
+    const double kR = __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z));
+    const int wch = f64_window_chunks(A.Gp, kR), wlog = 31 - __clz(wch), unit = f64_unit(kR);
 
     if (warp == F64_TMA_WARP) {
         // ---- TMA issue (one thread): the table tiles chunk by chunk into their ring
@@ -430,9 +436,8 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             if (lane == 0) mbar_arrive(acce);
             if (live) {
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    f64_accumulate(acc[k], low[k], T[k], low19[k], Ea + __shfl_sync(0xffffffffu, Eb, k >> 1));
-                }
+                for (int k = 0; k < 16; ++k)
+                    f64_accumulate(acc[k], low[k], T[k], low19[k], Ea + __shfl_sync(0xffffffffu, Eb, k >> 1), unit);
             }
         }
         // results: row lrow of D is A_T row lrow of the tile (overlap K) or, from ns on, its A_T V_T row (Q)
@@ -445,12 +450,12 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             for (int k = 0; k < 16; k += 2) {
                 const int c = c0 + (col0 + k) / 2;
                 if (c < A.n_half)
-                    out[c] = make_double2(f64_total(acc[k], low[k]), f64_total(acc[k + 1], low[k + 1]));
+                    out[c] = make_double2(f64_total(acc[k], low[k], unit), f64_total(acc[k + 1], low[k + 1], unit));
             }
         }
     } else {
-        // ---- producers: thread = (half column, node pair); one FP64 FMA per element rounds the exact product
-        // W A_P to the window's grid.  The next chunk's A_P and W are loaded before this chunk is written.
+        // ---- producers: thread = (half column, node pair); one FP64 multiplication per element, then an integer shift
+        // rounds W A_P to the window's grid.  The next chunk's A_P and W are loaded before this chunk is written.
         const int p = tid & 15, cl = tid >> 4, c = c0 + cl;
         const bool valid = c < A.n_half;
         const int d = valid ? abs(A.half_q[c] - qp) : 0;

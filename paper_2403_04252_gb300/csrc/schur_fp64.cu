@@ -7,7 +7,7 @@
 // (k_schur_digits; the representation of mol_fp64.cu, windows of 512 k) and multiplied by k_schur_f64tc, both operands
 // by TMA.  On the CUDA cores the update takes 4 N_P^2 N_T FP64 flops of the factorisation's 4 N_P^2 N_T + (4/3) N_P^3 at two
 // FMAs per clock per SM: 22 of 30 us per p + H position (N_T = N_P = 190).  Factorisation of 672 such positions, update
-// on the CUDA cores -> here: 34.6 -> 15.5 ms; N = 572, 288 positions: 53.7 -> 21.2 ms; N_T = 57, N_P = 52: 0.37 -> 0.27 ms.
+// on the CUDA cores -> here: 34.6 -> 15.5 ms; N = 572, 288 positions: 53.7 -> 21.2 ms; N_T = 59, N_P = 50: 0.37 -> 0.27 ms.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(SD_THREADS, 1) k_schur_f64tc(const __grid_cons
                     long long T;
                     uint32_t low19;
                     f64_levels(v, u, T, low19);
-                    f64_accumulate(acc[4 * g + u], low[4 * g + u], T, low19, Em + __shfl_sync(0xffffffffu, En, 4 * g + u));
+                    f64_accumulate(acc[4 * g + u], low[4 * g + u], T, low19, Em + __shfl_sync(0xffffffffu, En, 4 * g + u), F64_UNIT);
                 }
             }
             tc_fence_before();
@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(SD_THREADS, 1) k_schur_f64tc(const __grid_cons
             for (int k = 0; k < 16; ++k) {
                 const int n = n0 + col0 + k;
                 if (n >= A.NP || n > m) continue;
-                const double c = f64_total(acc[k], low[k]);
+                const double c = f64_total(acc[k], low[k], F64_UNIT);
                 double* p = reinterpret_cast<double*>(S + (size_t)(A.N_T + m) + (size_t)(A.N_T + n) * A.N);
                 if (half) p[1] = -c;
                 else p[0] = (m == n ? 1.0 : 0.0) - c;

@@ -84,8 +84,8 @@ static __device__ __forceinline__ void f64_levels(const float (&v)[F64_LEV][4], 
 }
 
 // One window's sum added to the running sum: T 2^(E - 42) to acc (one FP64 FMA), the low part 2^(E - 61) to low in FP32, in
-// units of 2^-unit, which keeps it for windows of 2^E from 2^(-65 - unit) to 2^(164 - unit).  Zero below FP64's range, NaN
-// for a row with a non-finite value.
+// units of 2^-unit, which keeps it for windows of 2^E from 2^(-65 - unit) to 2^(164 - unit) (-1000 < unit < 1000).  Zero
+// below FP64's range, NaN for a row with a non-finite value.
 constexpr int F64_UNIT = 100;
 static __device__ __forceinline__ void f64_accumulate(double& acc, float& low, long long T, uint32_t low19, int E, int unit) {
     const double X = __dsub_rn(__longlong_as_double(T + 0x4338000000000000ll), 6755399441055744.0);

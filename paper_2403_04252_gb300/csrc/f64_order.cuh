@@ -37,10 +37,6 @@ static __device__ __forceinline__ int f64_window_chunks(int G, double kR) {
     return 512.0 * q <= lim ? 16 : 128.0 * q <= lim ? 4 : 64.0 * q <= lim ? 2 : 1;
 }
 
-// Unit 2^-unit of the sums' low parts: elements fall like exp(-kappa R), and FP32 holds windows of 2^-165 to 2^64 with the
-// one, 2^-215 to 2^14 with the other (below that an element keeps 2^-42 of its window's scale).
-static __device__ __forceinline__ int f64_unit(double kR) { return kR > 64.0 ? 150 : 100; }
-
 // Exponent s of the scale at tau: (kappa R / 4) tau log2(e), as far as FP64's range allows.
 static __device__ __forceinline__ int f64_scale(double kR, double tau) {
     return __double2int_rn(0.25 * 1.4426950408889634 * fmin(kR, 400.0) * tau);

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
     const char* nb = A.node + (size_t)e * A.node_bytes;
     const int nk = A.nk;
     const double kR = __dmul_rn(A.kappa, dist_R(A.ev[e].b, A.ev[e].z));
-    const int wch = f64_window_chunks(A.Gp, kR), wlog = 31 - __clz(wch), unit = f64_unit(kR);
+    const int wch = f64_window_chunks(A.Gp, kR), wlog = 31 - __clz(wch);
 
     if (warp == F64_TMA_WARP) {
         // ---- TMA issue (one thread): the table tiles chunk by chunk into their ring
@@ -407,6 +407,14 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
         }
         bool ok = true;
         const int nwin = (nk + wch - 1) >> wlog;
+        // the low parts' unit follows the largest scales of the element's two rows
+        int ua = F64_EMIN, ub = F64_EMIN;
+        for (int j = 0; j < nwin; ++j) {
+            if (lrow < 2 * ns) ua = max(ua, ea[(size_t)j * A.tc_rows + row0 + lrow]);
+            if (ebv) ub = max(ub, eb[ebo + j]);
+        }
+        ua = F64_UNIT - max(-500, min(ua, 500));
+        ub = -max(-500, min(ub, 500));
         for (int j = 0; j < nwin && ok; ++j) {
             const int Ea = lrow < 2 * ns ? ea[(size_t)j * A.tc_rows + row0 + lrow] : F64_EMIN;
             const int Eb = ebv ? eb[ebo + j] : F64_EMIN;
@@ -437,19 +445,20 @@ __global__ void __launch_bounds__(F64_THREADS, 1) k_mol_f64tc(const __grid_const
             if (live) {
 #pragma unroll
                 for (int k = 0; k < 16; ++k)
-                    f64_accumulate(acc[k], low[k], T[k], low19[k], Ea + __shfl_sync(0xffffffffu, Eb, k >> 1), unit);
+                    f64_accumulate(acc[k], low[k], T[k], low19[k], Ea + __shfl_sync(0xffffffffu, Eb, k >> 1),
+                                   ua + __shfl_sync(0xffffffffu, ub, k >> 1));
             }
         }
         // results: row lrow of D is A_T row lrow of the tile (overlap K) or, from ns on, its A_T V_T row (Q)
-        if (ok && lrow < 2 * ns) {
+        if (ok) {
             const int x = lrow < ns ? 0 : 1;
-            const int i = A.qg_rows[tile * A.qg_max + (lrow < ns ? lrow : lrow - ns)];
+            const int i = lrow < 2 * ns ? A.qg_rows[tile * A.qg_max + (lrow < ns ? lrow : lrow - ns)] : 0;
             const size_t plane = (size_t)A.N_T * A.n_half;
             double2* out = reinterpret_cast<double2*>(A.mol) + (size_t)e * 2 * plane + (size_t)x * plane + (size_t)i * A.n_half;
 #pragma unroll
             for (int k = 0; k < 16; k += 2) {
-                const int c = c0 + (col0 + k) / 2;
-                if (c < A.n_half)
+                const int c = c0 + (col0 + k) / 2, unit = ua + __shfl_sync(0xffffffffu, ub, k >> 1);
+                if (lrow < 2 * ns && c < A.n_half)
                     out[c] = make_double2(f64_total(acc[k], low[k], unit), f64_total(acc[k + 1], low[k + 1], unit));
             }
         }

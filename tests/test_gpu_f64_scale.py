@@ -26,3 +26,23 @@ def test_elements_scale_with_the_radial_functions(power):
 
     one, scaled = blocks(1.0), blocks(2.0 ** power)
     assert torch.equal(scaled, one * 2.0 ** power)
+
+
+@pytest.mark.parametrize("power", [-50, 20, 60])
+def test_small_elements_scale_with_both_centres(power):
+    import paper_2403_04252_gb300 as w
+    zs = np.array([-6.0, 30.0, -80.0])
+
+    def blocks(factor):
+        basis = wi.make_basis(1.0, 1.0, 2, 1, 3, 2.0, True, Nr=600, Geta=24, Gtau=24)
+        basis.T.f *= factor
+        basis.P.f *= factor
+        g = w.Basis(basis)
+        S, H = g.matrix_elements(0.8, 1.2, zs)
+        torch.cuda.synchronize()
+        g.close()
+        NT = basis.T.N
+        return torch.stack([w.natural(x)[:, :NT, NT:] for x in (S, H)])
+
+    one, scaled = blocks(1.0), blocks(2.0 ** power)
+    assert torch.equal(scaled, one * 4.0 ** power)

@@ -171,7 +171,10 @@ WPCCC_API wpccc_status wpccc_basis_info(wpccc_basis basis, int* N_T, int* N_P);
  * In one-centre mode S[k] = I and H[k] = D_T.
  *   z      host   [nz] positions
  *   S, H   device [nz][N][N] complex128, column-major; fully overwritten
- * Errors: EINVAL (nz < 1, b <= 0, v <= 0, null pointers), ENOMEM, ECUDA.
+ * With two centres the Eq. 9 contraction runs in exact fixed-point digits on the tensor cores (see wpccc_propagate,
+ * mode 0).  Where the device's memory does not hold one position's digits the FP64 pipe takes it, whose last bits differ.
+ * Errors: EINVAL (nz < 1, b <= 0, v <= 0, null pointers), ENOMEM, ETIMEOUT (a bounded wait of a kernel gave up),
+ * ECUDA.
  */
 WPCCC_API wpccc_status wpccc_matrix_elements(wpccc_basis basis, double b, double v, int nz, const double* z,
                                    void* S, void* H, void* stream);
@@ -195,8 +198,10 @@ WPCCC_API wpccc_status wpccc_matrix_elements_precision(wpccc_basis basis, double
  * memory inside a call, e.g. a host framework that reserved the device memory up
  * front (a further cudaMalloc would fail or fragment its pool), or a
  * latency-critical loop that cannot absorb the device-wide synchronisation of
- * cudaMalloc/cudaFree.  Same arguments and results as wpccc_matrix_elements
- * (S and H are written by the same kernels; the caller still owns them).
+ * cudaMalloc/cudaFree.  Same arguments as wpccc_matrix_elements and, to rounding, the same
+ * results: the Eq. 9 contraction runs on the FP64 pipe, whose scratch fits the array, in
+ * about ten times the time per position (581 against some 40 us for p + H).  The caller
+ * owns S and H.
  * Scratch memory: a fixed array of WPCCC_NOALLOC_SCRATCH_BYTES (64 MiB) inside
  * the library, which every GPU that loads the library holds until the process
  * exits.  Nothing in it needs clearing (every byte a call reads it first writes),
@@ -341,7 +346,7 @@ WPCCC_API wpccc_status wpccc_cross_sections(int n_b, const double* b, int n_obs,
  * invariant of the two-centre propagation (in one-centre mode S = I and both norms are c^+ c).
  *   b, v, z  host [n_paths];  c  device [n_paths][N] complex128;  out  device [n_paths][2] double
  * Blocks until done; allocates S and H for the positions (freed before it returns) and uses the basis
- * workspace.  Errors: EINVAL, ENOMEM, ECUDA.
+ * workspace.  Errors: EINVAL, ENOMEM, ETIMEOUT, ECUDA.
  */
 WPCCC_API wpccc_status wpccc_overlap_norms(wpccc_basis basis, int n_paths, const double* b, const double* v,
                                            const double* z, const void* c, double* out, void* stream);
@@ -413,9 +418,10 @@ WPCCC_API wpccc_status wpccc_basis_set_refine_iters(wpccc_basis basis, int iters
 WPCCC_API wpccc_status wpccc_basis_set_refine_tolerance(wpccc_basis basis, double tol);
 
 /*
- * Iteration limit of every mbarrier wait in device code: the tensor-core kernels' waits (precision modes 3-5;
- * the contraction's TMA thread counts polls in which neither of its buffers came free) and the RK4 sweep's
- * waits for the bulk copies that stage H in shared memory (precision modes 1-3, N <= 512).  A tensor-core
+ * Iteration limit of every mbarrier wait in device code: the tensor-core kernels' waits (the Eq. 9 contraction in
+ * every precision mode but 1, the Schur update; the four- and seven-slice contraction's TMA thread counts polls in
+ * which neither of its buffers came free) and the waits of the refined LU form's RK4 sweep for the bulk copies that
+ * stage H in shared memory (precision modes 1-3 without the Schur solve, N <= 512).  A tensor-core
  * CTA whose wait has polled `polls` times gives up, records the failure, lets the copies and tensor-core
  * operations it has in flight complete, frees its tensor memory and returns; an RK4 block records the
  * failure and goes on in step with its other threads, its copies landing before it returns.  The call then
@@ -504,7 +510,7 @@ WPCCC_API wpccc_status wpccc_basis_set_tangents(wpccc_basis basis, int n_par, co
  *   grad   device [n_paths][n_obs][n_par] double
  * Needs wpccc_basis_set_tangents first.  Two-centre bases only.  Blocks until done; allocates its
  * own checkpoint and segment buffers (freed before it returns) and uses the basis workspace.
- * Errors: EINVAL, EUNSUPPORTED (one-centre basis), ENOMEM, ESINGULAR, ENONFINITE, ECUDA.
+ * Errors: EINVAL, EUNSUPPORTED (one-centre basis), ENOMEM, ESINGULAR, ENONFINITE, ETIMEOUT, ECUDA.
  */
 WPCCC_API wpccc_status wpccc_propagate_adjoint(wpccc_basis basis, const wpccc_paths* paths, int n_obs,
                                                const double* g, int checkpoint_every, void* c, double* P,

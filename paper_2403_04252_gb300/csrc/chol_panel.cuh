@@ -17,7 +17,8 @@ static __device__ __forceinline__ double2 chol_step(double2 v, double2 l, double
 }
 
 // (sqrt(d), 1 / sqrt(d)); in FP64 by two Newton-Raphson steps r <- r + r (1 - d r^2) / 2 from the FP32 reciprocal square
-// root: an FP64 square root and division are long serial chains on this part's FP64 pipe
+// root: an FP64 square root and division are long serial chains on this part's FP64 pipe.  The square root is d r, within
+// two units in the last place, not the correctly rounded one.
 static __device__ __forceinline__ float2 sqrt_and_inverse(float d) {
     const float s = sqrt(d);
     return make_float2(s, 1.f / s);

@@ -17,7 +17,8 @@ static __device__ __forceinline__ int cluster_size() {
     return r;
 }
 // Barrier over all threads of the cluster; global- and shared-memory writes made before it are visible after it
-// (release / acquire at cluster scope).  Data that another block wrote is read with __ldcg.
+// (release / acquire at cluster scope), by plain loads too.  __ldcg marks reads of what other blocks wrote where the line
+// would not be read again from L1.
 static __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
 }

@@ -15,32 +15,8 @@ static __device__ inline double dist_R(double b, double z) {
     return __dsqrt_rn(__dadd_rn(__dmul_rn(b, b), __dmul_rn(z, z)));
 }
 
-// Largest j with r[j] <= x (-1 if x < r[0]); 5-point stencil start and Lagrange weights.
-// Returns false when x lies beyond the last grid point (the function is zero there).
-static __device__ inline bool stencil5(const double* __restrict__ r, int Nr, double x, int& s, double L[5]) {
-    if (x > r[Nr - 1]) return false;
-    int lo = -1, hi = Nr;
-    while (hi - lo > 1) {
-        int mid = (lo + hi) >> 1;
-        if (r[mid] <= x) lo = mid;
-        else hi = mid;
-    }
-    s = min(max(lo - 2, 0), Nr - 5);
-    double rn[5];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) rn[k] = r[s + k];
-#pragma unroll
-    for (int a = 0; a < 5; ++a) {
-        double p = 1.0;
-#pragma unroll
-        for (int c = 0; c < 5; ++c)
-            if (c != a) p *= (x - rn[c]) / (rn[a] - rn[c]);
-        L[a] = p;
-    }
-    return true;
-}
-
-// The same stencil by one warp: the start in every lane, weight a in lane a < 5.
+// Start of the 5-point stencil at x (two nodes left of the largest j with r[j] <= x) by one warp, in every lane; Lagrange
+// weight a in lane a < 5.  x <= r[Nr - 1].
 static __device__ inline void stencil5_warp(const double* __restrict__ r, int Nr, double x, int lane, int& s, double& L) {
     int lo = -1, hi = Nr;   // r[lo] <= x < r[hi]
     while (hi - lo > 1) {

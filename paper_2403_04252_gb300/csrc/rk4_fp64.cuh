@@ -13,8 +13,9 @@
 // panel by panel (32 rows, the panels to the blocks in turn): the owner solves the diagonal block and sends the 32
 // unknowns to all blocks, every block updates its own rows; the factor's tile is loaded before the barrier.
 // Measured, one block per path with a row per thread -> here, sweeps alone: one centre, N = 59, 8 paths of 800 steps
-// 42.6 -> 10.2 ms (13.3 -> 3.2 us per stage); two centres, LU, N = 109, 5 paths of 13 steps 10.3 -> 2.4 ms; Schur,
-// N = 380, 32 paths of 10 steps 22 -> 9.0 ms.
+// 42.6 -> 10.2 ms (13.3 -> 3.2 us per stage); two centres, LU, N = 109, 5 paths of 11 to 23 steps 10.3 -> 4.4 ms (inverted
+// diagonal blocks included, see rc_lu_solve); Schur, N = 380, 32 paths of 10 steps 22 -> 9.0 ms.  Slopes are formed with
+// 1 / v, one rounding more than a division by v.
 #pragma once
 
 #include "cluster.cuh"
@@ -271,7 +272,7 @@ static __device__ __noinline__ void rc_schur_solve(const RcCluster& cl, const do
 // t <- S^{-1} t (replicated) from P S = L U with inverted 32 x 32 diagonal blocks (launch_lu_invert_diag): perm[r] = row of t
 // that comes r-th.  z: scratch of N entries; part: RC_BLK.  The inverse turns a panel's chain of 32 dependent FP64 steps
 // into one product of 16 threads per row, whose entries are loaded before the barrier that makes the panel's right-hand
-// side known (N = 109, 5 paths of up to 23 steps: sweep 7.8 -> 4.4 ms, for 0.3 ms of inversion; the adjoint of p + Li,
+// side known (N = 109, 5 paths of 11 to 23 steps: sweep 7.8 -> 4.4 ms, for 0.3 ms of inversion; the adjoint of p + Li,
 // N = 379: 35 -> 28 ms).
 static __device__ __noinline__ void rc_lu_solve(const RcCluster& cl, const double2* __restrict__ LU, const uint16_t* perm,
                                                    int N, double2* t, double2* z, double2* part) {

@@ -21,7 +21,7 @@
 namespace wpccc {
 
 constexpr int SC_NB = 32;          // Cholesky panel width
-static_assert(SC_NB == 32, "the diagonal block is factorised by one warp, a row per lane");
+static_assert(SC_NB == 32, "the diagonal block is factorised with a row per lane");
 constexpr int SC_THREADS = 256;
 constexpr int SC_T = 64;           // update tile, complex elements; a thread holds 4 x 4 of them
 constexpr int SC_LD = SC_T + 1;    // its stride in shared memory (no bank conflicts on either index)
@@ -113,7 +113,7 @@ __device__ void cta_update_lower(typename SchurC<R>::type* __restrict__ C, int l
 // lower triangle (formed on the tensor cores); only the Cholesky factor is computed.
 //
 // Blocked right-looking Cholesky.  Per panel of 32 columns every block of the cluster factorises the 32 x 32
-// diagonal block for itself (one warp, a row per lane, in shared memory), the rows below go to the blocks' threads, a
+// diagonal block for itself (chol_panel.cuh: all warps, a row per lane, in shared memory), the rows below go to the blocks' threads, a
 // row each (L21 = A21 L11^{-+}, column by column in registers or shared memory), and the trailing tiles to the
 // blocks in turn: two cluster barriers per panel.  Every element goes through the same operations in the same order
 // as an unblocked column-by-column elimination within the panel, for any cluster size.  The FP64 factor is left for the

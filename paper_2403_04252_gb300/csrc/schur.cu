@@ -259,15 +259,16 @@ __global__ void __launch_bounds__(SC_THREADS) k_schur_factor(int N, int N_T, con
     if (tid == 0 && rank == 0) info_all[sys] = s_info;
 }
 
-// Blocks per system: doubled while there is no more than one block per SM, as long as each has a few 64 x 64 tiles.
+// Blocks per system: doubled while there is about one block per SM or less, as long as each has a few 64 x 64 tiles.
 // Factorisation in ms with 1, 2, 4 and 8 blocks (* the rule's), FP64 N_P = 190 with the update on the tensor cores:
 //   20 systems 2.18 1.56* 1.27 1.88, 50 systems 2.31 1.68* 2.13 3.00, 120 systems 2.57 2.84* 4.12 5.78, 160 4.20* 4.26 5.10 7.78;
 // FP32 N_P = 190: 50 systems 0.67 0.43* 0.36 0.53, 120 systems 0.69 0.49* 0.70 1.06, 160 0.78* 0.89 1.00 1.33;
-// FP32 N_P = 811: 20 systems 13.0 7.8 5.2 4.1*, 50 systems 16.4 10.8 8.3* 9.0, 80 systems 19.7 14.2* 14.4 13.7.
+// FP32 N_P = 811: 20 systems 13.0 7.8 5.2 4.1*, 50 systems 16.4 10.8 8.3* 9.0, 80 systems 19.7 14.2* 14.4 13.7;
+// FP64 N_P = 811: 100 systems 120 113* 92 (four), 160 systems 218 168* 149, 180 systems 220* 171 153, 250 systems 228* 227 214.
 static int schur_cluster(int NP, int batch, int sms) {
     const int tiles = ((NP + SC_T - 1) / SC_T) * ((NP + SC_T - 1) / SC_T + 1) / 2;
     int cl = 1;
-    while (cl < 8 && cl * batch <= sms && tiles >= 4 * cl) cl *= 2;
+    while (cl < 8 && cl * batch <= sms + sms / 16 && tiles >= 4 * cl) cl *= 2;
     return cl;
 }
 

@@ -1077,15 +1077,18 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
     };
     wpccc_status s = WPCCC_OK;
     bool digits = false, smallest = true;   // some set's plan takes the digits; all of those run one position at a time
+    size_t largest = 0;                     // bytes of the largest set's plan
     auto plan_sets = [&](size_t cap, bool cuda_cores) -> wpccc_status {
     digits = false;
     smallest = true;
+    largest = 0;
     for (int k = 0; k < n_sets; ++k) {
         wpccc_basis_s* B = bases[k];
         const size_t limit = std::min(B->ws_limit, cap);
         X->c[k] = static_cast<double2*>(c[k]);
         PropPlan P;
         if ((s = plan_build(B, &paths[k], precision_mode, 0, limit, P, cuda_cores)) != WPCCC_OK) return s;
+        largest = std::max(largest, P.bytes);
         if (P.elem_precision == ELEM_F64_TC && P.max_steps > 0) {
             digits = true;
             if (P.C > 1 || P.elem_batch > 1) smallest = false;
@@ -1133,8 +1136,8 @@ extern "C" wpccc_status wpccc_batch_create(int n_sets, const wpccc_basis* bases,
         cudaGetLastError();
         if (smallest) s = plan_sets((size_t)1 << 46, true);
         else {
-            for (int k = 0; k < n_sets; ++k) ws_cap = std::min(ws_cap, bases[k]->ws_limit);
-            s = plan_sets(ws_cap /= 2, false);
+            ws_cap = std::min(ws_cap, largest) / 2;
+            s = plan_sets(ws_cap, false);
         }
     }
     if (s != WPCCC_OK) return bail(s);

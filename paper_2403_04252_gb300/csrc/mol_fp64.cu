@@ -22,14 +22,14 @@
 // to 1.3e-15.  A small element whose rows peak at different nuclei is far below that product, so the nodes' order, the
 // windows' length and exact power-of-two scales keep the two together (f64_order.cuh): element by element the error
 // stays within what the chain leaves, at any distance.  The shorter windows cost a drain each, with two FP64 operations per
-// result: 33, 43, 65 and 119 us per p + H position with windows of 512, 128, 64 and 32 nodes (24 positions); 21 positions
+// result: 33, 43, 67 and 125 us per p + H position with windows of 512, 128, 64 and 32 nodes (24 positions); 21 positions
 // over |z| <= 20 take 1.3 to 1.4 ms a call, 1.20 with windows of 512 nodes throughout.
 //
 // What bounds it.  The FP64 pipe of this part does two FMAs per clock per SM, and the CUDA-core contraction takes
 // five FP64 operations per (target state, half column, node): 581 us per p + H position (N = 380, 2304 nodes).  Here
 // the FP64 pipe forms one product per generated element and two operations per result and window; the MMAs set
-// the pace (tensor pipe 61 % busy; a 128-row tile holds 22 to 100 rows of p + H).  Measured, 24 p + H positions:
-// 32 us per position, of which 18 us are the tensor cores' own time, plus 6 us for the operands (k_f64_slices).
+// the pace (tensor pipe 59 % busy; a 128-row tile holds 22 to 100 rows of p + H).  Measured, 24 p + H positions near the
+// target: 33 us per position, of which 18 us are the tensor cores' own time, plus 8 us for the operands (k_f64_slices).
 // The MMA queue is short, so the issuing thread's scalar work between two chunks shows in full: carrying the ring
 // positions along and testing the next chunk's barriers early took 2360 -> 1750 cycles per chunk (1281 of MMAs).
 

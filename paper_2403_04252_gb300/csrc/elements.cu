@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(128) k_node_tables(NodeArgs A, const EvalDesc*
     const double b = ev[e].b, v = ev[e].v, z = ev[e].z;
     const double R = dist_R(b, z);
     int k = g / A.Gtau, t = g - k * A.Gtau;
-    if (sizeof(T) == 8 && A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.Gtau, __dmul_rn(A.kappa, R)), k, t);
+    if (sizeof(T) == 8 && A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.G / A.Gtau, A.Gtau, __dmul_rn(A.kappa, R)), k, t);
     const double gR = __dmul_rn(A.gamma, R);
     const double eta = __dadd_rn(1.0, __ddiv_rn(A.s[k], gR));
     const double tau = A.tau[t];
@@ -1241,7 +1241,7 @@ __global__ void __launch_bounds__(256) k_direct_sr(SrArgs A, const EvalDesc* __r
     double* dt = I + (size_t)NA * A.nradP * LQ;
     for (int g = threadIdx.x; g < A.G; g += blockDim.x) {
         int k = g / A.Gtau, t = g - k * A.Gtau;
-        if (A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.Gtau, __dmul_rn(A.kappa, R)), k, t);
+        if (A.f64) f64_node(g, A.G / A.Gtau, A.Gtau, f64_block_width(A.G / A.Gtau, A.Gtau, __dmul_rn(A.kappa, R)), k, t);
         const double eta = __dadd_rn(1.0, __ddiv_rn(A.s[k], gR));
         const double tau = A.tau[t];
         const double rT = __dmul_rn(halfR, __dadd_rn(eta, tau));

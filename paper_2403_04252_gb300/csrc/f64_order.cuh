@@ -13,14 +13,17 @@
 //   z =  8: 12, 0.04 -> 1.5, 0.04 -> 30, 0.7      z = 30: 4e9, 0.1 -> 1.2, 0.07 -> 15, 0.4
 //   z = 16: 2e3, 0.06 -> 2.2, 0.05 -> 21, 0.4     z = 40: 3e13, 0.2 -> 2.3, 0.2 -> 26, 0.3
 //   z = 24: 3e6, 0.09 -> 15, 0.09 -> 21, 0.3      z = 80: 6e14, 0.3 -> 1.1, 0.1 -> 20, 0.3
-// and as well below the chain's for C6+ + H, He+ + He+ and rules of 50 x 30 to 128 x 48 nodes.
+// and as well below the chain's for C6+ + H, He+ + He+ and rules of 16 x 16 to 128 x 48 nodes.  It stays below 40 up to
+// kappa R = 150, and near 100 at 180; a rule whose windows cannot follow (31 x 7 nodes) reaches 170 at kappa R = 40.
 #pragma once
 
 namespace wpccc {
 
-// tau nodes per block: a sixth of them, fewer from kappa R = 48 on
-static __device__ __forceinline__ int f64_block_width(int Gtau, double kR) {
-    return max(1, min((Gtau + 3) / 6, (int)fmin(__ddiv_rn(8.0 * Gtau, kR), 1e6)));
+// tau nodes per block: a sixth of them, fewer from kappa R = 48 on; one more where a block of few eta nodes then ends on a
+// window's boundary (24 x 16 nodes, kappa R = 40: 1400 units with three, 9 with four).
+static __device__ __forceinline__ int f64_block_width(int Geta, int Gtau, double kR) {
+    const int w = max(1, min((Gtau + 3) / 6, (int)fmin(__ddiv_rn(8.0 * Gtau, kR), 1e6)));
+    return Geta <= 32 && w * Geta % 32 != 0 && (w + 1) * Geta % 32 == 0 ? w + 1 : w;
 }
 
 // Node g of the order: eta index k, tau index t.

@@ -21,7 +21,7 @@
 // blocks of two-centre p + H err by 1e-17 to 2e-17 (against long double, |z| <= 12), the chain of G multiply-adds by 8e-17
 // to 1.3e-15.  A small element whose rows peak at different nuclei is far below that product, so the nodes' order, the
 // windows' length and exact power-of-two scales keep the two together (f64_order.cuh): element by element the error
-// stays within what the chain leaves, at any distance.  The shorter windows cost a drain each, with two FP64 operations per
+// stays within what the chain leaves (its comment has the figures).  The shorter windows cost a drain each, with two FP64 operations per
 // result: 33, 43, 67 and 125 us per p + H position with windows of 512, 128, 64 and 32 nodes (24 positions); 21 positions
 // over |z| <= 20 take 1.3 to 1.4 ms a call, 1.20 with windows of 512 nodes throughout.
 //

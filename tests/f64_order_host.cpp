@@ -19,7 +19,7 @@ int main(int argc, char** argv) {
     const int Ge = std::atoi(argv[1]), Gt = std::atoi(argv[2]);
     const double kR = std::atof(argv[3]);
     std::printf("%d\n", 32 * wpccc::f64_window_chunks((Ge * Gt + 31) / 32 * 32, kR));
-    const int width = wpccc::f64_block_width(Gt, kR);
+    const int width = wpccc::f64_block_width(Ge, Gt, kR);
     for (int g = 0; g < Ge * Gt; ++g) {
         int k, t;
         wpccc::f64_node(g, Ge, Gt, width, k, t);

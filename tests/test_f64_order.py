@@ -54,7 +54,8 @@ def _fixed(x, win):
 
 
 @pytest.mark.parametrize("ZT,ZP,Geta,Gtau,z", [(1.0, 1.0, 48, 48, z) for z in (-2.0, 14.0, 16.0, 28.0, -36.0, 50.0, 90.0)] +
-                         [(2.0, 2.0, 48, 48, 14.0), (1.0, 6.0, 128, 48, 20.0), (1.0, 1.0, 50, 30, 24.0)])
+                         [(2.0, 2.0, 48, 48, 14.0), (1.0, 6.0, 128, 48, 20.0), (1.0, 1.0, 50, 30, 24.0), (1.0, 1.0, 24, 16, 40.0),
+                          (1.0, 1.0, 16, 16, -40.0), (1.0, 1.0, 48, 48, 150.0)])
 def test_small_elements_keep_the_accuracy_of_a_chain(order, ZT, ZP, Geta, Gtau, z):
     basis = wi.make_basis(ZT, ZP, (3, 3), (1, 1), (4, 4), 2.5, True, Geta=Geta, Gtau=Gtau)
     b, v = 1.0, 1.5

@@ -13,8 +13,9 @@
 //   z =  8: 12, 0.04 -> 1.5, 0.04 -> 30, 0.7      z = 30: 4e9, 0.1 -> 1.2, 0.07 -> 15, 0.4
 //   z = 16: 2e3, 0.06 -> 2.2, 0.05 -> 21, 0.4     z = 40: 3e13, 0.2 -> 2.3, 0.2 -> 26, 0.3
 //   z = 24: 3e6, 0.09 -> 15, 0.09 -> 21, 0.3      z = 80: 6e14, 0.3 -> 1.1, 0.1 -> 20, 0.3
-// and as well below the chain's for C6+ + H, He+ + He+ and rules of 16 x 16 to 128 x 48 nodes.  It stays below 40 up to
-// kappa R = 150, and near 100 at 180; a rule whose windows cannot follow (31 x 7 nodes) reaches 170 at kappa R = 40.
+// and as well at or below the chain's for C6+ + H, He+ + He+ and rules of 24 x 16 to 128 x 48 nodes at these kappa R.  Where it
+// ends: p + H stays below 40 up to kappa R = 150 and reaches 90 at 180, charges of 6 on both centres reach 100 from 144 on,
+// and rules too coarse for the distance 200 (31 x 7 nodes at kappa R = 40, 16 x 16 at 50).
 #pragma once
 
 namespace wpccc {
